@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) k_adj_order(KParams<T> P, const T* __rest
     if (x > P.nx || y > P.ny) return;
     const long long o = P.org + (long long)y * P.pitch + x;
     const long long os = P.org + (long long)map_index(y, P.ny, P.py) * P.pitch + map_index(x, P.nx, P.px);
-    const T inv = T(1) / psi[os];
+    const T inv = dev::rcp(psi[os]);
 #pragma unroll
     for (int i = 0; i < NP - 1; ++i) {
         T s = T(0);

@@ -186,20 +186,31 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
     k.gw2 = (T)(wd / cs2);
     k.lw1 = (T)(wa / cs2);
     k.lw2 = (T)(wd / cs2);
+    k.lk1 = (T)(0.75 * p->width * wa / cs2);
+    k.lk2 = (T)(0.75 * p->width * wd / cs2);
+    k.w9[0] = (T)w0;
+    k.w9[1] = (T)wa;
+    k.w9[2] = (T)wd;
     k.w1d[0] = (T)(d0 / 2.0);
     k.w1d[1] = (T)(1.0 - d0);
     k.w1d[2] = (T)(d0 / 2.0);
     for (int i = 0; i < N; ++i) {
         k.rho[i] = (T)p->rho[i];
         k.nu[i] = (T)p->nu[i];
+        k.drho[i] = (T)(p->rho[i] - p->rho[N - 1]);
+        k.dnu[i] = (T)(p->nu[i] - p->nu[N - 1]);
+        double b2 = 0.0;
         k.sigN[i] = (T)p->sigma[i][N - 1];
         for (int j = 0; j < N; ++j) {
             const double s = p->sigma[i][j];
+            k.sig[i][j] = (T)s;
+            b2 += 2.0 * 3.0 * s / p->width;
             k.beta2[i][j] = (T)(i == j ? 0.0 : 2.0 * 3.0 * s / p->width);  // 2 beta, beta = 3 sigma / eps
             k.kap[i][j] = (T)(0.75 * p->width * s);                       // -kappa_ij = 3 eps sigma / 4
             k.wet[i][j] = (T)(3.0 * s);
             k.invsig[i][j] = (T)(i == j ? 0.0 : 1.0 / s);
         }
+        k.beta2s[i] = (T)b2;
     }
     k.m0 = (T)p->m0;
     // Hermite norms N_ab = n_a n_b, n = (1, d0, d0 (1 - d0)), order
@@ -214,9 +225,13 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
         const double s[9] = {p->s_f[0], s1, s1, p->s_f[1], p->s_f[1], p->s_f[2],
                              p->s_f[3], p->s_f[3], p->s_f[4]};
         for (int a = 0; a < 9; ++a) k.lamf[i][a] = (T)(s[a] / Nab[a]);
+        k.ceta[i] = (T)(cs2 * p->eta[i]);
+        k.cV[i] = (T)(0.5 * s1 / n1 - 1.0 / n1);
     }
     k.lg00 = (T)(p->s_g[0]);
     k.lg1 = (T)(p->s_g[1] / n1);
+    k.cg0 = (T)(0.5 * p->s_g[0] - 1.0);
+    k.cg1 = (T)(0.5 * p->s_g[1] / n1 - 1.0 / n1);
     k.lg3 = (T)(p->s_g[2] / (n1 * n2));
     k.lg4 = (T)(p->s_g[3] / (n2 * n2));
     k.invN20 = (T)(1.0 / n2);
@@ -235,6 +250,9 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
     // |u|^2 and m^C.u coefficient of Eq. 19 once s_0 = -w0 psi m.u / (1 - cs2)
     k.gam = (T)(K / 2.0 - w0 / (1.0 - cs2));
     k.c2m3cs2 = (T)(1.0 - 3.0 * cs2);
+    k.two_cs2 = (T)(2.0 * cs2);
+    k.cs4 = (T)(cs2 * cs2);
+    k.one_m_cs2 = (T)(1.0 - cs2);
     k.body[0] = (T)p->body_force[0];
     k.body[1] = (T)p->body_force[1];
 }

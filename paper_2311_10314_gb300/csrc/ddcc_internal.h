@@ -33,8 +33,13 @@ struct KParams {
     T cs2, inv_cs2;
     T gw1, gw2;                   // w_axis / cs2, w_diag / cs2 (gradient stencil)
     T lw1, lw2;                   // w_axis / cs2, w_diag / cs2 (div(psi grad) stencil)
+    T lk1, lk2;                   // (3 eps / 4) times lw1, lw2
     T w1d[3];                     // 1D weights of c = -1, 0, +1: d0/2, 1-d0, d0/2
+    T w9[3];                      // 2D weights: rest, axis, diagonal
     T rho[kMaxPhases], nu[kMaxPhases];
+    T drho[kMaxPhases], dnu[kMaxPhases];   // rho_j - rho_N, nu_j - nu_N
+    T sig[kMaxPhases][kMaxPhases];     // sigma_ij
+    T beta2s[kMaxPhases];              // sum_{j != i} 2 beta_ij
     T beta2[kMaxPhases][kMaxPhases];   // 2 beta_ij = 6 sigma_ij / eps
     T kap[kMaxPhases][kMaxPhases];     // 3 eps sigma_ij / 4
     T wet[kMaxPhases][kMaxPhases];     // 3 sigma_ij
@@ -42,6 +47,8 @@ struct KParams {
     T invsig[kMaxPhases][kMaxPhases];  // 1 / sigma_ij (0 on the diagonal)
     T cos_uni[kMaxPhases];             // cos(theta_iN) when uniform
     T eta[kMaxPhases];
+    T ceta[kMaxPhases];                // cs2 eta_i
+    T cV[kMaxPhases];                  // coefficient of V in the first moments: lambda_1 / 2 - 1 / N_1
     T m0;
     // phase LB: lambda_ab = s_ab / N_ab in moment order
     // (00, 10, 01, 20, 02, 11, 21, 12, 22), and 1 / N_ab
@@ -49,6 +56,7 @@ struct KParams {
     T invN[9];
     // flow LB constant rates as lambda = s / N (00, 10, 01, 21, 12, 22)
     T lg00, lg1, lg3, lg4;
+    T cg0, cg1;                   // lg00 / 2 - 1 and lg1 / 2 - 1 / N_1
     T invN20, invN11;             // 1 / N for the per-node s21 and s22 rows
     T nu_to_s21, nu_to_s22;       // 2 / (1 - cs2) and 1 / cs2 (Eq. 16)
     T damp;                       // 1 / eps0^3
@@ -59,6 +67,7 @@ struct KParams {
     T cP;                         // cs2 / (1 - w0)
     T gam;                        // K / 2 - w0 / (1 - cs2)
     T c2m3cs2;                    // 1 - 3 cs2
+    T two_cs2, cs4, one_m_cs2;    // 2 cs2, cs2^2, 1 - cs2
     T body[2];
 };
 

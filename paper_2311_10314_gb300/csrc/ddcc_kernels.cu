@@ -89,6 +89,7 @@ __device__ void compute_mu_tile(const KParams<T>& P, Smem<T, NP>& sm, int tid) {
 
 template <typename T, int NP>
 struct TileAcc {
+    const KParams<T>& P;
     const Smem<T, NP>& sm;
     int cy, cx, hy, hx;
     long long o, plane;
@@ -97,6 +98,9 @@ struct TileAcc {
     const T* __restrict__ gin;
     __device__ T C(int j, int dy, int dx) const { return sm.C[j][cy + dy][cx + dx]; }
     __device__ T psi(int dy, int dx) const { return sm.psi[cy + dy][cx + dx]; }
+    __device__ T psi_rho(int dy, int dx) const {
+        return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
+    }
     __device__ T mu(int j, int dy, int dx) const { return sm.mu[j][hy + dy][hx + dx]; }
     __device__ T a(int dy, int dx) const { return sm.a[hy + dy][hx + dx]; }
     __device__ T lag(int k) const { return lag_in[k * plane + o]; }
@@ -178,7 +182,7 @@ __global__ void __launch_bounds__(NT) k_step(KParams<T> P, Fields<T> F, int cur)
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
     const long long o = P.org + (long long)y * P.pitch + x;
-    TileAcc<T, NP> acc{sm, (int)threadIdx.y + 2, (int)threadIdx.x + 2, (int)threadIdx.y + 1,
+    TileAcc<T, NP> acc{P, sm, (int)threadIdx.y + 2, (int)threadIdx.x + 2, (int)threadIdx.y + 1,
                        (int)threadIdx.x + 1, o, P.plane, lag_in, fin, gin};
     TileSink<T, NP> sink;
     sink.o = o;
@@ -238,12 +242,16 @@ struct TLay {
 template <typename T, int NP, bool TF>
 struct TmaAcc {
     using L = TLay<T, NP, TF>;
+    const KParams<T>& P;
     const T* sm;
     int tx, ty;
     __device__ T C(int j, int dy, int dx) const {
         return sm[L::c_off + ((size_t)j * (BY + 4) + ty + 2 + dy) * L::HX + tx + 4 + dx];
     }
     __device__ T psi(int dy, int dx) const { return sm[L::st_off + (size_t)(ty + 2 + dy) * L::HX + tx + 4 + dx]; }
+    __device__ T psi_rho(int dy, int dx) const {
+        return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
+    }
     __device__ T mu(int j, int dy, int dx) const {
         return sm[L::mu_off + ((size_t)j * (BY + 2) + ty + 1 + dy) * (BX + 2) + tx + 1 + dx];
     }
@@ -322,7 +330,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
     const long long o = P.org + (long long)y * P.pitch + x;
-    TmaAcc<T, NP, TF> acc{sm, (int)threadIdx.x, (int)threadIdx.y};
+    TmaAcc<T, NP, TF> acc{P, sm, (int)threadIdx.x, (int)threadIdx.y};
     TileSink<T, NP> sink;
     sink.o = o;
     sink.plane = P.plane;
@@ -373,7 +381,7 @@ struct FLay {
     static constexpr int LAG_BOX = NLAG * BY * BX;
     static constexpr int ST_BOX = NST * HY * HX;
     static constexpr int A_BOX = (BY + 2) * HX;
-    static constexpr int C_ARR = (NP - 1) * HY * HX;
+    static constexpr int C_ARR = (sizeof(T) == 8 ? NP : NP - 1) * HY * HX;   // C_i, and in FP64 psi rho
     static constexpr int MU = NP * (BY + 2) * (BX + 2);
     static constexpr size_t fh_off = 0;
     static constexpr size_t g_off = fh_off + pad(FH_BOX);
@@ -392,12 +400,17 @@ struct FLay {
 template <typename T, int NP, bool TF>
 struct FusedAcc {
     using L = FLay<T, NP, TF>;
+    const KParams<T>& P;
     const T* sm;
     int tx, ty;
     __device__ T C(int j, int dy, int dx) const {
         return sm[L::c_off + ((size_t)j * L::HY + ty + 2 + dy) * L::HX + tx + 4 + dx];
     }
     __device__ T psi(int dy, int dx) const { return sm[L::st_off + (size_t)(ty + 2 + dy) * L::HX + tx + 4 + dx]; }
+    __device__ T psi_rho(int dy, int dx) const {
+        if constexpr (sizeof(T) == 8) return C(NP - 1, dy, dx);
+        else return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
+    }
     __device__ T mu(int j, int dy, int dx) const {
         return sm[L::mu_off + ((size_t)j * (BY + 2) + ty + 1 + dy) * (BX + 2) + tx + 1 + dx];
     }
@@ -460,17 +473,52 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
         }
         return;
     }
-    // C_i = sum_p f^i_p / psi on the tile + 2-node halo (12 x 36 nodes)
-    for (int k = tid; k < L::HY * (BX + 4); k += NT) {
-        const int cy = k / (BX + 4), cx = k - cy * (BX + 4) + 2;   // box column of node x0-2+..
-        const T inv = T(1) / sm[L::st_off + (size_t)cy * L::HX + cx];
-        const T* fb = sm + L::fh_off + (size_t)cy * L::HX + cx;
+    // C_i = sum_p f^i_p / psi on the tile + 2-node halo.  FP32: four columns
+    // of one phase per item as 16-byte accesses over whole box rows (40
+    // columns), so a warp reads consecutive quads: node by node over the 36
+    // columns needed, every warp spanned two rows and met two-way bank
+    // conflicts (256 x 256, N = 3: 11.0 -> 10.3 us a step).  FP64 (bound by its FP64 pipe): only the 12 x 36 nodes
+    // needed, and psi rho, which the update differentiates, once per node
+    // here instead of once per neighbour there.
+    if constexpr (sizeof(T) == 4) {
+        constexpr int NQ = L::HY * L::HX / 4, PL = L::HY * L::HX;
 #pragma unroll
-        for (int i = 0; i < NP - 1; ++i) {
-            T s = T(0);
+        for (int r = 0; r < ((NP - 1) * NQ + NT - 1) / NT; ++r) {
+            const int k = tid + r * NT;
+            if (k < (NP - 1) * NQ) {
+                const int i = k / NQ, o = 4 * (k - i * NQ);
+                const T* fb = sm + L::fh_off + (size_t)(9 * i) * PL + o;
+                float4 c = *reinterpret_cast<const float4*>(fb);
 #pragma unroll
-            for (int p = 0; p < 9; ++p) s += fb[(size_t)(9 * i + p) * L::HY * L::HX];
-            sm[L::c_off + ((size_t)i * L::HY + cy) * L::HX + cx] = s * inv;
+                for (int p = 1; p < 9; ++p) {
+                    const float4 v = *reinterpret_cast<const float4*>(fb + (size_t)p * PL);
+                    c.x += v.x;
+                    c.y += v.y;
+                    c.z += v.z;
+                    c.w += v.w;
+                }
+                const float4 ps = *reinterpret_cast<const float4*>(sm + L::st_off + o);
+                *reinterpret_cast<float4*>(sm + L::c_off + (size_t)i * PL + o) =
+                    make_float4(c.x * dev::rcp(ps.x), c.y * dev::rcp(ps.y), c.z * dev::rcp(ps.z),
+                                c.w * dev::rcp(ps.w));
+            }
+        }
+    } else {
+        for (int k = tid; k < L::HY * (BX + 4); k += NT) {
+            const int cy = k / (BX + 4), cx = k - cy * (BX + 4) + 2;   // box column of node x0-2+..
+            const T psi = sm[L::st_off + (size_t)cy * L::HX + cx];
+            const T inv = dev::rcp(psi);
+            const T* fb = sm + L::fh_off + (size_t)cy * L::HX + cx;
+            T* cb = sm + L::c_off + (size_t)cy * L::HX + cx;
+            T Cv[NP - 1];
+#pragma unroll
+            for (int i = 0; i < NP - 1; ++i) {
+                T s = fb[(size_t)(9 * i) * L::HY * L::HX];
+#pragma unroll
+                for (int p = 1; p < 9; ++p) s += fb[(size_t)(9 * i + p) * L::HY * L::HX];
+                cb[(size_t)i * L::HY * L::HX] = Cv[i] = s * inv;
+            }
+            cb[(size_t)(NP - 1) * L::HY * L::HX] = dev::psi_rho<T, NP>(P, psi, [&](int j) { return Cv[j]; });
         }
     }
     __syncthreads();
@@ -501,7 +549,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
     const long long o = P.org + (long long)y * P.pitch + x;
-    FusedAcc<T, NP, TF> acc{sm, (int)threadIdx.x, (int)threadIdx.y};
+    FusedAcc<T, NP, TF> acc{P, sm, (int)threadIdx.x, (int)threadIdx.y};
     // most tiles push only into the domain's interior: fixed neighbour
     // offsets, no wrap or bounce-back, 32-bit offsets (a block-uniform branch)
     if (off32 && x0 >= 1 && y0 >= 1 && x0 + BX < P.nx && y0 + BY < P.ny) {
@@ -610,7 +658,7 @@ __global__ void __launch_bounds__(256) k_order_param(KParams<T> P, const T* __re
          idx += (long long)gridDim.x * blockDim.x) {
         const int y = (int)(idx / P.nx), x = (int)(idx - (long long)y * P.nx);
         const long long o = P.org + (long long)y * P.pitch + x;
-        const T inv = T(1) / psi[o];
+        const T inv = dev::rcp(psi[o]);
 #pragma unroll
         for (int i = 0; i < NP - 1; ++i) {
             T s = T(0);

@@ -119,6 +119,7 @@ struct Rings {
 template <typename T, int NP, bool TF>
 struct SweepAcc {
     using L = Lay<T, NP, TF>;
+    const KParams<T>& P;
     const T* st_r[3];
     const T* lag_r[3];
     const T* pop_r;
@@ -126,6 +127,9 @@ struct SweepAcc {
     const T* M_r[3];
     __device__ T C(int j, int dy, int dx) const { return C_r[dy + 1][j * L::CW + 2 + dx]; }
     __device__ T psi(int dy, int dx) const { return st_r[dy + 1][4 + dx]; }
+    __device__ T psi_rho(int dy, int dx) const {
+        return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
+    }
     __device__ T mu(int j, int dy, int dx) const { return M_r[dy + 1][j * L::MW + 1 + dx]; }
     __device__ T a(int dy, int dx) const { return lag_r[dy + 1][4 + dx]; }
     __device__ T lag(int k) const { return lag_r[1][k * L::PLANE + 4]; }
@@ -233,7 +237,7 @@ __global__ void __launch_bounds__(Lay<T, NP, TF>::NT, 1)
     auto compute_C = [&](int y0r, int nrows) {
         for (int k = tid; k < nrows * L::CW; k += NT) {
             const int row = y0r + k / L::CW, c = k % L::CW;
-            const T inv = T(1) / R.st_row(row)[c + 2];
+            const T inv = dev::rcp(R.st_row(row)[c + 2]);
             const T* pr = R.pop_row(row) + c + 2;
 #pragma unroll
             for (int i = 0; i < NP - 1; ++i) {
@@ -327,7 +331,7 @@ __global__ void __launch_bounds__(Lay<T, NP, TF>::NT, 1)
         const int y = r + ty;
         if (tx < W && x < P.nx && y < yb) {
             const long long o = P.org + (long long)y * P.pitch + x;
-            SweepAcc<T, NP, TF> acc;
+            SweepAcc<T, NP, TF> acc{P};
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 acc.st_r[d] = R.st_row(y - 1 + d) + tx;
