@@ -128,10 +128,11 @@ struct SweepArgs {
 // TMA-staged tile collide-stream kernel: 32 x 8 tiles whose populations,
 // lagged planes and stencil halos arrive by tensor copies.
 constexpr int kTileHaloW = kTileX + 8;   // halo box: tile + 4 columns a side
+constexpr int kWideX = 64, kWideY = 4;   // the fused kernel's other tile (fused_tile_wide)
 template <typename T>
 struct TileTmaArgs {
-    const CUtensorMap* tm_pop;   // box {32, 8, 9N} over the input population planes, or
-                                 // (fused kernel) box {40, 12, 9(N-1)} over the f planes
+    const CUtensorMap* tm_pop;   // box {32, 8, 9N} over the input population planes, or (fused
+                                 // kernel, TX x TY tiles) {TX+8, TY+4, 9(N-1)} over the f planes
     const CUtensorMap* tm_g;     // (fused kernel) box {32, 8, 9} over the input g planes
     const CUtensorMap* tm_lag;   // box {32, 8, 2N+3} over the input lagged planes
     const CUtensorMap* tm_c;     // box {40, 12, N-1} over the order-parameter planes
@@ -141,13 +142,14 @@ struct TileTmaArgs {
     T* pop_out;
     T* lag_out;
     int* err;
+    int wide;                    // (fused kernel) 64 x 4 tiles instead of 32 x 8
 };
 template <typename T>
 size_t tile_tma_smem_bytes(int N, bool theta_field);
 template <typename T>
 cudaError_t launch_collide_tma(const TileTmaArgs<T>& a, cudaStream_t s);
 template <typename T>
-size_t tile_fused_smem_bytes(int N, bool theta_field);
+size_t tile_fused_smem_bytes(int N, bool theta_field, bool wide);
 template <typename T>
 cudaError_t launch_collide_fused(const TileTmaArgs<T>& a, cudaStream_t s);
 

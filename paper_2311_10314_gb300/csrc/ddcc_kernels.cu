@@ -368,21 +368,21 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
 // resident CTAs.
 constexpr int kPrefetchQuarterWaves = 3;
 
-template <typename T, int NP, bool TF>
+template <typename T, int NP, bool TF, int TX, int TY>
 struct FLay {
     static constexpr int NF = 9 * (NP - 1);
     static constexpr int NLAG = 2 * NP + 3;
     static constexpr int NST = TF ? NP : 1;
-    static constexpr int HX = kTileHaloW;
-    static constexpr int HY = BY + 4;
+    static constexpr int HX = TX + 8;                        // halo box columns x0-4 .. x0+TX+3
+    static constexpr int HY = TY + 4;
     static constexpr int pad(int e) { return (e * (int)sizeof(T) + 127) / 128 * 128 / (int)sizeof(T); }
-    static constexpr int FH_BOX = NF * HY * HX;              // rows y0-2 .. y0+9, columns x0-4 .. x0+35
-    static constexpr int G_BOX = 9 * BY * BX;
-    static constexpr int LAG_BOX = NLAG * BY * BX;
+    static constexpr int FH_BOX = NF * HY * HX;              // rows y0-2 .. y0+TY+1
+    static constexpr int G_BOX = 9 * TY * TX;
+    static constexpr int LAG_BOX = NLAG * TY * TX;
     static constexpr int ST_BOX = NST * HY * HX;
-    static constexpr int A_BOX = (BY + 2) * HX;
+    static constexpr int A_BOX = (TY + 2) * HX;
     static constexpr int C_ARR = (sizeof(T) == 8 ? NP : NP - 1) * HY * HX;   // C_i, and in FP64 psi rho
-    static constexpr int MU = NP * (BY + 2) * (BX + 2);
+    static constexpr int MU = NP * (TY + 2) * (TX + 2);
     static constexpr size_t fh_off = 0;
     static constexpr size_t g_off = fh_off + pad(FH_BOX);
     static constexpr size_t lag_off = g_off + pad(G_BOX);
@@ -397,9 +397,9 @@ struct FLay {
     static constexpr unsigned tx_tile = (unsigned)((G_BOX + LAG_BOX) * sizeof(T));
 };
 
-template <typename T, int NP, bool TF>
+template <typename T, int NP, bool TF, int TX, int TY>
 struct FusedAcc {
-    using L = FLay<T, NP, TF>;
+    using L = FLay<T, NP, TF, TX, TY>;
     const KParams<T>& P;
     const T* sm;
     int tx, ty;
@@ -412,28 +412,28 @@ struct FusedAcc {
         else return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
     }
     __device__ T mu(int j, int dy, int dx) const {
-        return sm[L::mu_off + ((size_t)j * (BY + 2) + ty + 1 + dy) * (BX + 2) + tx + 1 + dx];
+        return sm[L::mu_off + ((size_t)j * (TY + 2) + ty + 1 + dy) * (TX + 2) + tx + 1 + dx];
     }
     __device__ T a(int dy, int dx) const { return sm[L::a_off + (size_t)(ty + 1 + dy) * L::HX + tx + 4 + dx]; }
-    __device__ T lag(int k) const { return sm[L::lag_off + ((size_t)k * BY + ty) * BX + tx]; }
+    __device__ T lag(int k) const { return sm[L::lag_off + ((size_t)k * TY + ty) * TX + tx]; }
     __device__ T f(int i, int p) const {
         return sm[L::fh_off + ((size_t)(9 * i + p) * L::HY + ty + 2) * L::HX + tx + 4];
     }
-    __device__ T g(int p) const { return sm[L::g_off + ((size_t)p * BY + ty) * BX + tx]; }
+    __device__ T g(int p) const { return sm[L::g_off + ((size_t)p * TY + ty) * TX + tx]; }
 };
 
-template <typename T, int NP, bool TF>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
+template <typename T, int NP, bool TF, int TX, int TY>
+__global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? 2 : 1)
     k_step_fused(const __grid_constant__ CUtensorMap tm_fh, const __grid_constant__ CUtensorMap tm_g,
                  const __grid_constant__ CUtensorMap tm_lag, const __grid_constant__ CUtensorMap tm_st,
                  const __grid_constant__ CUtensorMap tm_a, KParams<T> P, T* __restrict__ pop_out,
                  T* __restrict__ lag_out, int* __restrict__ err, int pf_dist, int off32) {
-    using L = FLay<T, NP, TF>;
+    using L = FLay<T, NP, TF, TX, TY>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     T* sm = reinterpret_cast<T*>(smem_raw);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw + L::bar_byte_off);
-    const int tid = threadIdx.x + BX * threadIdx.y;
-    const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
+    const int tid = threadIdx.x + TX * threadIdx.y;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     if (tid == 0) {
         tma::mbar_init(&bars[0], 1);
         tma::mbar_init(&bars[1], 1);
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
         // keeps streaming while the resident CTAs compute
         const int nb = gridDim.x * gridDim.y, b = blockIdx.y * gridDim.x + blockIdx.x + pf_dist;
         if (pf_dist > 0 && b < nb) {
-            const int px0 = (b % gridDim.x) * BX, py0 = (b / gridDim.x) * BY;
+            const int px0 = (b % gridDim.x) * TX, py0 = (b / gridDim.x) * TY;
             tma::prefetch_3d(&tm_fh, px0, py0 - 2 + kGY, 0);
             tma::prefetch_3d(&tm_st, px0, py0 - 2 + kGY, 0);
             tma::prefetch_3d(&tm_g, px0 + kGX, py0 + kGY, 0);
@@ -483,8 +483,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     if constexpr (sizeof(T) == 4) {
         constexpr int NQ = L::HY * L::HX / 4, PL = L::HY * L::HX;
 #pragma unroll
-        for (int r = 0; r < ((NP - 1) * NQ + NT - 1) / NT; ++r) {
-            const int k = tid + r * NT;
+        for (int r = 0; r < ((NP - 1) * NQ + (TX * TY) - 1) / (TX * TY); ++r) {
+            const int k = tid + r * (TX * TY);
             if (k < (NP - 1) * NQ) {
                 const int i = k / NQ, o = 4 * (k - i * NQ);
                 const T* fb = sm + L::fh_off + (size_t)(9 * i) * PL + o;
@@ -504,8 +504,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
             }
         }
     } else {
-        for (int k = tid; k < L::HY * (BX + 4); k += NT) {
-            const int cy = k / (BX + 4), cx = k - cy * (BX + 4) + 2;   // box column of node x0-2+..
+        for (int k = tid; k < L::HY * (TX + 4); k += (TX * TY)) {
+            const int cy = k / (TX + 4), cx = k - cy * (TX + 4) + 2;   // box column of node x0-2+..
             const T psi = sm[L::st_off + (size_t)cy * L::HX + cx];
             const T inv = dev::rcp(psi);
             const T* fb = sm + L::fh_off + (size_t)cy * L::HX + cx;
@@ -523,8 +523,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     }
     __syncthreads();
     // mu on the tile + 1-node halo
-    for (int k = tid; k < (BY + 2) * (BX + 2); k += NT) {
-        const int ly = k / (BX + 2), lx = k - ly * (BX + 2);
+    for (int k = tid; k < (TY + 2) * (TX + 2); k += (TX * TY)) {
+        const int ly = k / (TX + 2), lx = k - ly * (TX + 2);
         const T* cb = sm + L::c_off + (size_t)(ly + 1) * L::HX + lx + 3;
         const T* sb = sm + L::st_off + (size_t)(ly + 1) * L::HX + lx + 3;
         T cth[NP];
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
             P, [&](int j, int dy, int dx) { return cb[((size_t)j * L::HY + dy) * L::HX + dx]; },
             [&](int dy, int dx) { return sb[dy * L::HX + dx]; }, cth, mu);
 #pragma unroll
-        for (int i = 0; i < NP; ++i) sm[L::mu_off + ((size_t)i * (BY + 2) + ly) * (BX + 2) + lx] = mu[i];
+        for (int i = 0; i < NP; ++i) sm[L::mu_off + ((size_t)i * (TY + 2) + ly) * (TX + 2) + lx] = mu[i];
     }
     ok = tma::mbar_wait_bounded(&bars[1], 0);
     if (!__syncthreads_and(ok)) {
@@ -549,10 +549,10 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
     const long long o = P.org + (long long)y * P.pitch + x;
-    FusedAcc<T, NP, TF> acc{P, sm, (int)threadIdx.x, (int)threadIdx.y};
+    FusedAcc<T, NP, TF, TX, TY> acc{P, sm, (int)threadIdx.x, (int)threadIdx.y};
     // most tiles push only into the domain's interior: fixed neighbour
     // offsets, no wrap or bounce-back, 32-bit offsets (a block-uniform branch)
-    if (off32 && x0 >= 1 && y0 >= 1 && x0 + BX < P.nx && y0 + BY < P.ny) {
+    if (off32 && x0 >= 1 && y0 >= 1 && x0 + TX < P.nx && y0 + TY < P.ny) {
         InnerSink<T, NP> in{pop_out + o, lag_out + o, (int)P.plane, P.pitch};
         dev::node_update<T, NP, 0>(P, acc, in);
         return;
@@ -582,10 +582,10 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     dev::node_update<T, NP, 0>(P, acc, sink);
 }
 
-template <typename T, int NP, bool TF>
+template <typename T, int NP, bool TF, int TX, int TY>
 cudaError_t collide_fused_n(const TileTmaArgs<T>& a, cudaStream_t s) {
-    using L = FLay<T, NP, TF>;
-    const cudaError_t e = cudaFuncSetAttribute(k_step_fused<T, NP, TF>,
+    using L = FLay<T, NP, TF, TX, TY>;
+    const cudaError_t e = cudaFuncSetAttribute(k_step_fused<T, NP, TF, TX, TY>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
     if (e != cudaSuccess) return e;
     const KParams<T>& kp = *a.kp;
@@ -597,7 +597,7 @@ cudaError_t collide_fused_n(const TileTmaArgs<T>& a, cudaStream_t s) {
     const int pf_dist = kPrefetchQuarterWaves * sms * (sizeof(T) == 4 ? 2 : 1) / 4;
     // the inner tiles' 32-bit offsets reach every population and lagged plane
     const int off32 = (long long)(9 * NP) * kp.plane < (1LL << 31) ? 1 : 0;
-    k_step_fused<T, NP, TF><<<dim3((kp.nx + BX - 1) / BX, (kp.ny + BY - 1) / BY), dim3(BX, BY), L::bytes, s>>>(
+    k_step_fused<T, NP, TF, TX, TY><<<dim3((kp.nx + TX - 1) / TX, (kp.ny + TY - 1) / TY), dim3(TX, TY), L::bytes, s>>>(
         *a.tm_pop, *a.tm_g, *a.tm_lag, *a.tm_st, *a.tm_a, kp, a.pop_out, a.lag_out, a.err, pf_dist, off32);
     return cudaGetLastError();
 }
@@ -957,30 +957,45 @@ size_t tile_tma_smem_bytes(int N, bool tf) {
         default: return 0;
     }
 }
-template <typename T>
-size_t tile_fused_smem_bytes(int N, bool tf) {
+// The fused kernel's tile: 32 x 8, or in FP32 64 x 4 (see fused_tile_wide).
+template <typename T, int TX, int TY>
+size_t fused_smem_shape(int N, bool tf) {
     switch (N * 2 + (tf ? 1 : 0)) {
-        case 4: return FLay<T, 2, false>::bytes;
-        case 5: return FLay<T, 2, true>::bytes;
-        case 6: return FLay<T, 3, false>::bytes;
-        case 7: return FLay<T, 3, true>::bytes;
-        case 8: return FLay<T, 4, false>::bytes;
-        case 9: return FLay<T, 4, true>::bytes;
+        case 4: return FLay<T, 2, false, TX, TY>::bytes;
+        case 5: return FLay<T, 2, true, TX, TY>::bytes;
+        case 6: return FLay<T, 3, false, TX, TY>::bytes;
+        case 7: return FLay<T, 3, true, TX, TY>::bytes;
+        case 8: return FLay<T, 4, false, TX, TY>::bytes;
+        case 9: return FLay<T, 4, true, TX, TY>::bytes;
         default: return 0;
     }
 }
 template <typename T>
-cudaError_t launch_collide_fused(const TileTmaArgs<T>& a, cudaStream_t s) {
+size_t tile_fused_smem_bytes(int N, bool tf, bool wide) {
+    if constexpr (sizeof(T) == 4) {
+        if (wide) return fused_smem_shape<T, kWideX, kWideY>(N, tf);
+    }
+    return fused_smem_shape<T, BX, BY>(N, tf);
+}
+template <typename T, int TX, int TY>
+cudaError_t fused_shape(const TileTmaArgs<T>& a, cudaStream_t s) {
     const bool tf = a.kp->has_cos_field != 0;
     switch (a.kp->N * 2 + (tf ? 1 : 0)) {
-        case 4: return collide_fused_n<T, 2, false>(a, s);
-        case 5: return collide_fused_n<T, 2, true>(a, s);
-        case 6: return collide_fused_n<T, 3, false>(a, s);
-        case 7: return collide_fused_n<T, 3, true>(a, s);
-        case 8: return collide_fused_n<T, 4, false>(a, s);
-        case 9: return collide_fused_n<T, 4, true>(a, s);
+        case 4: return collide_fused_n<T, 2, false, TX, TY>(a, s);
+        case 5: return collide_fused_n<T, 2, true, TX, TY>(a, s);
+        case 6: return collide_fused_n<T, 3, false, TX, TY>(a, s);
+        case 7: return collide_fused_n<T, 3, true, TX, TY>(a, s);
+        case 8: return collide_fused_n<T, 4, false, TX, TY>(a, s);
+        case 9: return collide_fused_n<T, 4, true, TX, TY>(a, s);
         default: return cudaErrorInvalidValue;
     }
+}
+template <typename T>
+cudaError_t launch_collide_fused(const TileTmaArgs<T>& a, cudaStream_t s) {
+    if constexpr (sizeof(T) == 4) {
+        if (a.wide) return fused_shape<T, kWideX, kWideY>(a, s);
+    }
+    return fused_shape<T, BX, BY>(a, s);
 }
 template <typename T>
 cudaError_t launch_collide_tma(const TileTmaArgs<T>& a, cudaStream_t s) {
@@ -1065,7 +1080,7 @@ cudaError_t launch_wall_accumulate(const KParams<T>& kp, const T* stage, T* psi,
     template cudaError_t launch_fill_ghosts2<T>(const GhostRing<T>&, const GhostRing<T>&, const KParams<T>&,    \
                                                 cudaStream_t);                                            \
     template size_t tile_tma_smem_bytes<T>(int, bool);                                           \
-    template size_t tile_fused_smem_bytes<T>(int, bool);                                         \
+    template size_t tile_fused_smem_bytes<T>(int, bool, bool);                                   \
     template cudaError_t launch_walls_init<T>(const KParams<T>&, T*, T*, cudaStream_t);          \
     template cudaError_t launch_open_bc<T>(const KParams<T>&, T*, T*, const T*, const T*, cudaStream_t); \
     template cudaError_t launch_wall_accumulate<T>(const KParams<T>&, const T*, T*, T*, cudaStream_t); \

@@ -1,0 +1,52 @@
+"""The step's kernel variants, each chosen by a rule on sizes and types, at the
+sizes where it can go wrong, against the FP64 oracle: edges of tiles,
+remainders, the smallest and largest of a variant's range.
+
+Bars: those of the parity tests -- FP64 1e-10 in C on psi >= 0.01 and in u,
+FP32 2e-5 in C and 1e-6 in u after a few steps.
+"""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+from oracle import Oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def D():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2311_10314_gb300 import build as B
+    B.build()
+    import paper_2311_10314_gb300 as D
+    return D
+
+
+def _against_oracle(D, pb, precision, steps, **kw):
+    o = Oracle(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field)
+    o.step(steps)
+    ref = {k: v.numpy() for k, v in o.macroscopic().items()}
+    sim = D.Sim(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field, precision=precision, **kw)
+    sim.step(steps)
+    got = sim.fields()
+    sim.close()
+    fl = pb.psi >= 0.01
+    tc, tu = (1e-10, 1e-10) if precision == D.DDCC_FP64 else (2e-5, 1e-6)
+    assert np.abs(ref["C"] - got["C"])[:, fl].max() <= tc
+    assert max(np.abs(ref[k] - got[k])[fl].max() for k in ("ux", "uy")) <= tu
+
+
+@pytest.mark.parametrize("nx,ny,N,py,field", [
+    (64, 5601, 4, 1, True),      # one tile wide, one row over a tile
+    (191, 1871, 4, 0, False),    # a column short of three tiles, walls
+    (256, 2300, 3, 1, True),
+    (641, 1201, 2, 0, True),     # one column into the eleventh tile
+])
+def test_fp32_wide_tiles(D, nx, ny, N, py, field):
+    """States beyond L2 (over 64 MB) take the 64 x 4 tiles in FP32."""
+    assert nx * ny * (11 * N + 3) * 4 > 64 << 20
+    pb = W.random_problem(nx, ny, N, seed=nx + N, periodic_y=py, theta_field=field, width=6.0, n_circles=12, n_drops=9)
+    _against_oracle(D, pb, D.DDCC_FP32, 3)
