@@ -110,7 +110,8 @@ typedef struct ddcc_handle ddcc_handle;
  * Bytes of device workspace ddcc_create() needs for these parameters, or 0
  * if they are invalid.  The workspace holds two copies of the populations
  * and of the lagged fields (ping-pong), psi, the contact-angle field, the
- * order-parameter scratch and reduction scratch.
+ * order-parameter scratch and reduction scratch; in FP64 also the chemical
+ * potentials and psi rho of the current step and the terms of psi alone.
  */
 size_t ddcc_workspace_bytes(const ddcc_params* params);
 
@@ -185,7 +186,7 @@ int ddcc_set_inflow(ddcc_handle* h, const double* u_in, const double* C_in);
 /*
  * Advance nsteps >= 0 time steps (Eqs. 3.1 and 3.2 with the equilibria,
  * sources, velocity and pressure of Sec. 3).  Asynchronous on the stream.
- * On the fused tile path, calls of four steps or more replay a CUDA graph of
+ * On the fused tile path and the FP64 path, calls of four steps or more replay a CUDA graph of
  * two steps, captured on the first such call (not while profiling); the
  * arithmetic is the same as launching the kernels one by one.
  */
@@ -268,8 +269,8 @@ int ddcc_set_rows(ddcc_handle* h, int y0, int nrows, const void* dev_buf);
  * stream, writes for each kernel kind k < max_kinds the summed device time
  * in milliseconds (ms_out[k]) and the number of launches (launches_out[k]),
  * clears the record and returns the number of kinds (4: 0 = order
- * parameters and 1 = collide-stream of the tile path, 2 = row sweep,
- * 3 = ghost-frame fills of the tile path).
+ * parameters (in FP64 with the chemical potentials) and 1 = collide-stream of
+ * the tile path, 2 = row sweep, 3 = ghost-frame fills of the tile path).
  * Either output may be NULL.
  */
 int ddcc_profile(ddcc_handle* h, int enable);
@@ -277,10 +278,11 @@ int ddcc_kernel_times(ddcc_handle* h, double* ms_out, int64_t* launches_out, int
 
 /*
  * Which kernels ddcc_step() runs for this handle: DDCC_PATH_TILE (the
- * default: one TMA-staged tile kernel that forms the order parameters from
- * the staged phase populations and makes the whole update, plus two small
- * ghost-frame fills; grids narrower than its halo boxes fall back to an
- * order-parameter pass and a plain-load tile kernel) or DDCC_PATH_SWEEP
+ * default.  FP32: one TMA-staged tile kernel that forms the order parameters
+ * from the staged phase populations and makes the whole update, plus a
+ * ghost-frame fill; grids narrower than its halo boxes fall back to an
+ * order-parameter pass and a plain-load tile kernel.  FP64: one kernel for
+ * the volume fractions and chemical potentials, one for the update) or DDCC_PATH_SWEEP
  * (with DDCC_FLAG_SWEEP, when the grid is at least one sweep strip wide and
  * 8 rows high and the device has the shared memory).
  */
@@ -313,9 +315,10 @@ size_t ddcc_adjoint_bytes(const ddcc_handle* h);
  * ddcc_save_state() layout, 256-byte aligned, distinct), leaving the
  * handle's own state and step count untouched; the adjoint sweep uses it to
  * recompute a checkpointed segment without copying.  state_in must have
- * filled ghost frames, as every state the library writes has; state_out
- * gets them.  The step-count word of state_out is not written.  Only the
- * fused tile path provides it: DDCC_ERR_UNSUPPORTED otherwise (the caller
+ * the ghost rings that the step and ddcc_adjoint_step read (of the phase
+ * populations and of plane a), as every state the library writes for that
+ * precision has; state_out gets them.  The step-count word of state_out is
+ * not written.  Only the fused tile path and the FP64 path provide it: DDCC_ERR_UNSUPPORTED otherwise (the caller
  * then loads, steps and saves).
  */
 int ddcc_step_between(ddcc_handle* h, const void* state_in, void* state_out);

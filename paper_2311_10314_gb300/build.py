@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libddcc.so")
-SOURCES = ["ddcc_kernels.cu", "ddcc_sweep.cu", "ddcc_api.cu", "ddcc_noalloc.cu", "ddcc_adjoint.cu", "ddcc_selftest.cu",
+SOURCES = ["ddcc_kernels.cu", "ddcc_fp64.cu", "ddcc_sweep.cu", "ddcc_api.cu", "ddcc_noalloc.cu", "ddcc_adjoint.cu", "ddcc_selftest.cu",
            "ddcc_peak.cu", "ddcc_slab.cu", "ddcc3d.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # Single-precision division and square root use the hardware approximations

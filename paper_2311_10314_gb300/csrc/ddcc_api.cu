@@ -41,7 +41,7 @@ struct ddcc_handle {
     CUtensorMap tm_pop[2], tm_lag[2], tm_st;
     // TMA-staged tile kernel
     int n_walls;          // solids given by their own psi_k (ddcc_create_walls), else 0
-    int use_tile_tma;     // 1: halo-staged tile kernel, 2: fused order parameters
+    int use_tile_tma;     // FP32 1: halo-staged tile kernel, 2: fused order parameters; FP64 3: ddcc_fp64.cu
     int tile_wide;        // the fused kernel runs 64 x 4 tiles instead of 32 x 8
     CUtensorMap tt_pop[2], tt_lag[2], tt_c, tt_st, tt_a[2], tt_fh[2], tt_g[2];
     // the fused tile step as a CUDA graph of two steps (from copy 0 back to
@@ -132,7 +132,7 @@ bool valid_params(const ddcc_params* p) {
 }
 
 struct Layout {
-    size_t pop[2], lag[2], st, C, macro, partial, stage, inflow, mass, flag, total;
+    size_t pop[2], lag[2], st, C, macro, mu, chi, st64, partial, stage, inflow, mass, flag, total;
     size_t plane_bytes;
 };
 
@@ -157,6 +157,11 @@ Layout layout_of(const ddcc_params* p) {
     L.st = take(pb * N);
     L.C = take(pb * (N - 1));
     L.macro = take(pb * (2 * N + 4));
+    if (p->precision == DDCC_FP64) {
+        L.mu = take(pb * N);
+        L.chi = take(pb);
+        L.st64 = take(pb * static64_planes());
+    }
     L.partial = take(sizeof(double) * kMassBlocks * kMaxPhases);
     L.stage = take(sizeof(double) * (size_t)p->nx * p->ny * (N - 1));
     L.inflow = take(es * (size_t)p->ny * N);
@@ -286,6 +291,11 @@ void carve(ddcc_handle* h, const Layout& L, Fields<T>& f) {
     f.cosf = reinterpret_cast<T*>(b + L.st + L.plane_bytes);
     f.C = reinterpret_cast<T*>(b + L.C);
     f.macro = reinterpret_cast<T*>(b + L.macro);
+    if (sizeof(T) == 8) {
+        f.mu = reinterpret_cast<T*>(b + L.mu);
+        f.chi = reinterpret_cast<T*>(b + L.chi);
+        f.st64 = reinterpret_cast<T*>(b + L.st64);
+    }
     f.partial = reinterpret_cast<double*>(b + L.partial);
     f.stage = reinterpret_cast<double*>(b + L.stage);
     f.inflow = reinterpret_cast<T*>(b + L.inflow);
@@ -397,10 +407,9 @@ int setup_sweep(ddcc_handle* h) {
 // Smaller states stay in L2, where the 32 x 8 tile's smaller halo counts
 // (256 x 256, N = 3: 10.3 us a step against 11.2).  More rows of tiles than
 // a launch grid has keep the taller tile.
-// FP64 is bound by its FP64 pipe: the tile with the smaller halo.
 template <typename T>
 bool fused_tile_wide(const ddcc_params& p) {
-    if (sizeof(T) != 4 || p.nx < kWideX || (p.ny + kWideY - 1) / kWideY > 65535) return false;
+    if (p.nx < kWideX || (p.ny + kWideY - 1) / kWideY > 65535) return false;
     const int pad_wide = (p.nx + kWideX - 1) / kWideX * kWideX, pad = (p.nx + kTileX - 1) / kTileX * kTileX;
     const long long state = (long long)p.nx * p.ny * (11 * p.nphase + 3) * (long long)sizeof(T);
     return pad_wide <= pad + pad / 16 && state > kWideStateBytes;
@@ -508,6 +517,7 @@ int create_t(ddcc_handle* h, const double* psi, const double* cosf, const double
         if (cosf && (st = upload<T>(h, cosf, f.cosf, N - 1))) return st;
     }
     DDCC_CU(launch_fill_ghosts<T>(f.psi, k.has_cos_field ? N : 1, k, h->stream));
+    if constexpr (sizeof(T) == 8) DDCC_CU(launch_static64(k, f.psi, f.st64, h->stream));
     st = upload<T>(h, C0, f.C, N - 1);
     if (st) return st;
     DDCC_CU(launch_init<T>(k, f, 0, h->stream));
@@ -515,7 +525,19 @@ int create_t(ddcc_handle* h, const double* psi, const double* cosf, const double
     DDCC_CU(launch_fill_ghosts<T>(f.lag[0], lag_planes(N), k, h->stream));
     const int st2 = setup_sweep<T>(h);
     if (st2) return st2;
-    return h->use_sweep ? DDCC_OK : setup_tile_tma<T>(h);
+    if (h->use_sweep) return DDCC_OK;
+    if constexpr (sizeof(T) == 8) {
+        h->use_tile_tma = 3;
+        return DDCC_OK;
+    } else {
+        return setup_tile_tma<T>(h);
+    }
+}
+
+// The FP64 step's arguments: populations and lagged planes in and out.
+Step64Args args64(const Fields<double>& f, const double* pop_in, const double* lag_in, double* pop_out,
+                  double* lag_out) {
+    return Step64Args{pop_in, lag_in, pop_out, lag_out, nullptr, f.psi, f.cosf, f.st64, f.C, f.chi, f.mu};
 }
 
 template <typename T>
@@ -532,6 +554,16 @@ int step_plain(ddcc_handle* h, int64_t n) {
             if ((st = prof_begin(h, 2))) return st;
             DDCC_CU(launch_sweep<T>(a, h->stream));
             if ((st = prof_end(h))) return st;
+        } else if constexpr (sizeof(T) == 8) {
+            const Step64Args a = args64(f, f.f[c], f.lag[c], f.f[1 - c], f.lag[1 - c]);
+            if ((st = prof_begin(h, 0))) return st;
+            DDCC_CU(launch_fields64(k, a, h->stream));
+            if ((st = prof_end(h))) return st;
+            if ((st = prof_begin(h, 1))) return st;
+            DDCC_CU(launch_update64(k, a, h->stream));
+            if ((st = prof_end(h))) return st;
+            if (h->prm.flags & DDCC_FLAG_OPEN_X)
+                DDCC_CU(launch_open_bc<T>(k, f.f[1 - c], f.lag[1 - c], f.psi, f.inflow, h->stream));
         } else if (h->use_tile_tma == 2) {
             TileTmaArgs<T> a{&h->tt_fh[c], &h->tt_g[c], &h->tt_lag[c], &h->tt_c, &h->tt_st, &h->tt_a[c], &k,
                              f.f[1 - c], f.lag[1 - c], f.flag, h->tile_wide};
@@ -612,7 +644,7 @@ void build_step_graph(ddcc_handle* h) {
 
 template <typename T>
 int step_t(ddcc_handle* h, int64_t n) {
-    if (h->profiling || h->use_sweep || h->use_tile_tma != 2 || n < 4) return step_plain<T>(h, n);
+    if (h->profiling || h->use_sweep || h->use_tile_tma < 2 || n < 4) return step_plain<T>(h, n);
     if (h->graph_state == 0) build_step_graph<T>(h);
     if (h->graph_state != 1) return step_plain<T>(h, n);
     int st;
@@ -665,7 +697,14 @@ int read_t(ddcc_handle* h, int field, double* out) {
         else if (field >= DDCC_FIELD_MU && field < DDCC_FIELD_MU + N) plane = N + 4 + field - DDCC_FIELD_MU;
         if (plane < 0) return DDCC_ERR_PARAM;
         if (!h->macro_valid) {
-            DDCC_CU(launch_macro<T>(k, f, h->cur, h->stream));
+            if constexpr (sizeof(T) == 8) {
+                Step64Args a = args64(f, f.f[h->cur], f.lag[h->cur], nullptr, nullptr);
+                a.macro = f.macro;
+                DDCC_CU(launch_fields64(k, a, h->stream));
+                DDCC_CU(launch_update64(k, a, h->stream));
+            } else {
+                DDCC_CU(launch_macro<T>(k, f, h->cur, h->stream));
+            }
             h->macro_valid = 1;
         }
         src = f.macro + (size_t)plane * k.plane;
@@ -768,7 +807,7 @@ int adjoint_initial_t(ddcc_handle* h, const double* C0, const void* adj0, void* 
 // (both in the saved-state layout), through tensor maps of those buffers.
 template <typename T>
 int step_between_t(ddcc_handle* h, const void* state_in, void* state_out) {
-    if (h->use_sweep || h->use_tile_tma != 2 || (h->prm.flags & DDCC_FLAG_OPEN_X)) return DDCC_ERR_UNSUPPORTED;
+    if (h->use_sweep || h->use_tile_tma < 2 || (h->prm.flags & DDCC_FLAG_OPEN_X)) return DDCC_ERR_UNSUPPORTED;
     KParams<T>& k = kp_of<T>(h);
     Fields<T>& f = fd_of<T>(h);
     const int N = h->prm.nphase;
@@ -778,12 +817,18 @@ int step_between_t(ddcc_handle* h, const void* state_in, void* state_out) {
     const T* in_lag = reinterpret_cast<const T*>(static_cast<const char*>(state_in) + kAlign + pb);
     T* out_pop = reinterpret_cast<T*>(static_cast<char*>(state_out) + kAlign);
     T* out_lag = reinterpret_cast<T*>(static_cast<char*>(state_out) + kAlign + pb);
-    FusedMaps m;
-    if (!encode_fused<T>(&m, in_pop, in_lag, k, h->tile_wide)) return DDCC_ERR_CUDA;
-    TileTmaArgs<T> a{&m.fh, &m.g, &m.lag, &h->tt_c, &h->tt_st, &m.a, &k, out_pop, out_lag, f.flag, h->tile_wide};
-    DDCC_CU(launch_collide_fused<T>(a, h->stream));
-    DDCC_CU(launch_fill_ghosts2<T>(GhostRing<T>{out_pop, 9 * (N - 1), kFusedGhostF, kFusedGhostF},
-                                   GhostRing<T>{out_lag, 1, kFusedGhostA, kFusedGhostA}, k, h->stream));
+    if constexpr (sizeof(T) == 8) {
+        const Step64Args a = args64(f, in_pop, in_lag, out_pop, out_lag);
+        DDCC_CU(launch_fields64(k, a, h->stream));
+        DDCC_CU(launch_update64(k, a, h->stream));
+    } else {
+        FusedMaps m;
+        if (!encode_fused<T>(&m, in_pop, in_lag, k, h->tile_wide)) return DDCC_ERR_CUDA;
+        TileTmaArgs<T> a{&m.fh, &m.g, &m.lag, &h->tt_c, &h->tt_st, &m.a, &k, out_pop, out_lag, f.flag, h->tile_wide};
+        DDCC_CU(launch_collide_fused<T>(a, h->stream));
+        DDCC_CU(launch_fill_ghosts2<T>(GhostRing<T>{out_pop, 9 * (N - 1), kFusedGhostF, kFusedGhostF},
+                                       GhostRing<T>{out_lag, 1, kFusedGhostA, kFusedGhostA}, k, h->stream));
+    }
     return DDCC_OK;
 }
 
@@ -1218,7 +1263,7 @@ int ddcc_adjoint_segment_pipelined(ddcc_handle* h, const void* const* states, in
         for (int s = 0; s < n; ++s)
             if (next[t] == states[s]) return DDCC_ERR_PARAM;
     }
-    if (n_next > 1 && (h->use_sweep || h->use_tile_tma != 2)) return DDCC_ERR_UNSUPPORTED;
+    if (n_next > 1 && (h->use_sweep || h->use_tile_tma < 2)) return DDCC_ERR_UNSUPPORTED;
     if (n_next > 1 && !h->side) {
         // all three or none
         cudaStream_t side = nullptr;

@@ -6,6 +6,7 @@
 //   accessor  C(j, dy, dx)  C_j (j < N-1) at the neighbour (x+dx, y+dy)
 //             psi(dy, dx)   the characteristic function psi
 //             mu(j, dy, dx) mu_j (j < N) of Eq. 2.14
+//             grad_psi(P, gx, gy)  grad psi at the node
 //             psi_rho(dy, dx)  psi rho
 //             a(dy, dx)     the lagged antisymmetric-flux field a
 //             lag(k)        lagged plane k at the node
@@ -103,16 +104,13 @@ __device__ __forceinline__ void grad9(const KParams<T>& P, const A& chi, T& gx, 
 // g'(1 - c) = -g'(c) and sum_j C_j = 1: they vanish for two phases, are
 // -g'(C_k) of the third for three, and for four three pairs give the other
 // three.  For two phases mu_2 = -mu_1.
+// agp3 = 3 |grad psi| (3 with several solids) and inv_p0 = 1 / psi at the node.
 template <typename T, int NP, class CA, class PA>
-__device__ __forceinline__ void chem_pot(const KParams<T>& P, const CA& Cx, const PA& Ps,
-                                         const T* cth, T mu[NP]) {
+__device__ __forceinline__ void chem_pot_with(const KParams<T>& P, const CA& Cx, const PA& Ps,
+                                              const T* cth, T agp3, T inv_p0, T mu[NP]) {
     const T p0 = Ps(0, 0);
     const T pE = Ps(0, 1), pW = Ps(0, -1), pN = Ps(1, 0), pS = Ps(-1, 0);
     const T pNE = Ps(1, 1), pNW = Ps(1, -1), pSW = Ps(-1, -1), pSE = Ps(-1, 1);
-    T gpx, gpy;
-    grad9(P, [&](int dy, int dx) { return Ps(dy, dx); }, gpx, gpy);
-    // with several solids the angle planes already carry |grad psi_k|
-    const T agp3 = T(3) * (P.wet_field ? T(1) : root(gpx * gpx + gpy * gpy));
     T Cv[NP], V[NP];
     T sumC = T(0), sumL = T(0);
 #pragma unroll
@@ -130,7 +128,6 @@ __device__ __forceinline__ void chem_pot(const KParams<T>& P, const CA& Cx, cons
     }
     Cv[NP - 1] = T(1) - sumC;
     V[NP - 1] = -sumL;
-    const T inv_p0 = rcp(p0);
     // a_j = sigma_jN cos(theta_jN) (zero for j = N, sigma_NN = 0), so that
     // cos(theta_jq) = (a_j - a_q) / sigma_jq, antisymmetric in (j, q)
     if constexpr (NP == 2) {
@@ -184,6 +181,16 @@ __device__ __forceinline__ void chem_pot(const KParams<T>& P, const CA& Cx, cons
             mu[i] = bulk + v * inv_p0;
         }
     }
+}
+
+template <typename T, int NP, class CA, class PA>
+__device__ __forceinline__ void chem_pot(const KParams<T>& P, const CA& Cx, const PA& Ps,
+                                         const T* cth, T mu[NP]) {
+    T gpx, gpy;
+    grad9(P, [&](int dy, int dx) { return Ps(dy, dx); }, gpx, gpy);
+    // with several solids the angle planes already carry |grad psi_k|
+    const T agp3 = T(3) * (P.wet_field ? T(1) : root(gpx * gpx + gpy * gpy));
+    chem_pot_with<T, NP>(P, Cx, Ps, cth, agp3, rcp(Ps(0, 0)), mu);
 }
 
 // Hermite moments m_ab = sum_p v_p h_a(cx_p) h_b(cy_p), h = (1, c, c^2 - cs2),
@@ -294,9 +301,9 @@ __device__ __forceinline__ T psi_rho(const KParams<T>& P, T psi, const CA& C) {
 // the capillary force through mu_j - mu_N, and m^C = -m0 sum_j
 // (rho_j - rho_N) Q_j because the Q_j add up to zero.  With the pair
 // identities of chem_pot, psi rho formed once per node and the reciprocals
-// above, the FP64 step (bound by its FP64 pipe) went from 629 to 511 us at
-// 512 x 512, N = 4, and from 51 to 40 us at 64 x 64, N = 2; in FP32, bound by
-// memory, these changes alone leave the time as it was.
+// above, the FP64 tile step (bound by its FP64 pipe) went from 629 to 511 us
+// at 512 x 512, N = 4, and from 51 to 40 us at 64 x 64, N = 2; in FP32, bound
+// by memory, these changes alone leave the time as it was.
 template <typename T, int NP, int MODE, class Acc, class Sink>
 __device__ __forceinline__ void node_update(const KParams<T>& P, const Acc& A, Sink& out) {
     const T cs2 = P.cs2;
@@ -324,7 +331,7 @@ __device__ __forceinline__ void node_update(const KParams<T>& P, const Acc& A, S
     const T s21 = rcp(inv_s21);
     const T s22 = rcp(nu * P.nu_to_s22 + T(0.5));
     T gpx, gpy;
-    grad9(P, [&](int dy, int dx) { return A.psi(dy, dx); }, gpx, gpy);
+    A.grad_psi(P, gpx, gpy);
     T gprx, gpry;
     grad9(P, [&](int dy, int dx) { return A.psi_rho(dy, dx); }, gprx, gpry);
 

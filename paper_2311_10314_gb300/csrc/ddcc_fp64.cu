@@ -20,6 +20,8 @@
 //    free beside the FP64 pipe), so no ghost frame is read; the one-node
 //    ghost ring of the lagged plane a, which the reverse step reads, is
 //    written along with the plane.
+// Against the one-kernel tile step with the same node arithmetic: 512 x 512,
+// N = 4, 511 -> 440 us a step; 64 x 64, N = 2, 40 -> 20 us.
 #include "ddcc_device.cuh"
 
 namespace ddcc {

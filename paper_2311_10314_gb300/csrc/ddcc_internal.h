@@ -81,6 +81,9 @@ struct Fields {
     T* cosf;          // N-1 planes or null
     T* C;             // N-1 planes (order-parameter scratch)
     T* macro;         // 2N+4 planes (read-out scratch)
+    T* mu;            // (FP64) N planes: chemical potentials of the current step
+    T* chi;           // (FP64) 1 plane: psi rho of the current step
+    T* st64;          // (FP64) static64_planes() planes of psi's own terms, formed at create
     double* partial;  // kMassBlocks * kMaxPhases
     double* stage;    // host-input staging (double), max(N-1,1) planes
     T* inflow;        // open x ends: u_in (ny values), then C_in ((N-1) x ny)
@@ -152,6 +155,20 @@ template <typename T>
 size_t tile_fused_smem_bytes(int N, bool theta_field, bool wide);
 template <typename T>
 cudaError_t launch_collide_fused(const TileTmaArgs<T>& a, cudaStream_t s);
+
+// The FP64 step (ddcc_fp64.cu): C, psi rho and mu to planes, then the node
+// update from them; macro non-null: the read-out of the current state instead
+// of the update.
+struct Step64Args {
+    const double *pop_in, *lag_in;
+    double *pop_out, *lag_out, *macro;
+    const double *psi, *cosf, *st;
+    double *C, *chi, *mu;
+};
+int static64_planes();
+cudaError_t launch_static64(const KParams<double>& kp, const double* psi, double* st, cudaStream_t s);
+cudaError_t launch_fields64(const KParams<double>& kp, const Step64Args& a, cudaStream_t s);
+cudaError_t launch_update64(const KParams<double>& kp, const Step64Args& a, cudaStream_t s);
 
 template <typename T>
 size_t sweep_smem_bytes(int N, bool theta_field);

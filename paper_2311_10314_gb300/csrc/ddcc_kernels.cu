@@ -8,6 +8,7 @@
 //                  memory, mu_i (Eq. 2.14) is evaluated on the tile plus a
 //                  1-node halo, then every node runs dev::node_update and
 //                  pushes its post-collision populations to its neighbours.
+// These run the FP32 step; ddcc_fp64.cu has the FP64 one.
 // k_step_tma is the same tile step with every input staged by TMA tensor
 // copies (halo boxes of C, psi, cos(theta) and a first, then the tile's
 // populations and lagged planes, which land while mu is evaluated); it is
@@ -98,6 +99,9 @@ struct TileAcc {
     const T* __restrict__ gin;
     __device__ T C(int j, int dy, int dx) const { return sm.C[j][cy + dy][cx + dx]; }
     __device__ T psi(int dy, int dx) const { return sm.psi[cy + dy][cx + dx]; }
+    __device__ void grad_psi(const KParams<T>& Q, T& gx, T& gy) const {
+        dev::grad9(Q, [&](int dy, int dx) { return psi(dy, dx); }, gx, gy);
+    }
     __device__ T psi_rho(int dy, int dx) const {
         return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
     }
@@ -249,6 +253,9 @@ struct TmaAcc {
         return sm[L::c_off + ((size_t)j * (BY + 4) + ty + 2 + dy) * L::HX + tx + 4 + dx];
     }
     __device__ T psi(int dy, int dx) const { return sm[L::st_off + (size_t)(ty + 2 + dy) * L::HX + tx + 4 + dx]; }
+    __device__ void grad_psi(const KParams<T>& Q, T& gx, T& gy) const {
+        dev::grad9(Q, [&](int dy, int dx) { return psi(dy, dx); }, gx, gy);
+    }
     __device__ T psi_rho(int dy, int dx) const {
         return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
     }
@@ -261,10 +268,9 @@ struct TmaAcc {
     __device__ T g(int p) const { return sm[L::pop_off + ((size_t)(9 * (NP - 1) + p) * BY + ty) * BX + tx]; }
 };
 
-// Two CTAs per SM in FP32 (128 registers, ~69 KB of shared memory each);
-// FP64 tiles need twice the shared memory, so one.
+// Two CTAs per SM (128 registers, ~69 KB of shared memory each).
 template <typename T, int NP, bool TF>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(NT, 2)
     k_step_tma(const __grid_constant__ CUtensorMap tm_pop, const __grid_constant__ CUtensorMap tm_lag,
                const __grid_constant__ CUtensorMap tm_c, const __grid_constant__ CUtensorMap tm_st,
                const __grid_constant__ CUtensorMap tm_a, KParams<T> P, T* __restrict__ pop_out,
@@ -381,7 +387,7 @@ struct FLay {
     static constexpr int LAG_BOX = NLAG * TY * TX;
     static constexpr int ST_BOX = NST * HY * HX;
     static constexpr int A_BOX = (TY + 2) * HX;
-    static constexpr int C_ARR = (sizeof(T) == 8 ? NP : NP - 1) * HY * HX;   // C_i, and in FP64 psi rho
+    static constexpr int C_ARR = (NP - 1) * HY * HX;
     static constexpr int MU = NP * (TY + 2) * (TX + 2);
     static constexpr size_t fh_off = 0;
     static constexpr size_t g_off = fh_off + pad(FH_BOX);
@@ -407,9 +413,11 @@ struct FusedAcc {
         return sm[L::c_off + ((size_t)j * L::HY + ty + 2 + dy) * L::HX + tx + 4 + dx];
     }
     __device__ T psi(int dy, int dx) const { return sm[L::st_off + (size_t)(ty + 2 + dy) * L::HX + tx + 4 + dx]; }
+    __device__ void grad_psi(const KParams<T>& Q, T& gx, T& gy) const {
+        dev::grad9(Q, [&](int dy, int dx) { return psi(dy, dx); }, gx, gy);
+    }
     __device__ T psi_rho(int dy, int dx) const {
-        if constexpr (sizeof(T) == 8) return C(NP - 1, dy, dx);
-        else return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
+        return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
     }
     __device__ T mu(int j, int dy, int dx) const {
         return sm[L::mu_off + ((size_t)j * (TY + 2) + ty + 1 + dy) * (TX + 2) + tx + 1 + dx];
@@ -423,7 +431,7 @@ struct FusedAcc {
 };
 
 template <typename T, int NP, bool TF, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(TX * TY, 2)
     k_step_fused(const __grid_constant__ CUtensorMap tm_fh, const __grid_constant__ CUtensorMap tm_g,
                  const __grid_constant__ CUtensorMap tm_lag, const __grid_constant__ CUtensorMap tm_st,
                  const __grid_constant__ CUtensorMap tm_a, KParams<T> P, T* __restrict__ pop_out,
@@ -473,52 +481,31 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? 2 : 1)
         }
         return;
     }
-    // C_i = sum_p f^i_p / psi on the tile + 2-node halo.  FP32: four columns
-    // of one phase per item as 16-byte accesses over whole box rows (40
-    // columns), so a warp reads consecutive quads: node by node over the 36
-    // columns needed, every warp spanned two rows and met two-way bank
-    // conflicts (256 x 256, N = 3: 11.0 -> 10.3 us a step).  FP64 (bound by its FP64 pipe): only the 12 x 36 nodes
-    // needed, and psi rho, which the update differentiates, once per node
-    // here instead of once per neighbour there.
-    if constexpr (sizeof(T) == 4) {
-        constexpr int NQ = L::HY * L::HX / 4, PL = L::HY * L::HX;
+    // C_i = sum_p f^i_p / psi on the tile + 2-node halo: four columns of one
+    // phase per item as 16-byte accesses over whole box rows, so a warp reads
+    // consecutive quads (node by node over the columns needed, every warp
+    // spanned two rows and met two-way bank conflicts: 256 x 256, N = 3, 11.0
+    // -> 10.3 us a step).
+    constexpr int NQ = L::HY * L::HX / 4, PL = L::HY * L::HX;
 #pragma unroll
-        for (int r = 0; r < ((NP - 1) * NQ + (TX * TY) - 1) / (TX * TY); ++r) {
-            const int k = tid + r * (TX * TY);
-            if (k < (NP - 1) * NQ) {
-                const int i = k / NQ, o = 4 * (k - i * NQ);
-                const T* fb = sm + L::fh_off + (size_t)(9 * i) * PL + o;
-                float4 c = *reinterpret_cast<const float4*>(fb);
+    for (int r = 0; r < ((NP - 1) * NQ + (TX * TY) - 1) / (TX * TY); ++r) {
+        const int k = tid + r * (TX * TY);
+        if (k < (NP - 1) * NQ) {
+            const int i = k / NQ, o = 4 * (k - i * NQ);
+            const T* fb = sm + L::fh_off + (size_t)(9 * i) * PL + o;
+            float4 c = *reinterpret_cast<const float4*>(fb);
 #pragma unroll
-                for (int p = 1; p < 9; ++p) {
-                    const float4 v = *reinterpret_cast<const float4*>(fb + (size_t)p * PL);
-                    c.x += v.x;
-                    c.y += v.y;
-                    c.z += v.z;
-                    c.w += v.w;
-                }
-                const float4 ps = *reinterpret_cast<const float4*>(sm + L::st_off + o);
-                *reinterpret_cast<float4*>(sm + L::c_off + (size_t)i * PL + o) =
-                    make_float4(c.x * dev::rcp(ps.x), c.y * dev::rcp(ps.y), c.z * dev::rcp(ps.z),
-                                c.w * dev::rcp(ps.w));
+            for (int p = 1; p < 9; ++p) {
+                const float4 v = *reinterpret_cast<const float4*>(fb + (size_t)p * PL);
+                c.x += v.x;
+                c.y += v.y;
+                c.z += v.z;
+                c.w += v.w;
             }
-        }
-    } else {
-        for (int k = tid; k < L::HY * (TX + 4); k += (TX * TY)) {
-            const int cy = k / (TX + 4), cx = k - cy * (TX + 4) + 2;   // box column of node x0-2+..
-            const T psi = sm[L::st_off + (size_t)cy * L::HX + cx];
-            const T inv = dev::rcp(psi);
-            const T* fb = sm + L::fh_off + (size_t)cy * L::HX + cx;
-            T* cb = sm + L::c_off + (size_t)cy * L::HX + cx;
-            T Cv[NP - 1];
-#pragma unroll
-            for (int i = 0; i < NP - 1; ++i) {
-                T s = fb[(size_t)(9 * i) * L::HY * L::HX];
-#pragma unroll
-                for (int p = 1; p < 9; ++p) s += fb[(size_t)(9 * i + p) * L::HY * L::HX];
-                cb[(size_t)i * L::HY * L::HX] = Cv[i] = s * inv;
-            }
-            cb[(size_t)(NP - 1) * L::HY * L::HX] = dev::psi_rho<T, NP>(P, psi, [&](int j) { return Cv[j]; });
+            const float4 ps = *reinterpret_cast<const float4*>(sm + L::st_off + o);
+            *reinterpret_cast<float4*>(sm + L::c_off + (size_t)i * PL + o) =
+                make_float4(c.x * dev::rcp(ps.x), c.y * dev::rcp(ps.y), c.z * dev::rcp(ps.z),
+                            c.w * dev::rcp(ps.w));
         }
     }
     __syncthreads();
@@ -593,8 +580,8 @@ cudaError_t collide_fused_n(const TileTmaArgs<T>& a, cudaStream_t s) {
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         sms = 0;   // no prefetch
-    // a wave of resident CTAs (two per SM in FP32, one in FP64) ahead
-    const int pf_dist = kPrefetchQuarterWaves * sms * (sizeof(T) == 4 ? 2 : 1) / 4;
+    // a wave of resident CTAs (two per SM) ahead
+    const int pf_dist = kPrefetchQuarterWaves * sms * 2 / 4;
     // the inner tiles' 32-bit offsets reach every population and lagged plane
     const int off32 = (long long)(9 * NP) * kp.plane < (1LL << 31) ? 1 : 0;
     k_step_fused<T, NP, TF, TX, TY><<<dim3((kp.nx + TX - 1) / TX, (kp.ny + TY - 1) / TY), dim3(TX, TY), L::bytes, s>>>(
@@ -957,7 +944,7 @@ size_t tile_tma_smem_bytes(int N, bool tf) {
         default: return 0;
     }
 }
-// The fused kernel's tile: 32 x 8, or in FP32 64 x 4 (see fused_tile_wide).
+// The fused kernel's tile: 32 x 8 or 64 x 4 (see fused_tile_wide).
 template <typename T, int TX, int TY>
 size_t fused_smem_shape(int N, bool tf) {
     switch (N * 2 + (tf ? 1 : 0)) {
@@ -972,10 +959,7 @@ size_t fused_smem_shape(int N, bool tf) {
 }
 template <typename T>
 size_t tile_fused_smem_bytes(int N, bool tf, bool wide) {
-    if constexpr (sizeof(T) == 4) {
-        if (wide) return fused_smem_shape<T, kWideX, kWideY>(N, tf);
-    }
-    return fused_smem_shape<T, BX, BY>(N, tf);
+    return wide ? fused_smem_shape<T, kWideX, kWideY>(N, tf) : fused_smem_shape<T, BX, BY>(N, tf);
 }
 template <typename T, int TX, int TY>
 cudaError_t fused_shape(const TileTmaArgs<T>& a, cudaStream_t s) {
@@ -992,10 +976,7 @@ cudaError_t fused_shape(const TileTmaArgs<T>& a, cudaStream_t s) {
 }
 template <typename T>
 cudaError_t launch_collide_fused(const TileTmaArgs<T>& a, cudaStream_t s) {
-    if constexpr (sizeof(T) == 4) {
-        if (a.wide) return fused_shape<T, kWideX, kWideY>(a, s);
-    }
-    return fused_shape<T, BX, BY>(a, s);
+    return a.wide ? fused_shape<T, kWideX, kWideY>(a, s) : fused_shape<T, BX, BY>(a, s);
 }
 template <typename T>
 cudaError_t launch_collide_tma(const TileTmaArgs<T>& a, cudaStream_t s) {
@@ -1068,26 +1049,27 @@ cudaError_t launch_wall_accumulate(const KParams<T>& kp, const T* stage, T* psi,
 
 #define DDCC_INSTANTIATE(T)                                                                      \
     template cudaError_t launch_init<T>(const KParams<T>&, const Fields<T>&, int, cudaStream_t);  \
-    template cudaError_t launch_order_param<T>(const KParams<T>&, const Fields<T>&, int,          \
-                                               cudaStream_t);                                    \
-    template cudaError_t launch_collide<T>(const KParams<T>&, const Fields<T>&, int, cudaStream_t); \
-    template cudaError_t launch_macro<T>(const KParams<T>&, const Fields<T>&, int, cudaStream_t); \
     template cudaError_t launch_mass<T>(const KParams<T>&, const Fields<T>&, int, double*,        \
                                         cudaStream_t);                                           \
     template cudaError_t launch_convert<T>(const double*, T*, const KParams<T>&, int, cudaStream_t); \
     template cudaError_t launch_export<T>(const T*, double*, const KParams<T>&, cudaStream_t);    \
     template cudaError_t launch_fill_ghosts<T>(T*, int, const KParams<T>&, cudaStream_t, int, int);         \
-    template cudaError_t launch_fill_ghosts2<T>(const GhostRing<T>&, const GhostRing<T>&, const KParams<T>&,    \
-                                                cudaStream_t);                                            \
-    template size_t tile_tma_smem_bytes<T>(int, bool);                                           \
-    template size_t tile_fused_smem_bytes<T>(int, bool, bool);                                   \
     template cudaError_t launch_walls_init<T>(const KParams<T>&, T*, T*, cudaStream_t);          \
     template cudaError_t launch_open_bc<T>(const KParams<T>&, T*, T*, const T*, const T*, cudaStream_t); \
-    template cudaError_t launch_wall_accumulate<T>(const KParams<T>&, const T*, T*, T*, cudaStream_t); \
-    template cudaError_t launch_collide_fused<T>(const TileTmaArgs<T>&, cudaStream_t);           \
-    template cudaError_t launch_collide_tma<T>(const TileTmaArgs<T>&, cudaStream_t);
+    template cudaError_t launch_wall_accumulate<T>(const KParams<T>&, const T*, T*, T*, cudaStream_t);
 
 DDCC_INSTANTIATE(double)
 DDCC_INSTANTIATE(float)
+
+// the tile step and its read-out run in FP32; FP64 has its own (ddcc_fp64.cu)
+template cudaError_t launch_order_param<float>(const KParams<float>&, const Fields<float>&, int, cudaStream_t);
+template cudaError_t launch_collide<float>(const KParams<float>&, const Fields<float>&, int, cudaStream_t);
+template cudaError_t launch_macro<float>(const KParams<float>&, const Fields<float>&, int, cudaStream_t);
+template cudaError_t launch_fill_ghosts2<float>(const GhostRing<float>&, const GhostRing<float>&, const KParams<float>&,
+                                                cudaStream_t);
+template size_t tile_tma_smem_bytes<float>(int, bool);
+template size_t tile_fused_smem_bytes<float>(int, bool, bool);
+template cudaError_t launch_collide_fused<float>(const TileTmaArgs<float>&, cudaStream_t);
+template cudaError_t launch_collide_tma<float>(const TileTmaArgs<float>&, cudaStream_t);
 
 }  // namespace ddcc

@@ -127,6 +127,9 @@ struct SweepAcc {
     const T* M_r[3];
     __device__ T C(int j, int dy, int dx) const { return C_r[dy + 1][j * L::CW + 2 + dx]; }
     __device__ T psi(int dy, int dx) const { return st_r[dy + 1][4 + dx]; }
+    __device__ void grad_psi(const KParams<T>& Q, T& gx, T& gy) const {
+        dev::grad9(Q, [&](int dy, int dx) { return psi(dy, dx); }, gx, gy);
+    }
     __device__ T psi_rho(int dy, int dx) const {
         return dev::psi_rho<T, NP>(P, psi(dy, dx), [&](int j) { return C(j, dy, dx); });
     }

@@ -50,3 +50,29 @@ def test_fp32_wide_tiles(D, nx, ny, N, py, field):
     assert nx * ny * (11 * N + 3) * 4 > 64 << 20
     pb = W.random_problem(nx, ny, N, seed=nx + N, periodic_y=py, theta_field=field, width=6.0, n_circles=12, n_drops=9)
     _against_oracle(D, pb, D.DDCC_FP32, 3)
+
+
+@pytest.mark.parametrize("nx,ny,N,py,field", [
+    (3, 3, 2, 1, True),          # the smallest grid
+    (31, 5, 3, 0, True),         # under one block of either kernel
+    (33, 4, 4, 1, False),        # one column over a block
+    (64, 8, 2, 0, False),        # whole blocks
+    (65, 13, 3, 1, True),        # node numbering that straddles rows
+    (161, 97, 4, 0, True),
+])
+def test_fp64_step_and_ghost_ring(D, nx, ny, N, py, field):
+    """The FP64 pair of kernels, stepped plainly and replayed (9 steps), and
+    the one-node ghost ring of the lagged plane a in the saved state, which
+    the reverse step reads."""
+    from paper_2311_10314_gb300 import _lib
+    pb = W.random_problem(nx, ny, N, seed=nx + ny, periodic_y=py, theta_field=field, width=6.0)
+    _against_oracle(D, pb, D.DDCC_FP64, 9)
+    sim = D.Sim(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field, precision=D.DDCC_FP64)
+    sim.step(9)
+    state = sim.save_state()
+    sim.close()
+    org, pitch, plane = _lib.state_layout(nx, ny, N, 8)
+    a = torch.as_strided(state.view(torch.float64), (ny + 2, nx + 2), (pitch, 1),
+                         org + 9 * N * plane - pitch - 1).cpu().numpy()
+    wrap = np.pad(a[1:-1, 1:-1], ((0, 0), (1, 1)), mode="wrap")
+    assert np.array_equal(a, np.pad(wrap, ((1, 1), (0, 0)), mode="wrap" if py else "symmetric"))
