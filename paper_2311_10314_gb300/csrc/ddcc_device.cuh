@@ -73,6 +73,8 @@ __device__ __forceinline__ double root(double x) {
 // max(x, 0), and x with the sign of s, without the FP64 pipe
 __device__ __forceinline__ float clamp0(float x) { return fmaxf(x, 0.0f); }
 __device__ __forceinline__ double clamp0(double x) { return __double2hiint(x) < 0 ? 0.0 : x; }
+__device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool positive(double x) { return __double2hiint(x) > 0; }   // (subnormals count as zero)
 __device__ __forceinline__ float signed_as(float x, float s) { return copysignf(x, s); }
 __device__ __forceinline__ double signed_as(double x, double s) {
     return __hiloint2double((__double2hiint(s) & 0x80000000) | (__double2hiint(x) & 0x7fffffff),
