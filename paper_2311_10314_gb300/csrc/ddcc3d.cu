@@ -1,7 +1,8 @@
 // Three-dimensional DD-CCLB stepper (C ABI in include/ddcc3d.h): phase
 // populations on D3Q7, flow populations on D3Q15 (Sec. 3), periodic box.
 //
-// One step is three kernels over a 32 x 4 x 2 thread block per 256 nodes:
+// One step is three kernels with one thread per node, or in FP32 by default
+// one fused kernel (below):
 //   k3_order   C_i = sum_p f^i_p / psi                      (Sec. 3)
 //   k3_mu      mu_i of Eq. 2.14 from C and psi on the 15-point stencil
 //   k3_update  gradients (D3Q15-weighted isotropic stencils), mobility
@@ -26,8 +27,15 @@
 #include <cuda_runtime.h>
 
 #include "ddcc3d.h"
+#include "ddcc_device.cuh"
 
 namespace {
+
+using ddcc::dev::add_rn;
+using ddcc::dev::clamp0;
+using ddcc::dev::rcp;
+using ddcc::dev::root;
+using ddcc::dev::signed_as;
 
 constexpr int kMaxN = DDCC_MAX_PHASES;
 constexpr int kBX = 32, kBY = 4, kBZ = 2;
@@ -43,7 +51,6 @@ constexpr int kFusedTY = 8;          // rows of the fused step's column
 __host__ __device__ constexpr int cx(int p) { return p == 1 ? 1 : p == 2 ? -1 : p >= 7 ? (((p - 7) & 1) ? -1 : 1) : 0; }
 __host__ __device__ constexpr int cy(int p) { return p == 3 ? 1 : p == 4 ? -1 : p >= 7 ? (((p - 7) & 2) ? -1 : 1) : 0; }
 __host__ __device__ constexpr int cz(int p) { return p == 5 ? 1 : p == 6 ? -1 : p >= 7 ? (((p - 7) & 4) ? -1 : 1) : 0; }
-__host__ __device__ constexpr int cc(int p, int a) { return a == 0 ? cx(p) : a == 1 ? cy(p) : cz(p); }
 // the seven pairs of opposite velocities: p = pair_rep(q), c_pair_opp(q) = -c_p
 __host__ __device__ constexpr int pair_rep(int q) { return q < 3 ? 2 * q + 1 : 7 + (q - 3); }
 __host__ __device__ constexpr int pair_opp(int q) { return q < 3 ? 2 * q + 2 : 14 - (q - 3); }
@@ -56,25 +63,30 @@ struct P3 {
     int has_cos_field;
     T cs2, inv_cs2;
     T ga, gc;                  // w_axis / cs2, w_corner / cs2 (D3Q15 weights)
+    T la, lc;                  // (3 eps / 4) times ga, gc
     T w7_0, w7_1;              // D3Q7 weights
     T w15[3];                  // D3Q15 weights: rest, axis, corner
     T rho[kMaxN], nu[kMaxN];
+    T drho[kMaxN], dnu[kMaxN]; // rho_j - rho_N, nu_j - nu_N
     T beta2[kMaxN][kMaxN];     // 2 beta_ij = 6 sigma_ij / eps
-    T kap[kMaxN][kMaxN];       // 3 eps sigma_ij / 4
-    T wet[kMaxN][kMaxN];       // 3 sigma_ij
+    T beta2s[kMaxN];           // sum_{j != i} 2 beta_ij
+    T sig[kMaxN][kMaxN];       // sigma_ij
     T sigN[kMaxN];             // sigma_iN
     T invsig[kMaxN][kMaxN];
     T cos_uni[kMaxN];
-    T eta[kMaxN];
-    T m0, inv_m0;
-    T s0f, s21f, s1f[kMaxN];   // D3Q7 rates
+    T eta[kMaxN], ceta[kMaxN]; // eta_i, cs2 eta_i
+    T m0;
+    T hs21f;                   // D3Q7 s21 / 2
+    T h1f[kMaxN], h2f[kMaxN];  // s1 / 2 and s1 / 4 - 1 / 2 (odd part of the D3Q7 collision)
     T lg0, lg1, lg3, lg3c, lg4; // D3Q15 constant rates over the row norms
+    T cg0, cg1;                // lg0 / 2 - 1 and lg1 / 2 - 1 / cs2
     T inv_n2d, inv_n2o;        // 1 / norm of the s21 and s22 rows
     T nu_to_s21, inv_cs2_nu;   // 2 / (1 - cs2), 1 / cs2 (Eq. 16)
     T damp;                    // 1 / eps0^3
     T K, Hfac;                 // K = 1 - 2 d0; H = Hfac (s21 - 2)
     T A_P, cP, kk, c2m3;       // Eq. 19 coefficients; 1 - 3 cs2
-    T diag_den, off_den;       // 1 / (cs2 (1 - cs2)), 1 / cs2^2
+    T half_K, two_cs2, one_m;  // K / 2, 2 cs2, 1 - cs2
+    T q0, qa, qc;              // the last D3Q15 row at rest, axis and corner velocities
     T body[3];
 };
 
@@ -87,10 +99,15 @@ struct F3 {
     T* cosf;        // N-1 planes or null
     T* C;           // N-1 planes
     T* mu;          // N planes
+    T* chi;         // (FP64) 1 plane: psi rho of the current step
+    T* st;          // (FP64) kStatic planes of psi's own terms, formed at create
     double* stage;  // 1 double plane (host staging, read-out)
     double* partial;
     int* flag;
 };
+
+// (FP64) planes of what depends on psi alone: 1 / psi, grad psi, 3 |grad psi|
+enum { kInvPsi, kGrad, kAgp3 = kGrad + 3, kStatic };
 
 // lagged plane indices
 __host__ __device__ constexpr int lag_a(int k) { return k; }                   // xy, yz, zx
@@ -107,12 +124,26 @@ struct Site {
     __device__ long long self() const { return zo[1] + yo[1] + xo[1]; }
 };
 
+// Node of this thread.  FP32: blocks of 32 x 4 x 2 nodes.  FP64 (bound by FP64
+// warp instructions, 64 cycles each per SM sub-partition, also for a warp
+// that is half empty): nodes numbered row by row, one per thread of kLinear-
+// thread blocks, so that no lane goes to padding and the last wave is short.
+constexpr int kLinear = 64;
 template <typename T>
 __device__ __forceinline__ bool site(const P3<T>& P, Site& s) {
-    s.x = blockIdx.x * kBX + threadIdx.x;
-    s.y = blockIdx.y * kBY + threadIdx.y;
-    s.z = blockIdx.z * kBZ + threadIdx.z;
-    if (s.x >= P.nx || s.y >= P.ny || s.z >= P.nz) return false;
+    if constexpr (sizeof(T) == 8) {
+        const unsigned i = blockIdx.x * (unsigned)kLinear + threadIdx.x, nxy = (unsigned)P.nxy;
+        if (i >= nxy * (unsigned)P.nz) return false;
+        s.z = (int)(i / nxy);
+        const unsigned r = i - (unsigned)s.z * nxy;
+        s.y = (int)(r / (unsigned)P.nx);
+        s.x = (int)(r - (unsigned)s.y * (unsigned)P.nx);
+    } else {
+        s.x = blockIdx.x * kBX + threadIdx.x;
+        s.y = blockIdx.y * kBY + threadIdx.y;
+        s.z = blockIdx.z * kBZ + threadIdx.z;
+        if (s.x >= P.nx || s.y >= P.ny || s.z >= P.nz) return false;
+    }
     s.xo[0] = s.x == 0 ? P.nx - 1 : s.x - 1;
     s.xo[1] = s.x;
     s.xo[2] = s.x == P.nx - 1 ? 0 : s.x + 1;
@@ -124,124 +155,181 @@ __device__ __forceinline__ bool site(const P3<T>& P, Site& s) {
     s.zo[2] = (long long)(s.z == P.nz - 1 ? 0 : s.z + 1) * P.nxy;
     return true;
 }
+template <typename T>
+__host__ __device__ constexpr int node_threads() { return sizeof(T) == 8 ? kLinear : kThreads; }
 
 // Ping-pong buffer c of a pair without a dynamically indexed parameter array
 // (which would be copied to local memory).
 template <typename X>
 __device__ __forceinline__ X* pick(X* const (&a)[2], int c) { return c ? a[1] : a[0]; }
 
-// Rounded to nearest and never fused or reassociated by the compiler.
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
-
-template <typename T>
-__device__ __forceinline__ T gprime(T C) {
-    const T Cm = C - T(1);
-    return T(2) * C * Cm * Cm + T(2) * C * C * Cm;
+// psi rho, rho = rho_N + sum_j (rho_j - rho_N) C_j
+template <typename T, int NP, class CA>
+__device__ __forceinline__ T psi_rho(const P3<T>& P, T psi, const CA& C) {
+    T r = P.rho[NP];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) r += P.drho[j] * C(j);
+    return psi * r;
 }
 
 // ---------------------------------------------------------------------------
 // volume fractions
 // ---------------------------------------------------------------------------
 template <typename T, int NP>
-__global__ void __launch_bounds__(kThreads) k3_order(P3<T> P, F3<T> F, int cur) {
+__global__ void __launch_bounds__(node_threads<T>()) k3_order(P3<T> P, F3<T> F, int cur) {
     Site s;
     if (!site(P, s)) return;
     const long long i0 = s.self();
-    const T psi = F.psi[i0];
     const T* f = pick(F.f, cur);
+    const T inv = sizeof(T) == 8 ? F.st[kInvPsi * P.plane + i0] : rcp(F.psi[i0]);
+    T C[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-        T acc = T(0);
+        T acc = f[7 * i * P.plane + i0];
 #pragma unroll
-        for (int p = 0; p < 7; ++p) acc += f[(7 * i + p) * P.plane + i0];
-        F.C[i * P.plane + i0] = acc / psi;
+        for (int p = 1; p < 7; ++p) acc += f[(7 * i + p) * P.plane + i0];
+        F.C[i * P.plane + i0] = C[i] = acc * inv;
     }
+    if constexpr (sizeof(T) == 8) F.chi[i0] = psi_rho<T, NP>(P, F.psi[i0], [&](int j) { return C[j]; });
 }
 
 // ---------------------------------------------------------------------------
 // chemical potentials, Eq. 2.14 (beta_ij = 3 sigma_ij / eps)
 // ---------------------------------------------------------------------------
-// mu_i of one node from its stencil sums: L_j = div(psi grad C_j) and
-// grad psi, with the angles cos(theta_jN) (cN[N-1] = 0).
-template <typename T, int NP>
-__device__ __forceinline__ void mu_from_stencil(const P3<T>& P, T psi, const T C[NP + 1], const T L[NP + 1],
-                                                T gpx, T gpy, T gpz, const T cN[NP + 1], T mu[NP + 1]) {
-    constexpr int N = NP + 1;
-    const T agp = sqrt(gpx * gpx + gpy * gpy + gpz * gpz);
-    T wetj[N];    // sum_{q != j} cos(theta_jq) C_j C_q, cos(theta_jq) by Eq. 2.9 (sigma_NN = 0)
+// sum_p w_p c_p v(p) / cs2 on the 15-point stencil (p = 1..14), from the
+// pairs of opposite neighbours: an axis pair gives its difference to its
+// own component; the corner pairs (7, 14), (8, 13), (9, 12), (10, 11) give
+// their differences d, signed by the first member's velocity.
+template <typename T, class V>
+__device__ __forceinline__ void grad15(const P3<T>& P, const V& v, T g[3]) {
+    const T d0 = v(7) - v(14), d1 = v(8) - v(13), d2 = v(9) - v(12), d3 = v(10) - v(11);
+    const T s01 = d0 + d1, s23 = d2 + d3;
+    g[0] = P.ga * (v(1) - v(2)) + P.gc * ((d0 - d1) + (d2 - d3));
+    g[1] = P.ga * (v(3) - v(4)) + P.gc * (s01 - s23);
+    g[2] = P.ga * (v(5) - v(6)) + P.gc * (s01 + s23);
+}
+
+// One pair of opposite neighbours (difference d, first member p) added to a
+// gradient, corner pairs before axis pairs: the corners' signed sums take
+// their weight with the first axis pair of the component.  FP32 goes through
+// the pairs once for all its fields (loads of different fields between the
+// arithmetic of others), FP64 field by field (grad15, fewer operations).
+template <typename T>
+__device__ __forceinline__ void add_pair(const P3<T>& P, int q, T d, T g[3]) {
+    const int p = pair_rep(q);
+    if (q >= 3) {
+        const int sg[3] = {cx(p), cy(p), cz(p)};
 #pragma unroll
-    for (int j = 0; j < N; ++j) {
-        T acc = T(0);
-#pragma unroll
-        for (int q = 0; q < N; ++q)
-            if (q != j) acc += (P.sigN[j] * cN[j] - P.sigN[q] * cN[q]) * P.invsig[j][q] * C[j] * C[q];
-        wetj[j] = acc;
-    }
-    const T inv_psi = T(1) / psi;
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        const T gi = gprime(C[i]);
-        T acc = T(0);
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            if (j == i) continue;
-            acc += P.beta2[i][j] * psi * (gi - gprime(C[i] + C[j]));
-            acc += P.kap[i][j] * L[j];
-            acc += P.wet[i][j] * wetj[j] * agp;
-        }
-        mu[i] = acc * inv_psi;
+        for (int a = 0; a < 3; ++a) g[a] = q == 3 ? d : sg[a] > 0 ? g[a] + d : g[a] - d;
+    } else {
+        g[q] = P.ga * d + P.gc * g[q];
     }
 }
 
+// (3 eps / 4) div(psi grad C) = sum_p l_p (psi + psi_p)(C_p - C): the axis and
+// the corner neighbours are summed first and take their weight once
+template <typename T, class PV, class CV>
+__device__ __forceinline__ T lap15(const P3<T>& P, const PV& psum, const CV& C, T c0) {
+    T a = psum(1) * (C(1) - c0), c = psum(7) * (C(7) - c0);
+#pragma unroll
+    for (int p = 2; p < 7; ++p) a += psum(p) * (C(p) - c0);
+#pragma unroll
+    for (int p = 8; p < 15; ++p) c += psum(p) * (C(p) - c0);
+    return P.la * a + P.lc * c;
+}
+
+// mu of one node from the 15-point neighbourhood: psi(p) and C(j, p), p = 0 the
+// node; grad psi is returned in gp.
+template <typename T, int NP, class PV, class CV>
+__device__ __forceinline__ void mu_node(const P3<T>& P, const PV& psi, const CV& C, const T* cth, T mu[NP + 1], T gp[3]) {
+    const T p0 = psi(0);
+    T c0[NP], L[NP];
+    if constexpr (sizeof(T) == 8) {
+        T ps[15];
+#pragma unroll
+        for (int p = 1; p < 15; ++p) ps[p] = psi(p);
+        grad15(P, [&](int p) { return ps[p]; }, gp);
+#pragma unroll
+        for (int p = 1; p < 15; ++p) ps[p] += p0;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            c0[j] = C(j, 0);
+            L[j] = lap15(P, [&](int p) { return ps[p]; }, [&](int p) { return C(j, p); }, c0[j]);
+        }
+    } else {
+        T La[NP][2], Lc[NP][2];   // axis and corner sums, one per member of a pair
+#pragma unroll
+        for (int j = 0; j < NP; ++j) c0[j] = C(j, 0);
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+            const int q = k < 4 ? k + 3 : k - 4, p = pair_rep(q), o = pair_opp(q);
+            const T a = psi(p), b = psi(o);
+            add_pair(P, q, a - b, gp);
+            const T ta = p0 + a, tb = p0 + b;
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                const T da = ta * (C(j, p) - c0[j]), db = tb * (C(j, o) - c0[j]);
+                T* S = q >= 3 ? Lc[j] : La[j];
+                const bool first = q == 3 || q == 0;
+                S[0] = first ? da : S[0] + da;
+                S[1] = first ? db : S[1] + db;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NP; ++j) L[j] = P.la * (La[j][0] + La[j][1]) + P.lc * (Lc[j][0] + Lc[j][1]);
+    }
+    const T agp3 = T(3) * root(gp[0] * gp[0] + gp[1] * gp[1] + gp[2] * gp[2]);
+    ddcc::dev::mu_of<T, NP + 1>(P, c0, L, cth, agp3, rcp(p0), mu);
+}
+
 template <typename T, int NP>
-__global__ void __launch_bounds__(kThreads) k3_mu(P3<T> P, F3<T> F) {
-    constexpr int N = NP + 1;
+__device__ __forceinline__ void angles(const P3<T>& P, const F3<T>& F, long long i, T cth[NP]) {
+#pragma unroll
+    for (int j = 0; j < NP; ++j) cth[j] = P.has_cos_field ? F.cosf[j * P.plane + i] : P.cos_uni[j];
+}
+
+template <typename T, int NP>
+__global__ void __launch_bounds__(node_threads<T>()) k3_mu(P3<T> P, F3<T> F) {
     Site s;
     if (!site(P, s)) return;
     const long long i0 = s.self();
-    const T psi = F.psi[i0];
-    T C[N];
-    {
-        T sum = T(0);
+    T cth[NP], m[NP + 1];
+    angles<T, NP>(P, F, i0, cth);
+    auto at = [&](int p) { return s.at(cx(p), cy(p), cz(p)); };
+    if constexpr (sizeof(T) == 8) {
+        const T psi = __ldg(F.psi + i0);
+        T ps[15], c0[NP], L[NP];
+#pragma unroll
+        for (int p = 1; p < 15; ++p) ps[p] = psi + __ldg(F.psi + at(p));
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
-            C[j] = F.C[j * P.plane + i0];
-            sum += C[j];
+            const T* C = F.C + j * P.plane;
+            c0[j] = __ldg(C + i0);
+            L[j] = lap15(P, [&](int p) { return ps[p]; }, [&](int p) { return __ldg(C + at(p)); }, c0[j]);
         }
-        C[NP] = T(1) - sum;
+        ddcc::dev::mu_of<T, NP + 1>(P, c0, L, cth, __ldg(F.st + kAgp3 * P.plane + i0),
+                                    __ldg(F.st + kInvPsi * P.plane + i0), m);
+    } else {
+        T gp[3];
+        mu_node<T, NP>(P, [&](int p) { return F.psi[at(p)]; }, [&](int j, int p) { return F.C[j * P.plane + at(p)]; },
+                       cth, m, gp);
     }
-    T L[N];
 #pragma unroll
-    for (int j = 0; j < N; ++j) L[j] = T(0);
-    T gpx = T(0), gpy = T(0), gpz = T(0);
+    for (int i = 0; i < NP + 1; ++i) F.mu[i * P.plane + i0] = m[i];
+}
+
+// (FP64) the static planes from psi
+template <typename T>
+__global__ void __launch_bounds__(node_threads<T>()) k3_static(P3<T> P, F3<T> F) {
+    Site s;
+    if (!site(P, s)) return;
+    const long long i0 = s.self();
+    T g[3];
+    grad15(P, [&](int p) { return F.psi[s.at(cx(p), cy(p), cz(p))]; }, g);
+    F.st[kInvPsi * P.plane + i0] = rcp(F.psi[i0]);
 #pragma unroll
-    for (int p = 1; p < 15; ++p) {
-        const long long ip = s.at(cx(p), cy(p), cz(p));
-        const T w = p < 7 ? P.ga : P.gc;
-        const T psp = F.psi[ip];
-        const T wp = w * psp;
-        if (cx(p)) gpx += T(cx(p)) * wp;
-        if (cy(p)) gpy += T(cy(p)) * wp;
-        if (cz(p)) gpz += T(cz(p)) * wp;
-        const T wpsi = w * (psi + psp);
-        T sum = T(0);
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            const T Cp = F.C[j * P.plane + ip];
-            sum += Cp;
-            L[j] += wpsi * (Cp - C[j]);
-        }
-        L[NP] += wpsi * ((T(1) - sum) - C[NP]);
-    }
-    T cN[N];
-#pragma unroll
-    for (int j = 0; j < NP; ++j) cN[j] = P.has_cos_field ? F.cosf[j * P.plane + i0] : P.cos_uni[j];
-    cN[NP] = T(0);
-    T m[N];
-    mu_from_stencil<T, NP>(P, psi, C, L, gpx, gpy, gpz, cN, m);
-#pragma unroll
-    for (int i = 0; i < N; ++i) F.mu[i * P.plane + i0] = m[i];
+    for (int a = 0; a < 3; ++a) F.st[(kGrad + a) * P.plane + i0] = g[a];
+    F.st[kAgp3 * P.plane + i0] = T(3) * root(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
 }
 
 // The same chemical potentials for four consecutive x nodes per thread
@@ -291,24 +379,21 @@ __global__ void __launch_bounds__(kThreads, NP <= 2 ? 3 : 2) k3_mu4(P3<float> P,
     auto at = [&](int f, int k, int dx) {
         return dx == 0 ? v[f][k] : (dx < 0 ? (k == 0 ? lf[f] : v[f][k - 1]) : (k == 3 ? rt[f] : v[f][k + 1]));
     };
-    float psi[4], C[N][4], L[N][4], g[3][4];
+    float psi[4], C[NP][4], La[NP][4], Lc[NP][4], g[3][4];
     load_row(0, 0, true);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         psi[k] = v[0][k];
-        float sum = 0.f;
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
             C[j][k] = v[1 + j][k];
-            sum += C[j][k];
+            La[j][k] = Lc[j][k] = 0.f;
         }
-        C[NP][k] = 1.f - sum;
-#pragma unroll
-        for (int j = 0; j < N; ++j) L[j][k] = 0.f;
         g[0][k] = g[1][k] = g[2][k] = 0.f;
     }
     // neighbour (dx, dy, dz) of node k, stencil weight w, from the loaded row
     auto accumulate = [&](int dx, int dy, int dz, float w) {
+        const bool axis = dx * dx + dy * dy + dz * dz == 1;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const float psp = at(0, k, dx);
@@ -316,15 +401,13 @@ __global__ void __launch_bounds__(kThreads, NP <= 2 ? 3 : 2) k3_mu4(P3<float> P,
             if (dx) g[0][k] += float(dx) * wp;
             if (dy) g[1][k] += float(dy) * wp;
             if (dz) g[2][k] += float(dz) * wp;
-            const float wpsi = w * (psi[k] + psp);
-            float sum = 0.f;
+            const float ps = psi[k] + psp;
 #pragma unroll
             for (int j = 0; j < NP; ++j) {
-                const float Cp = at(1 + j, k, dx);
-                sum += Cp;
-                L[j][k] += wpsi * (Cp - C[j][k]);
+                const float d = ps * (at(1 + j, k, dx) - C[j][k]);
+                if (axis) La[j][k] += d;
+                else Lc[j][k] += d;
             }
-            L[NP][k] += wpsi * ((1.f - sum) - C[NP][k]);
         }
     };
     accumulate(1, 0, 0, P.ga);
@@ -357,14 +440,15 @@ __global__ void __launch_bounds__(kThreads, NP <= 2 ? 3 : 2) k3_mu4(P3<float> P,
     float out[N][4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        float Ck[N], Lk[N], ck[N], m[N];
+        float Ck[NP], Lk[NP], ck[NP], m[N];
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
+        for (int j = 0; j < NP; ++j) {
             Ck[j] = C[j][k];
-            Lk[j] = L[j][k];
-            ck[j] = j < NP ? cN[j < NP ? j : 0][k] : 0.f;
+            Lk[j] = P.la * La[j][k] + P.lc * Lc[j][k];
+            ck[j] = cN[j][k];
         }
-        mu_from_stencil<float, NP>(P, psi[k], Ck, Lk, g[0][k], g[1][k], g[2][k], ck, m);
+        const float agp3 = 3.f * root(g[0][k] * g[0][k] + g[1][k] * g[1][k] + g[2][k] * g[2][k]);
+        ddcc::dev::mu_of<float, N>(P, Ck, Lk, ck, agp3, rcp(psi[k]), m);
 #pragma unroll
         for (int i = 0; i < N; ++i) out[i][k] = m[i];
     }
@@ -376,240 +460,225 @@ __global__ void __launch_bounds__(kThreads, NP <= 2 ? 3 : 2) k3_mu4(P3<float> P,
 // ---------------------------------------------------------------------------
 // node update (kMacro = false) or read-out of rho, u, P (kMacro = true)
 // ---------------------------------------------------------------------------
-// sum_p w_p c_p v(p) / cs2 on the 15-point stencil (p = 1..14), from the
-// pairs of opposite neighbours: an axis pair gives its difference to its
-// own component; the corner pairs (7, 14), (8, 13), (9, 12), (10, 11) give
-// their differences d, signed by the first member's velocity.
-template <typename T, class V>
-__device__ __forceinline__ void grad15(const P3<T>& P, const V& v, T g[3]) {
-    const T d0 = v(7) - v(14), d1 = v(8) - v(13), d2 = v(9) - v(12), d3 = v(10) - v(11);
-    const T s01 = d0 + d1, s23 = d2 + d3;
-    g[0] = P.ga * (v(1) - v(2)) + P.gc * ((d0 - d1) + (d2 - d3));
-    g[1] = P.ga * (v(3) - v(4)) + P.gc * (s01 - s23);
-    g[2] = P.ga * (v(5) - v(6)) + P.gc * (s01 + s23);
-}
-
-// Where the node update reads psi, C and mu: neighbour p of the velocity
-// list (p = 0 the node itself) and the global index of that neighbour (the
-// lagged field a is read there, populations are pushed there).
-template <typename T>
+// Where the node update reads its fields: neighbour p of the velocity list
+// (p = 0 the node itself) and the global index of that neighbour (the lagged
+// field a is read there, populations are pushed there).
+template <typename T, int NP>
 struct GlobalSrc {     // the per-step C and mu planes in global memory
+    const P3<T>& P;
+    const F3<T>& F;
     Site s;
-    const T* psi_;
-    const T* C_;
-    const T* mu_;
-    const T* g_;       // flow populations and lagged planes of the input copy
+    const T* f_;       // populations and lagged planes of the input copy
+    const T* g_;
     const T* lag_;
-    long long plane;
     __device__ long long at(int p) const { return s.at(cx(p), cy(p), cz(p)); }
-    __device__ T g(int p) const { return g_[p * plane + s.self()]; }
-    __device__ T lag(int k) const { return lag_[k * plane + s.self()]; }
-    __device__ T psi(int p) const { return psi_[at(p)]; }
-    __device__ T C(int j, int p) const { return C_[j * plane + at(p)]; }
-    __device__ T mu(int j, int p) const { return mu_[j * plane + at(p)]; }
+    __device__ T f(int i, int p) const { return __ldg(f_ + (7 * i + p) * P.plane + s.self()); }
+    __device__ T g(int p) const { return __ldg(g_ + p * P.plane + s.self()); }
+    __device__ T lag(int k) const { return __ldg(lag_ + k * P.plane + s.self()); }
+    __device__ T a(int k, int p) const { return __ldg(lag_ + lag_a(k) * P.plane + at(p)); }
+    __device__ T psi(int p) const { return __ldg(F.psi + at(p)); }
+    __device__ T C(int j, int p) const { return __ldg(F.C + j * P.plane + at(p)); }
+    __device__ T mu(int j, int p) const { return __ldg(F.mu + j * P.plane + at(p)); }
+    __device__ T psirho(int p) const {
+        if constexpr (sizeof(T) == 8) return __ldg(F.chi + at(p));
+        else return psi_rho<T, NP>(P, psi(p), [&](int j) { return C(j, p); });
+    }
+    __device__ void grad_psi(T gp[3]) const {
+        if constexpr (sizeof(T) == 8) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) gp[a] = __ldg(F.st + (kGrad + a) * P.plane + s.self());
+        } else {
+            grad15(P, [&](int p) { return psi(p); }, gp);
+        }
+    }
 };
 
+// sum_j C_j = 1 (C_N is defined by it), so sums over all phases reduce to the
+// N-1 evolved ones: rho and grad rho through rho_j - rho_N, the capillary
+// force through mu_j - mu_N, m^C = -m0 sum_j (rho_j - rho_N) Q_j because the
+// Q_j = C_j (grad mu_j - sum_k C_k grad mu_k) add up to zero.  For two phases
+// mu_2 = -mu_1.  kMacro: rho, u and P of the state go to the planes at out
+// instead.
+// FP64 (three kernels, bound by FP64 warp instructions): 96 x 80 x 72, N = 3,
+// 1116 + 341 + 35 us for update, mu and C before sums over all phases, pair
+// identities of mu, psi's own terms, 256-thread blocks of 32 x 4 x 2 nodes and
+// divisions by the operator went; 10 steps and a read-out 18.0 -> 9.4 ms.
+// FP32 (fused): 24% fewer instructions, 753 -> 722 us at 208 x 192 x 160; the
+// loads and stores of this kernel alone take 504 us there (loads 314), the
+// stores in 128-byte rows of 45 planes.
 template <typename T, int NP, bool kMacro, class S>
-__device__ __forceinline__ void update_node(const P3<T>& P, const F3<T>& F, int cur, int field, double* out,
-                                            const S& src) {
-    constexpr int N = NP + 1;
+__device__ __forceinline__ void update_node(const P3<T>& P, const F3<T>& F, int cur, T* out, const S& src) {
+    constexpr int N = NP + 1, NM = NP == 1 ? 1 : N;
     const long long i0 = src.at(0);
     const int nxt = cur ^ 1;
     const T psi = src.psi(0);
     const T cs2 = P.cs2;
-    T C[N], mu[N];
+    T C[N], gC[NP][3], mu[NM], gmu[NM][3], G[3], gpr[3];
+    T dA[3];   // -div A: (d_y a_xy - d_z a_zx, d_z a_yz - d_x a_xy, d_x a_zx - d_y a_yz)
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+        for (int j = 0; j < NP; ++j) grad15(P, [&](int p) { return src.C(j, p); }, gC[j]);
+#pragma unroll
+        for (int j = 0; j < NM; ++j) grad15(P, [&](int p) { return src.mu(j, p); }, gmu[j]);
+        grad15(P, [&](int p) { return src.psirho(p); }, gpr);
+        T gaxy[3], gayz[3], gazx[3];
+        grad15(P, [&](int p) { return src.a(0, p); }, gaxy);
+        grad15(P, [&](int p) { return src.a(1, p); }, gayz);
+        grad15(P, [&](int p) { return src.a(2, p); }, gazx);
+        dA[0] = gaxy[1] - gazx[2];
+        dA[1] = gayz[2] - gaxy[0];
+        dA[2] = gazx[0] - gayz[1];
+    } else {
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+            const int q = k < 4 ? k + 3 : k - 4, p = pair_rep(q), o = pair_opp(q);
+            // a first: from global memory
+            const T dxy = q != 2 ? src.a(0, p) - src.a(0, o) : T(0);
+            const T dyz = q != 0 ? src.a(1, p) - src.a(1, o) : T(0);
+            const T dzx = q != 1 ? src.a(2, p) - src.a(2, o) : T(0);
+#pragma unroll
+            for (int j = 0; j < NP; ++j) add_pair(P, q, src.C(j, p) - src.C(j, o), gC[j]);
+#pragma unroll
+            for (int j = 0; j < NM; ++j) add_pair(P, q, src.mu(j, p) - src.mu(j, o), gmu[j]);
+            add_pair(P, q, src.psirho(p) - src.psirho(o), gpr);
+            if (q >= 3) {
+                const T sx = T(cx(p)), sy = T(cy(p)), sz = T(cz(p));
+                const T t0 = sy * dxy - sz * dzx, t1 = sz * dyz - sx * dxy, t2 = sx * dzx - sy * dyz;
+                dA[0] = q == 3 ? t0 : dA[0] + t0;
+                dA[1] = q == 3 ? t1 : dA[1] + t1;
+                dA[2] = q == 3 ? t2 : dA[2] + t2;
+            } else {
+                // weight the corners' sums once, with the first axis pair
+                if (q == 0) {
+                    dA[0] *= P.gc;
+                    dA[1] = P.gc * dA[1] - P.ga * dxy;
+                    dA[2] = P.gc * dA[2] + P.ga * dzx;
+                } else if (q == 1) {
+                    dA[0] += P.ga * dxy;
+                    dA[2] -= P.ga * dyz;
+                } else {
+                    dA[0] -= P.ga * dzx;
+                    dA[1] += P.ga * dyz;
+                }
+            }
+        }
+    }
+    T rho = P.rho[NP], nu = P.nu[NP], grho[3];
     {
         T sum = T(0);
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
             C[j] = src.C(j, 0);
-            sum += C[j];
+            sum = j == 0 ? C[0] : sum + C[j];
+            rho += P.drho[j] * C[j];
+            nu += P.dnu[j] * C[j];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) grho[a] = j == 0 ? P.drho[0] * gC[0][a] : grho[a] + P.drho[j] * gC[j][a];
         }
         C[NP] = T(1) - sum;
     }
 #pragma unroll
-    for (int j = 0; j < N; ++j) mu[j] = src.mu(j, 0);
-
-    // gradients on the 15-point stencil: psi, C_j (j < N-1), mu_j, psi rho,
-    // and the derivatives of a_xy, a_yz, a_zx the divergence needs.  FP64
-    // (bound by its FP64 pipe) takes them field by field from the pairs of
-    // opposite neighbours (grad15, fewer operations); FP32 (bound by the
-    // fused kernel's registers) in one pass over the neighbours.
-    const T* lagc = pick(F.lag, cur);
-    T gps[3], gpr[3], gC[NP][3], gmu[N][3];
-    T dxy_y, dxy_x, dyz_z, dyz_y, dzx_x, dzx_z;
-    if constexpr (sizeof(T) == 8) {
-        grad15(P, [&](int p) { return src.psi(p); }, gps);
+    for (int j = 0; j < NM; ++j) mu[j] = src.mu(j, 0);
+    if constexpr (NP == 1) {
+        const T dC = C[0] - C[1];
 #pragma unroll
-        for (int j = 0; j < NP; ++j) grad15(P, [&](int p) { return src.C(j, p); }, gC[j]);
-#pragma unroll
-        for (int j = 0; j < N; ++j) grad15(P, [&](int p) { return src.mu(j, p); }, gmu[j]);
-        grad15(P, [&](int p) {
-            T rhop = T(0), sum = T(0);
-#pragma unroll
-            for (int j = 0; j < NP; ++j) {
-                const T Cp = src.C(j, p);
-                sum += Cp;
-                rhop += P.rho[j] * Cp;
-            }
-            rhop += P.rho[NP] * (T(1) - sum);
-            return src.psi(p) * rhop;
-        }, gpr);
-        T gaxy[3], gayz[3], gazx[3];
-        grad15(P, [&](int p) { return lagc[lag_a(0) * P.plane + src.at(p)]; }, gaxy);
-        grad15(P, [&](int p) { return lagc[lag_a(1) * P.plane + src.at(p)]; }, gayz);
-        grad15(P, [&](int p) { return lagc[lag_a(2) * P.plane + src.at(p)]; }, gazx);
-        dxy_x = gaxy[0];
-        dxy_y = gaxy[1];
-        dyz_y = gayz[1];
-        dyz_z = gayz[2];
-        dzx_z = gazx[2];
-        dzx_x = gazx[0];
+        for (int a = 0; a < 3; ++a) G[a] = dC * gmu[0][a];
     } else {
-        gps[0] = gps[1] = gps[2] = T(0);
-        gpr[0] = gpr[1] = gpr[2] = T(0);
 #pragma unroll
-        for (int j = 0; j < NP; ++j) gC[j][0] = gC[j][1] = gC[j][2] = T(0);
+        for (int j = 0; j < NM; ++j)
 #pragma unroll
-        for (int j = 0; j < N; ++j) gmu[j][0] = gmu[j][1] = gmu[j][2] = T(0);
-        dxy_y = dxy_x = dyz_z = dyz_y = dzx_x = dzx_z = T(0);
-#pragma unroll
-        for (int p = 1; p < 15; ++p) {
-            const long long ip = src.at(p);
-            const T w = p < 7 ? P.ga : P.gc;
-            const T psp = src.psi(p);
-            T rhop = T(0), sum = T(0);
-#pragma unroll
-            for (int j = 0; j < NP; ++j) {
-                const T Cp = src.C(j, p);
-                sum += Cp;
-                rhop += P.rho[j] * Cp;
-                const T wc = w * Cp;
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    if (cc(p, a)) gC[j][a] += T(cc(p, a)) * wc;
-            }
-            rhop += P.rho[NP] * (T(1) - sum);
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                const T wm = w * src.mu(j, p);
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    if (cc(p, a)) gmu[j][a] += T(cc(p, a)) * wm;
-            }
-            const T wp = w * psp, wpr = w * psp * rhop;
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-                if (cc(p, a)) {
-                    gps[a] += T(cc(p, a)) * wp;
-                    gpr[a] += T(cc(p, a)) * wpr;
-                }
-            const T axy = w * lagc[lag_a(0) * P.plane + ip];
-            const T ayz = w * lagc[lag_a(1) * P.plane + ip];
-            const T azx = w * lagc[lag_a(2) * P.plane + ip];
-            if (cx(p)) { dxy_x += T(cx(p)) * axy; dzx_x += T(cx(p)) * azx; }
-            if (cy(p)) { dxy_y += T(cy(p)) * axy; dyz_y += T(cy(p)) * ayz; }
-            if (cz(p)) { dyz_z += T(cz(p)) * ayz; dzx_z += T(cz(p)) * azx; }
-        }
+            for (int a = 0; a < 3; ++a) G[a] = j == 0 ? C[0] * gmu[0][a] : G[a] + C[j] * gmu[j][a];
     }
-    T grho[3];
+    T Q[NP][3], mC[3];   // mC: psi m^C
+    const T pm0 = -(P.m0 * psi);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        T gN = T(0), acc = T(0);
+        T t = T(0);
 #pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            gN -= gC[j][a];
-            acc += P.rho[j] * gC[j][a];
+        for (int i = 0; i < NP; ++i) {
+            Q[i][a] = C[i] * (gmu[i][a] - G[a]);
+            t = i == 0 ? P.drho[0] * Q[0][a] : t + P.drho[i] * Q[i][a];
         }
-        grho[a] = acc + P.rho[NP] * gN;
+        mC[a] = pm0 * t;
     }
+    T gps[3];
+    src.grad_psi(gps);
 
-    T rho = T(0), nu = T(0);
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-        rho += C[j] * P.rho[j];
-        nu += C[j] * P.nu[j];
-    }
     const T t21 = nu * P.nu_to_s21 + T(0.5);   // 1 / s21
-    const T s21 = T(1) / t21;
-    const T s22 = T(1) / (nu * P.inv_cs2_nu + T(0.5));
+    const T s21 = rcp(t21);
+    const T s22 = rcp(nu * P.inv_cs2_nu + T(0.5));
 
-    // mobility (Eq. 2.5): M_ij = -m0 C_i C_j, M_ii = m0 C_i sum_{j != i} C_j;
-    // m^C = -sum_ij rho_i M_ij grad mu_j
-    T mC[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            T Mij;
-            if (i == j) {
-                T o = T(0);
-#pragma unroll
-                for (int q = 0; q < N; ++q)
-                    if (q != i) o += C[q];
-                Mij = P.m0 * C[i] * o;
-            } else {
-                Mij = -P.m0 * C[i] * C[j];
-            }
-#pragma unroll
-            for (int a = 0; a < 3; ++a) mC[a] -= P.rho[i] * Mij * gmu[j][a];
-        }
-
-    // force without P grad psi and the damping: sum_i psi mu_i grad C_i,
-    // -div A (A_jk = psi (m^C_j u_k - u_j m^C_k)/2, lagged), psi rho b
+    // force without P grad psi and the damping: psi (sum_j (mu_j - mu_N) grad
+    // C_j + rho b) - div A (A_jk = psi (m^C_j u_k - u_j m^C_k)/2, lagged)
     T Fv[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        T acc = T(0), gN = T(0);
+        T t = rho * P.body[a];
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
-            acc += psi * mu[j] * gC[j][a];
-            gN -= gC[j][a];
+            T dm;
+            if constexpr (NP == 1) dm = mu[0] + mu[0];
+            else dm = mu[j] - mu[NM - 1];
+            t += dm * gC[j][a];
         }
-        acc += psi * mu[NP] * gN;
-        Fv[a] = acc;
+        Fv[a] = psi * t + dA[a];
     }
-    Fv[0] += dxy_y - dzx_z;
-    Fv[1] += dyz_z - dxy_x;
-    Fv[2] += dzx_x - dyz_y;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Fv[a] += psi * rho * P.body[a];
 
-    T g[15];
+    // D3Q15 moments.  Opposite velocities come in seven pairs: an even
+    // polynomial of c takes the pairs' sums, an odd one their differences; the
+    // four corner pairs' signs are those of grad15.
+    T j3[3], t3[3], e2[3], o2[3], xyz, corner, mm, sum_g;
+    {
+        T gs[7], gd[7];
 #pragma unroll
-    for (int p = 0; p < 15; ++p) g[p] = src.g(p);
-    T sum_g = T(0), J[3] = {T(0), T(0), T(0)};
+        for (int q = 0; q < 7; ++q) {
+            const T a = src.g(pair_rep(q)), b = src.g(pair_opp(q));
+            gs[q] = a + b;
+            gd[q] = a - b;
+        }
+        const T m01 = gd[3] - gd[4], m23 = gd[5] - gd[6], s01 = gd[3] + gd[4], s23 = gd[5] + gd[6];
+        t3[0] = m01 + m23;
+        t3[1] = s01 - s23;
+        t3[2] = s01 + s23;
+        xyz = m01 - m23;
+        const T c01 = gs[3] + gs[4], c23 = gs[5] + gs[6], n01 = gs[3] - gs[4], n23 = gs[5] - gs[6];
+        corner = c01 + c23;
+        o2[0] = n01 - n23;
+        o2[1] = c01 - c23;
+        o2[2] = n01 + n23;
+        sum_g = (gs[0] + gs[1]) + (gs[2] + corner);
+        mm = src.g(0) + sum_g;
 #pragma unroll
-    for (int p = 1; p < 15; ++p) {
-        sum_g += g[p];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            if (cc(p, a)) J[a] += T(cc(p, a)) * g[p];
+        for (int a = 0; a < 3; ++a) {
+            j3[a] = gd[a] + t3[a];
+            e2[a] = gs[a] + corner;
+        }
     }
-    const T damp = (T(1) - psi) * P.damp;
-    const T den = psi * rho + T(0.5) * damp;
-    const T Hc = P.Hfac * (s21 - T(2));
-    const T inv_den = T(1) / den;
-    T u0[3], e[3], bv[3];
+    const T psirho = psi * rho;
+    const T damp = P.damp - P.damp * psi;
+    const T inv_den = rcp(psirho + T(0.5) * damp);
+    const T hi = T(0.5) * inv_den;
+    const T Hs = P.Hfac - T(2) * P.Hfac * t21;   // H / s21
+    const T Ap = P.A_P * psi;
+    const T gam = P.kk * psirho;
+    // Eq. 19 with u = u0 + P e: cP gam e.e P^2 + (cP (b + 2 gam u0).e - psi) P
+    // + cP (G0 + (b + gam u0).u0) = 0
+    T u0[3], e[3], ee, we, vu;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        u0[a] = (J[a] + T(0.5) * Fv[a]) * inv_den;
-        e[a] = T(0.5) * gps[a] * inv_den;
-        bv[a] = P.A_P * psi * grho[a] + P.kk * psi * mC[a] + Hc * t21 * gpr[a];
+        u0[a] = (j3[a] + T(0.5) * Fv[a]) * inv_den;
+        e[a] = gps[a] * hi;
+        const T v = Ap * grho[a] + P.kk * mC[a] + Hs * gpr[a] + gam * u0[a];
+        const T w = v + gam * u0[a];
+        ee = a == 0 ? e[0] * e[0] : ee + e[a] * e[a];
+        we = a == 0 ? w * e[0] : we + w * e[a];
+        vu = a == 0 ? v * u0[0] : vu + v * u0[a];
     }
-    const T gam = P.kk * psi * rho;
-    const T G0 = sum_g - T(0.5) * P.K * src.lag(lag_pm<NP>());
-    const T ee = e[0] * e[0] + e[1] * e[1] + e[2] * e[2];
-    const T be = bv[0] * e[0] + bv[1] * e[1] + bv[2] * e[2];
-    const T ue = u0[0] * e[0] + u0[1] * e[1] + u0[2] * e[2];
-    const T bu = bv[0] * u0[0] + bv[1] * u0[1] + bv[2] * u0[2];
-    const T uu = u0[0] * u0[0] + u0[1] * u0[1] + u0[2] * u0[2];
     const T qa = P.cP * gam * ee;
-    const T qb = P.cP * (be + T(2) * gam * ue) - psi;
-    const T qc = P.cP * (G0 + bu + gam * uu);
-    const T disc = fmax(qb * qb - T(4) * qa * qc, T(0));
-    const T root = sqrt(disc);
-    const T Pp = T(-2) * qc / (qb < T(0) ? qb - root : qb + root);
+    const T qb = P.cP * we - psi;
+    const T qc = P.cP * ((sum_g - P.half_K * src.lag(lag_pm<NP>())) + vu);
+    const T disc = clamp0(qb * qb - T(4) * qa * qc);
+    const T Pp = T(-2) * qc * rcp(qb + signed_as(root(disc), qb));
     T u[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -617,18 +686,14 @@ __device__ __forceinline__ void update_node(const P3<T>& P, const F3<T>& F, int 
         Fv[a] += Pp * gps[a] - damp * u[a];
     }
     if constexpr (kMacro) {
-        double v = 0.0;
-        if (field == DDCC_FIELD_RHO) v = (double)rho;
-        else if (field == DDCC_FIELD_UX) v = (double)u[0];
-        else if (field == DDCC_FIELD_UY) v = (double)u[1];
-        else if (field == DDCC_FIELD_UZ) v = (double)u[2];
-        else if (field == DDCC_FIELD_P) v = (double)Pp;
-        out[i0] = v;
+        out[i0] = rho;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) out[(1 + a) * P.plane + i0] = u[a];
+        out[4 * P.plane + i0] = Pp;
         return;
     } else {
         T* lagn = pick(F.lag, nxt);
         // ---- phase LB (Eqs. 3.1, 3.5-3.7), D3Q7 ----
-        const T* fcur = pick(F.f, cur);
         T* fnew = pick(F.f, nxt);
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
@@ -636,188 +701,135 @@ __device__ __forceinline__ void update_node(const P3<T>& P, const F3<T>& F, int 
             T psiC = T(0);
 #pragma unroll
             for (int p = 0; p < 7; ++p) {
-                f[p] = fcur[(7 * i + p) * P.plane + i0];
-                psiC += f[p];
+                f[p] = src.f(i, p);
+                psiC = p == 0 ? f[0] : psiC + f[p];
             }
-            // S_i = psi [(C_i sum_{j != i} C_j - 1) grad mu_i - sum_{j != i} C_i C_j grad mu_j]
-            T V[3];
-            T o = T(0);
-#pragma unroll
-            for (int q = 0; q < N; ++q)
-                if (q != i) o += C[q];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                T S = (C[i] * o - T(1)) * gmu[i][a];
-#pragma unroll
-                for (int j = 0; j < N; ++j)
-                    if (j != i) S -= C[i] * C[j] * gmu[j][a];
-                S *= psi;
-                const T cu = psiC * u[a];
-                V[a] = (cu - src.lag(lag_cu(i, a)))
-                       + cs2 * P.eta[i] * (mu[i] * gps[a] - S);
-                lagn[lag_cu(i, a) * P.plane + i0] = cu;
-            }
-            const T epm = P.eta[i] * psi * mu[i];
+            const T csepm = P.ceta[i] * (psi * mu[i]);
             // Lambda v, v = f - f^eq + F/2, on the D3Q7 rows 1, c_a,
             // c_a^2 - cs2 (S = s0, s1, s21) from the moments of v: the zeroth
             // vanishes (sum f^eq = psi C = sum f, sum F = 0); the first is
             // j_a(f) - psi C u_a + V_a / 2; the raw second, sum_{+-a} v, is
-            // e_a(f) - d0 eta psi mu (Eqs. 3.5, 3.6, B.5b, B.5c)
-            T Es = T(0), wv[7];
+            // e_a(f) - d0 eta psi mu (Eqs. 3.5, 3.6, B.5b, B.5c).  F_p = w_p
+            // c_p . V / cs2 is +-V_a / 2 (w_1 = cs2 / 2) and zero at rest.
+            // V = d_t(psi C u) + cs2 eta (mu grad psi - S), S = psi (Q - grad mu)
+            T hE[3], h[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 const T fp = f[1 + 2 * a], fm = f[2 + 2 * a];
-                const T Ja = P.s1f[i] * ((fp - fm) - psiC * u[a] + T(0.5) * V[a]);
-                const T Ea = P.s21f * ((fp + fm) - cs2 * epm);
-                wv[1 + 2 * a] = T(0.5) * (Ea + Ja);
-                wv[2 + 2 * a] = T(0.5) * (Ea - Ja);
-                Es += Ea;
+                const T cu = psiC * u[a];
+                const T V = (cu - src.lag(lag_cu(i, a))) +
+                            P.ceta[i] * (mu[i] * gps[a] + psi * (gmu[i][a] - Q[i][a]));
+                lagn[lag_cu(i, a) * P.plane + i0] = cu;
+                h[a] = P.h1f[i] * ((fp - fm) - cu) + P.h2f[i] * V;
+                hE[a] = P.hs21f * ((fp + fm) - csepm);
             }
-            wv[0] = -Es;
-            // F_p = w_p c_p . V / cs2 (Eq. 3.6): zero at rest, +-w1 V_a / cs2.
-            // The rest population's new value f_0 - wv_0 is rounded
+            // The rest population's new value f_0 + 2 sum_a hE_a is rounded
             // explicitly and its exact rounding error (TwoSum) is split
             // evenly between the populations p = 1 and 2 (+x and -x), so
             // sum_p f keeps the exchange and no direction is preferred.
-            const T o0 = add_rn(f[0], -wv[0]);
+            const T w0 = T(2) * ((hE[0] + hE[1]) + hE[2]);
+            const T o0 = add_rn(f[0], w0);
             const T bb = add_rn(o0, -f[0]);
-            const T err = T(0.5) * add_rn(add_rn(f[0], -add_rn(o0, -bb)), add_rn(-wv[0], -bb));
+            const T err = T(0.5) * add_rn(add_rn(f[0], -add_rn(o0, -bb)), add_rn(w0, -bb));
             fnew[(7 * i) * P.plane + i0] = o0;
 #pragma unroll
-            for (int p = 1; p < 7; ++p) {
-                const int a = (p - 1) >> 1;
-                const T Fp = T(cc(p, a)) * P.w7_1 * V[a] * P.inv_cs2;
-                T out = f[p] - wv[p] + Fp;
-                if (p <= 2) out = add_rn(out, err);
-                fnew[(7 * i + p) * P.plane + src.at(p)] = out;
+            for (int a = 0; a < 3; ++a) {
+                // the two parts are joined first: in a steady flow hE is below
+                // the ulp of f and would be lost on its own every step
+                T op = f[1 + 2 * a] - (hE[a] + h[a]), om = f[2 + 2 * a] - (hE[a] - h[a]);
+                if (a == 0) {
+                    op = add_rn(op, err);
+                    om = add_rn(om, err);
+                }
+                fnew[(7 * i + 1 + 2 * a) * P.plane + src.at(1 + 2 * a)] = op;
+                fnew[(7 * i + 2 + 2 * a) * P.plane + src.at(2 + 2 * a)] = om;
             }
         }
 
         // ---- flow LB (Eqs. 3.2, 3.8, 3.10), D3Q15 ----
-        T diag[3], off[3], Tn[6];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            diag[a] = psi * rho * u[a] * u[a] + psi * mC[a] * u[a];
-            Tn[a] = psi * mC[a] * u[a];
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int a = k, b = (k + 1) % 3;
-            off[k] = psi * rho * u[a] * u[b] + T(0.5) * (psi * mC[a] * u[b] + psi * u[a] * mC[b]);
-            Tn[3 + k] = T(0.5) * (psi * mC[a] * u[b] + psi * u[a] * mC[b]);
-        }
-        const T ugpr = u[0] * gpr[0] + u[1] * gpr[1] + u[2] * gpr[2];
-        T M2[6];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            M2[a] = (Tn[a] - src.lag(lag_T<NP>(a))) + T(2) * cs2 * u[a] * gpr[a] + P.c2m3 * ugpr;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int a = k, b = (k + 1) % 3;
-            M2[3 + k] = (Tn[3 + k] - src.lag(lag_T<NP>(3 + k)))
-                        + cs2 * (u[a] * gpr[b] + gpr[a] * u[b]);
-        }
-        const T a0 = psi * (u[0] * grho[0] + u[1] * grho[1] + u[2] * grho[2]);
-        const T psiP = psi * Pp;
         // The collision runs in moment space on the orthogonal D3Q15 rows
         // h_k: with v = g - g^eq + G/2 and G = w (sum_k h_k <h_k, G> / |h_k|^2)
         // (G is w times a polynomial of degree <= 2),
         //   g* = g - Lambda v + G = g - w sum_k h_k mu_k,
         //   mu_k = (s_k / |h_k|^2) <h_k, v> - <h_k, G> / |h_k|^2.
         // <h_k, g^eq> (Eq. 3.8, g_0 stored as g_0 - rho0) = 0, psi rho u_a,
-        // diag_a + psi P, off_k, 0 (third order), -2 cs2 psi P (the rest
+        // A_aa + psi P, A_ab, 0 (third order), -2 cs2 psi P (the rest
         // population's -psi P / cs2 on the last row); <h_k, G> (Eq. 3.10) =
-        // a0, F_a, M_aa, M_ab, 0 (Eqs. B.5d, B.5e).
-        // Opposite velocities come in seven pairs (p, pb), c_pb = -c_p: an even
-        // polynomial of c takes the pair's sum g_p + g_pb, an odd one its
-        // difference, and the collided pair is g - w (E +- O) with E, O the
-        // even and odd parts of sum_k h_k(c_p) m_k.
-        T gs[7], gd[7];
+        // a0, F_a, M_aa, M_ab, 0 (Eqs. B.5d, B.5e); A = psi rho u u + T,
+        // T = psi (m^C u + u m^C) / 2.
+        const T psiP = psi * Pp;
+        T s[3], ugpr = T(0), pm = T(0), m1[3], m4[3], m7[3];
 #pragma unroll
-        for (int q = 0; q < 7; ++q) {
-            gs[q] = g[pair_rep(q)] + g[pair_opp(q)];
-            gd[q] = g[pair_rep(q)] - g[pair_opp(q)];
+        for (int a = 0; a < 3; ++a) {
+            s[a] = u[a] * gpr[a];
+            ugpr = a == 0 ? s[0] : ugpr + s[a];
         }
-        T m[15];
-        {
-            T mm = g[0], j[3] = {T(0), T(0), T(0)}, e2[3] = {T(0), T(0), T(0)};
-            T o2[3] = {T(0), T(0), T(0)}, t3[3] = {T(0), T(0), T(0)}, xyz = T(0), corner = T(0);
+        const T cu3 = P.c2m3 * ugpr;
+        const T l2d = P.inv_n2d * s21, c2d = T(0.5) * l2d - P.inv_n2d;
+        const T l2o = P.inv_n2o * s22, c2o = T(0.5) * l2o - P.inv_n2o;
+        const T cmm = cs2 * mm;
 #pragma unroll
-            for (int q = 0; q < 7; ++q) {
-                const int p = pair_rep(q);
-                mm += gs[q];
+        for (int a = 0; a < 3; ++a) {
+            const int b = (a + 1) % 3;
+            const T ja = psirho * u[a];
+            const T Taa = mC[a] * u[a];
+            const T Aaa = ja * u[a] + Taa;
+            pm = a == 0 ? Aaa : pm + Aaa;
+            const T p1 = mC[a] * u[b], p2 = u[a] * mC[b];
+            const T Tab = T(0.5) * (p1 + p2);
+            const T Aab = ja * u[b] + Tab;
+            const T Maa = (Taa - src.lag(lag_T<NP>(a))) + P.two_cs2 * s[a] + cu3;
+            const T Mab = (Tab - src.lag(lag_T<NP>(3 + a))) + cs2 * (u[a] * gpr[b] + gpr[a] * u[b]);
+            m1[a] = P.lg1 * (j3[a] - ja) + P.cg1 * Fv[a];
+            m4[a] = l2d * ((e2[a] - cmm) - (Aaa + psiP)) + c2d * Maa;
+            m7[a] = l2o * (o2[a] - Aab) + c2o * Mab;
+            lagn[lag_T<NP>(a) * P.plane + i0] = Taa;
+            lagn[lag_T<NP>(3 + a) * P.plane + i0] = Tab;
+            lagn[lag_a(a) * P.plane + i0] = T(0.5) * (p1 - p2);
+        }
+        lagn[lag_pm<NP>() * P.plane + i0] = pm;
+        const T a0 = psi * (u[0] * grho[0] + u[1] * grho[1] + u[2] * grho[2]);
+        const T m0 = P.lg0 * mm + P.cg0 * a0;
+        const T m14 = P.lg4 * (corner - cs2 * (e2[0] + e2[1] + e2[2]) + P.two_cs2 * (cmm + psiP));
+        const T m13 = P.lg3c * xyz;
+        // sum_k h_k(c) mu_k: even part by the velocity's kind (rest, axis,
+        // corner), odd part from the first- and third-order rows
+        const T sd = (m4[0] + m4[1]) + m4[2];
+        const T base = m0 - cs2 * sd;
+        const T Ea = base + P.qa * m14, Ec = (base + sd) + P.qc * m14;
+        T Oa[3], Oc[3];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    if (cc(p, a)) {
-                        j[a] = cc(p, a) > 0 ? j[a] + gd[q] : j[a] - gd[q];
-                        e2[a] += gs[q];
-                    }
-                }
-                if (p >= 7) {
-                    corner += gs[q];
-                    xyz = cx(p) * cy(p) * cz(p) > 0 ? xyz + gd[q] : xyz - gd[q];
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        o2[k] = cc(p, k) * cc(p, (k + 1) % 3) > 0 ? o2[k] + gs[q] : o2[k] - gs[q];
-                        t3[k] = cc(p, k) > 0 ? t3[k] + gd[q] : t3[k] - gd[q];
-                    }
-                }
-            }
-            m[0] = P.lg0 * (mm + T(0.5) * a0) - a0;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                m[1 + a] = P.lg1 * (j[a] - psi * rho * u[a] + T(0.5) * Fv[a]) - Fv[a] * P.inv_cs2;
-                m[4 + a] = P.inv_n2d * (s21 * ((e2[a] - cs2 * mm) - (diag[a] + psiP) + T(0.5) * M2[a]) - M2[a]);
-                m[7 + a] = P.inv_n2o * (s22 * (o2[a] - off[a] + T(0.5) * M2[3 + a]) - M2[3 + a]);
-                m[10 + a] = P.lg3 * (t3[a] - cs2 * j[a]);
-            }
-            m[13] = P.lg3c * xyz;
-            m[14] = P.lg4 * (corner - cs2 * (e2[0] + e2[1] + e2[2]) + T(2) * cs2 * cs2 * mm + T(2) * cs2 * psiP);
+        for (int a = 0; a < 3; ++a) {
+            const T r = P.lg3 * (t3[a] - cs2 * j3[a]);   // row c_a (c_b^2 - cs2)
+            Oa[a] = m1[a] - cs2 * r;
+            Oc[a] = m1[a] + P.one_m * r;
         }
         T* gnew = pick(F.g, nxt);
-        const T c4 = T(2) * cs2 * cs2;
-        gnew[src.at(0)] = g[0] - P.w15[0] * (m[0] - cs2 * (m[4] + m[5] + m[6]) + c4 * m[14]);
-#pragma unroll
-        for (int q = 0; q < 7; ++q) {
+        gnew[i0] = src.g(0) - P.w15[0] * (base + P.q0 * m14);
+        auto put = [&](int q, T E, T O, T w) {
             const int p = pair_rep(q), pb = pair_opp(q);
-            const int x = cx(p), y = cy(p), z = cz(p);
-            T E = m[0] + (T(x * x) - cs2) * m[4] + (T(y * y) - cs2) * m[5] + (T(z * z) - cs2) * m[6];
-            if (x * y) E += T(x * y) * m[7];
-            if (y * z) E += T(y * z) * m[8];
-            if (z * x) E += T(z * x) * m[9];
-            E += (T(x * x * y * y * z * z) - cs2 * T(x * x + y * y + z * z) + c4) * m[14];
-            T O = T(0);
-            if (x) O += T(x) * m[1];
-            if (y) O += T(y) * m[2];
-            if (z) O += T(z) * m[3];
-            if (x) O += T(x) * (T(y * y) - cs2) * m[10];
-            if (y) O += T(y) * (T(z * z) - cs2) * m[11];
-            if (z) O += T(z) * (T(x * x) - cs2) * m[12];
-            if (x * y * z) O += T(x * y * z) * m[13];
-            const T wp = P.w15[p < 7 ? 1 : 2];
-            gnew[p * P.plane + src.at(p)] = g[p] - wp * (E + O);
-            gnew[pb * P.plane + src.at(pb)] = g[pb] - wp * (E - O);
-        }
-        // lagged: a (three components), T, psi m.u
+            gnew[p * P.plane + src.at(p)] = src.g(p) - w * (E + O);
+            gnew[pb * P.plane + src.at(pb)] = src.g(pb) - w * (E - O);
+        };
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int a = k, b = (k + 1) % 3;
-            lagn[lag_a(k) * P.plane + i0] = T(0.5) * psi * (mC[a] * u[b] - u[a] * mC[b]);
-        }
-#pragma unroll
-        for (int k = 0; k < 6; ++k) lagn[lag_T<NP>(k) * P.plane + i0] = Tn[k];
-        lagn[lag_pm<NP>() * P.plane + i0] =
-            psi * (rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) + mC[0] * u[0] + mC[1] * u[1] + mC[2] * u[2]);
+        for (int a = 0; a < 3; ++a) put(a, Ea + m4[a], Oa[a], P.w15[1]);
+        // corner pairs: signs (x, y, z) = (+++), (-++), (+-+), (--+)
+        const T Ep = Ec + m7[0], Em = Ec - m7[0];             // by the sign of xy
+        const T yp = m7[1] + m7[2], ym = m7[1] - m7[2];       // yz, zx
+        const T xp = Oc[0] + Oc[1], xm = Oc[0] - Oc[1];
+        const T zp = Oc[2] + m13, zm = Oc[2] - m13;           // xyz = +-1
+        put(3, Ep + yp, xp + zp, P.w15[2]);
+        put(4, Em + ym, zm - xm, P.w15[2]);
+        put(5, Em - ym, xm + zm, P.w15[2]);
+        put(6, Ep - yp, zp - xp, P.w15[2]);
     }
 }
 
 template <typename T, int NP, bool kMacro>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1) k3_update(P3<T> P, F3<T> F, int cur, int field,
-                                                      double* out) {
+__global__ void __launch_bounds__(node_threads<T>(), sizeof(T) == 4 ? 2 : 4) k3_update(P3<T> P, F3<T> F, int cur, T* out) {
     Site s;
     if (!site(P, s)) return;
-    update_node<T, NP, kMacro>(P, F, cur, field, out,
-                               GlobalSrc<T>{s, F.psi, F.C, F.mu, pick(F.g, cur), pick(F.lag, cur), P.plane});
+    update_node<T, NP, kMacro>(P, F, cur, out, GlobalSrc<T, NP>{P, F, s, pick(F.f, cur), pick(F.g, cur), pick(F.lag, cur)});
 }
 
 // ---------------------------------------------------------------------------
@@ -837,13 +849,16 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1) k3_update(P3
 //   * the mu pass for plane z+1 starts after the barrier that follows the
 //     C pass, when every thread has finished the update of plane z-1, so
 //     the slot of mu at z-2 is free.
-// With kVec (FP32, nx a multiple of 4, so that a periodic wrap maps aligned
-// quads to aligned quads) the phase populations and psi of the C region
-// arrive by 16-byte cp.async copies issued one plane ahead: the thread that
-// forms C for a quad of 4 nodes copies that quad's 7(N-1) + 1 values and
-// nothing else, so it waits for its own copies only and needs no barrier.
+// In FP32 the phase populations and psi of the C region arrive by cp.async
+// copies issued one plane ahead: by 16 bytes with kVec (nx a multiple of 4,
+// so that a periodic wrap maps aligned quads to aligned quads), else node by
+// node.  The thread that forms C for a quad of 4 nodes, or a node, copies
+// the 7(N-1) + 1 values of each and nothing else, so it waits for its own
+// copies only and needs no barrier.
 // The copies of plane z+3 fly during the mu pass and the update of plane z.
-// With kStage (kVec and N <= 3, where the staging still leaves room for two
+// (101 x 77 x 63, N = 2, where the copies are by node: 68 us a step with
+// plain loads, 62 with the copies.)
+// With kStage (FP32 and N <= 3, where the staging still leaves room for two
 // CTAs per SM) each thread also copies its own node's 15 flow populations
 // and 3N + 4 lagged values of plane z+1 (4-byte cp.async) as soon as its
 // update of plane z has read those of plane z; they fly during the C pass,
@@ -863,43 +878,78 @@ struct FusedGeom {
     static constexpr int KC = (CN + NT - 1) / NT;                   // C-region nodes per thread
     static constexpr int KM = (MN + NT - 1) / NT;                   // mu-region nodes per thread
     static constexpr int NQ = CN / 4;                               // quads of the C region
-    static constexpr int RAW = kVec ? (7 * NP + 1) * CN : 0;        // staged populations and psi
+    static constexpr bool kRaw = sizeof(T) == 4;                    // C pass fed by cp.async
+    static constexpr int RAW = kRaw ? (7 * NP + 1) * CN : 0;        // staged populations and psi
     static constexpr int NSTG = 15 + 3 * N + 4;                     // own-node g and lagged values
     static constexpr int STG = kStage ? NSTG * NT : 0;
-    static constexpr size_t smem = sizeof(T) * (5 * (NP + 1) * CN + 3 * N * MN + RAW + STG);
+    static constexpr int NMU = NP == 1 ? 1 : N;                     // mu planes (N = 2: mu_2 = -mu_1)
+    static constexpr int BASE = 5 * (NP + 1) * CN + 3 * NMU * MN + RAW + STG;
+    // psi rho (with mu, three planes) and grad psi of the own nodes (two planes)
+    // kept by the mu pass, where two CTAs with them still leave the SM's
+    // larger L1 (shared memory up to 196 of its 256 KB; each CTA costs 1 KB and
+    // the column indices more): the update reads plane a's neighbours and its
+    // own populations through L1.  At N = 3 with staged copies they do not
+    // fit: 807 us a step with them, 722 with both formed again from C and psi
+    // (208 x 192 x 160).
+    static constexpr bool kKeep = sizeof(T) * (BASE + 3 * MN + 2 * 3 * NT) + 1280 <= 196 * 1024 / 2;
+    static constexpr int NM = NMU + (kKeep ? 1 : 0);                // planes of the mu ring
+    static constexpr int GP = kKeep ? 2 * 3 * NT : 0;
+    static constexpr size_t smem = sizeof(T) * (BASE + (kKeep ? 3 * MN : 0) + GP);
     static_assert(!kVec || (sizeof(T) == 4 && NQ <= NT), "one quad per thread, FP32");
-    static_assert(!kStage || kVec, "staging needs the cp.async path");
+    static_assert(!kStage || kRaw, "staging needs the cp.async path");
 };
 
 template <typename T, int NP, int TY, bool kVec, bool kStage>
-struct SmemSrc {     // C, psi and mu from the shared-memory rings
+struct SmemSrc {     // C, psi, mu and psi rho from the shared-memory rings
     using G = FusedGeom<T, NP, TY, kVec, kStage>;
     const T* sC;     // C ring: slot k holds NP x CN values
     const T* sPs;    // psi ring: slot k holds CN values
-    const T* sMu;    // mu ring: slot k holds N x MN values
+    const T* sMu;    // mu ring: slot k holds NM x MN values
+    const T* sGp;    // (kKeep) grad psi: two slots of 3 x NT values
+    const P3<T>* P;
     const T* stg;    // (kStage) own-node g (15) and lagged planes 3.. (NT apart)
-    const T* g_;     // else the flow populations and lagged planes in global memory
+    const T* f_;     // populations and lagged planes in global memory
+    const T* g_;
     const T* lag_;
     long long plane;
     int c5[3], m3[3];  // ring slots of planes z-1, z, z+1
+    int gp2;           // grad psi's slot of plane z
     int ci, mi;        // the node in the C and mu regions
     int tid;
     int xo[3], yo[3], zo[3];  // wrapped x, y nx, z nx ny of the node and its neighbours
     __device__ int at(int p) const { return zo[cz(p) + 1] + yo[cy(p) + 1] + xo[cx(p) + 1]; }
+    __device__ T f(int i, int p) const { return __ldg(f_ + (7 * i + p) * plane + at(0)); }
     __device__ T g(int p) const {
         if constexpr (kStage) return stg[p * G::NT + tid];
-        else return g_[p * plane + at(0)];
+        else return __ldg(g_ + p * plane + at(0));
     }
     __device__ T lag(int k) const {   // k >= 3: the own node's lagged planes past a
         if constexpr (kStage) return stg[(12 + k) * G::NT + tid];
-        else return lag_[k * plane + at(0)];
+        else return __ldg(lag_ + k * plane + at(0));
     }
+    __device__ T a(int k, int p) const { return __ldg(lag_ + lag_a(k) * plane + at(p)); }
     __device__ T psi(int p) const { return sPs[c5[cz(p) + 1] * G::CN + ci + cy(p) * G::CW + cx(p)]; }
     __device__ T C(int j, int p) const {
         return sC[(c5[cz(p) + 1] * NP + j) * G::CN + ci + cy(p) * G::CW + cx(p)];
     }
     __device__ T mu(int j, int p) const {
-        return sMu[(m3[cz(p) + 1] * G::N + j) * G::MN + mi + cy(p) * G::MW + cx(p)];
+        return sMu[(m3[cz(p) + 1] * G::NM + j) * G::MN + mi + cy(p) * G::MW + cx(p)];
+    }
+    __device__ T psirho(int p) const {
+        if constexpr (G::kKeep) return mu(G::NM - 1, p);
+        else return psi_rho<T, NP>(*P, psi(p), [&](int j) { return C(j, p); });
+    }
+    __device__ void grad_psi(T gp[3]) const {
+        if constexpr (G::kKeep) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) gp[a] = sGp[(gp2 * 3 + a) * G::NT + tid];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 7; ++k) {
+                const int q = k < 4 ? k + 3 : k - 4;
+                add_pair(*P, q, psi(pair_rep(q)) - psi(pair_opp(q)), gp);
+            }
+        }
     }
 };
 
@@ -928,8 +978,9 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* sC = reinterpret_cast<T*>(smem_raw);    // 5 slots x NP x CN
     T* sPs = sC + 5 * NP * CN;                  // 5 slots x CN
-    T* sMu = sPs + 5 * CN;                      // 3 slots x N x MN
-    T* sRaw = sMu + 3 * N * MN;                 // (kVec) 7 NP + 1 planes x CN
+    T* sMu = sPs + 5 * CN;                      // 3 slots x NM x MN
+    T* sGp = sMu + 3 * G::NM * MN;              // (kKeep) 2 slots x 3 x NT
+    T* sRaw = sGp + G::GP;                      // (FP32) 7 NP + 1 planes x CN
     T* sStg = sRaw + G::RAW;                    // (kStage) NSTG x NT
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * kBX, y0 = blockIdx.y * TY;
@@ -947,8 +998,25 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
     for (int k = tid; k < G::CH; k += NT) ys[k] = wrap_index(y0 + k - 2, P.ny) * P.nx;
     __syncthreads();
 
-    // (kVec) copy the populations and psi of this thread's quad at plane z
+    // (FP32) copy the populations and psi of this thread's quad (kVec), or of
+    // its nodes one by one, at plane z
     auto issue = [&](int z, bool any) {
+        if constexpr (G::kRaw && !kVec) {
+            if (any) {
+                const long long zo = zoff(z);
+#pragma unroll
+                for (int r = 0; r < G::KC; ++r) {
+                    const int k = tid + r * NT;
+                    if (k < CN) {
+                        const long long g = zo + ys[k / CW] + xs[k % CW];
+#pragma unroll
+                        for (int q = 0; q < 7 * NP; ++q) cp_async4(sRaw + q * CN + k, fcur + q * P.plane + g);
+                        cp_async4(sRaw + 7 * NP * CN + k, F.psi + g);
+                    }
+                }
+            }
+            cp_async_commit();
+        }
         if constexpr (kVec) {
             if (any && tid < G::NQ) {
                 const int o = 4 * tid;   // quad tid: row o / CW, columns o % CW .. + 3
@@ -983,31 +1051,38 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
                         acc.w += v.w;
                     }
                     *reinterpret_cast<float4*>(c + j * CN + o) =
-                        make_float4(acc.x / psi.x, acc.y / psi.y, acc.z / psi.z, acc.w / psi.w);
+                        make_float4(acc.x * rcp(psi.x), acc.y * rcp(psi.y), acc.z * rcp(psi.z), acc.w * rcp(psi.w));
                 }
             }
         } else {
             const long long zo = zoff(z);
+            if constexpr (G::kRaw) {
+                if (steady) cp_async_wait<1>();
+                else cp_async_wait<0>();
+            }
 #pragma unroll
             for (int r = 0; r < G::KC; ++r) {
                 const int k = tid + r * NT;
                 if (k < CN) {
                     const long long i = zo + ys[k / CW] + xs[k % CW];
-                    const T psi = F.psi[i];
+                    const T psi = G::kRaw ? sRaw[7 * NP * CN + k] : F.psi[i];
                     ps[k] = psi;
+                    const T inv = rcp(psi);
 #pragma unroll
                     for (int j = 0; j < NP; ++j) {
                         T acc = T(0);
 #pragma unroll
-                        for (int p = 0; p < 7; ++p) acc += fcur[(7 * j + p) * P.plane + i];
-                        c[j * CN + k] = acc / psi;
+                        for (int p = 0; p < 7; ++p)
+                            acc += G::kRaw ? sRaw[(7 * j + p) * CN + k] : fcur[(7 * j + p) * P.plane + i];
+                        c[j * CN + k] = acc * inv;
                     }
                 }
             }
         }
     };
 
-    // mu at plane z on the mu region (as k3_mu, same summation order)
+    // mu at plane z on the mu region (as k3_mu); kKeep: psi rho there, which
+    // the update differentiates, and grad psi of the column's own nodes
     auto mu_pass = [&](int z) {
         const T* cpl[3];
         const T* ppl[3];
@@ -1016,57 +1091,29 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
             cpl[d] = sC + slot5(z - 1 + d) * NP * CN;
             ppl[d] = sPs + slot5(z - 1 + d) * CN;
         }
-        T* m = sMu + slot3(z) * N * MN;
+        T* m = sMu + slot3(z) * G::NM * MN;
+        T* gps = sGp + ((z - zb) & 1) * 3 * NT;   // two slots: the update of plane z - 2 is done
         const long long zo = zoff(z);
 #pragma unroll
         for (int r = 0; r < G::KM; ++r) {
             const int k = tid + r * NT;
             if (k < MN) {
-                const int c0 = (k / MW + 1) * CW + k % MW + 3;
-                const T psi = ppl[1][c0];
-                T C[N];
-                {
-                    T sum = T(0);
+                const int row = k / MW, col = k % MW;
+                const int c0 = (row + 1) * CW + col + 3;
+                T cth[NP], mv[N], gp[3];
+                angles<T, NP>(P, F, zo + ys[row + 1] + xs[col + 3], cth);
+                mu_node<T, NP>(
+                    P, [&](int p) { return ppl[cz(p) + 1][c0 + cy(p) * CW + cx(p)]; },
+                    [&](int j, int p) { return cpl[cz(p) + 1][j * CN + c0 + cy(p) * CW + cx(p)]; }, cth, mv, gp);
 #pragma unroll
-                    for (int j = 0; j < NP; ++j) {
-                        C[j] = cpl[1][j * CN + c0];
-                        sum += C[j];
-                    }
-                    C[NP] = T(1) - sum;
+                for (int i = 0; i < G::NMU; ++i) m[i * MN + k] = mv[i];
+                if (G::kKeep)
+                    m[(G::NM - 1) * MN + k] =
+                        psi_rho<T, NP>(P, ppl[1][c0], [&](int j) { return cpl[1][j * CN + c0]; });
+                if (G::kKeep && row >= 1 && row <= TY && col >= 1 && col <= kBX) {
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) gps[a * NT + (row - 1) * kBX + col - 1] = gp[a];
                 }
-                T L[N];
-#pragma unroll
-                for (int j = 0; j < N; ++j) L[j] = T(0);
-                T gpx = T(0), gpy = T(0), gpz = T(0);
-#pragma unroll
-                for (int p = 1; p < 15; ++p) {
-                    const int o = c0 + cy(p) * CW + cx(p);
-                    const T w = p < 7 ? P.ga : P.gc;
-                    const T psp = ppl[cz(p) + 1][o];
-                    const T wp = w * psp;
-                    if (cx(p)) gpx += T(cx(p)) * wp;
-                    if (cy(p)) gpy += T(cy(p)) * wp;
-                    if (cz(p)) gpz += T(cz(p)) * wp;
-                    const T wpsi = w * (psi + psp);
-                    T sum = T(0);
-#pragma unroll
-                    for (int j = 0; j < NP; ++j) {
-                        const T Cp = cpl[cz(p) + 1][j * CN + o];
-                        sum += Cp;
-                        L[j] += wpsi * (Cp - C[j]);
-                    }
-                    L[NP] += wpsi * ((T(1) - sum) - C[NP]);
-                }
-                T cN[N];
-#pragma unroll
-                for (int j = 0; j < NP; ++j)
-                    cN[j] = P.has_cos_field ? F.cosf[j * P.plane + zo + ys[k / MW + 1] + xs[k % MW + 3]]
-                                            : P.cos_uni[j];
-                cN[NP] = T(0);
-                T mv[N];
-                mu_from_stencil<T, NP>(P, psi, C, L, gpx, gpy, gpz, cN, mv);
-#pragma unroll
-                for (int i = 0; i < N; ++i) m[i * MN + k] = mv[i];
             }
         }
     };
@@ -1079,7 +1126,10 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
     src.sC = sC;
     src.sPs = sPs;
     src.sMu = sMu;
+    src.sGp = sGp;
+    src.P = &P;
     src.stg = sStg;
+    src.f_ = fcur;
     src.g_ = pick(F.g, cur);
     src.lag_ = pick(F.lag, cur);
     src.plane = P.plane;
@@ -1104,7 +1154,7 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
                 for (int k = 3; k < n_lag(N); ++k) cp_async4(sStg + (12 + k) * NT + tid, src.lag_ + k * P.plane + i);
             }
         }
-        if constexpr (kVec) cp_async_commit();
+        if constexpr (G::kRaw) cp_async_commit();
     };
 
     for (int z = zb - 2; z <= zb + 1; ++z) {
@@ -1130,7 +1180,8 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
                 src.m3[d] = slot3(z - 1 + d);
             }
             if constexpr (kStage) cp_async_wait<1>();   // raw(z + 3) may still fly
-            update_node<T, NP, false>(P, F, cur, 0, nullptr, src);
+            src.gp2 = (z - zb) & 1;
+            update_node<T, NP, false>(P, F, cur, nullptr, src);
         }
         stage(z + 1, z + 1 < ze);
     }
@@ -1140,7 +1191,7 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
 // initial state, staging, read-out, reduction
 // ---------------------------------------------------------------------------
 template <typename T, int NP>
-__global__ void __launch_bounds__(kThreads) k3_init(P3<T> P, F3<T> F) {
+__global__ void __launch_bounds__(node_threads<T>()) k3_init(P3<T> P, F3<T> F) {
     Site s;
     if (!site(P, s)) return;
     const long long i0 = s.self();
@@ -1286,6 +1337,7 @@ Layout layout(const ddcc3d_params* p) {
     const int N = p->nphase;
     L.plane_bytes = round256(n * e);
     L.planes = 2 * (7 * (N - 1) + 15) + 2 * n_lag(N) + 1 + (N - 1) + (N - 1) + N;
+    if (p->precision == DDCC_FP64) L.planes += 1 + kStatic;
     L.stage = round256(n * 8);
     L.partial = round256((kMassBlocks + 1) * kMaxN * 8);   // + the N-1 totals
     L.flag = 256;
@@ -1309,6 +1361,8 @@ void make_params(const ddcc3d_params* p, P3<T>& K) {
     const double wa = (d0 - d0 * d0) / 2.0, wc = d0 * d0 / 8.0, w0 = 1.0 - 3.0 * d0 + 2.0 * d0 * d0;
     K.ga = (T)(wa / cs2);
     K.gc = (T)(wc / cs2);
+    K.la = (T)(0.75 * p->width * wa / cs2);
+    K.lc = (T)(0.75 * p->width * wc / cs2);
     K.w7_0 = (T)(1.0 - 3.0 * d0);
     K.w7_1 = (T)(d0 / 2.0);
     K.w15[0] = (T)w0;
@@ -1318,29 +1372,36 @@ void make_params(const ddcc3d_params* p, P3<T>& K) {
     for (int i = 0; i < N; ++i) {
         K.rho[i] = (T)p->rho[i];
         K.nu[i] = (T)p->nu[i];
+        K.drho[i] = (T)(p->rho[i] - p->rho[N - 1]);
+        K.dnu[i] = (T)(p->nu[i] - p->nu[N - 1]);
+        double b2 = 0.0;
         K.sigN[i] = (T)p->sigma[i][N - 1];
         for (int j = 0; j < N; ++j) {
             const double s = p->sigma[i][j];
             K.beta2[i][j] = (T)(6.0 * s / p->width);
-            K.kap[i][j] = (T)(0.75 * p->width * s);
-            K.wet[i][j] = (T)(3.0 * s);
+            b2 += 6.0 * s / p->width;
+            K.sig[i][j] = (T)s;
             K.invsig[i][j] = (T)(i == j ? 0.0 : 1.0 / s);
         }
+        K.beta2s[i] = (T)b2;
     }
     for (int i = 0; i < N - 1; ++i) {
         K.eta[i] = (T)p->eta[i];
         // Eq. 17: m0 = (1/s1 - 1/2) eta_i cs2
-        K.s1f[i] = (T)(1.0 / (p->m0 / (p->eta[i] * cs2) + 0.5));
+        const double s1 = 1.0 / (p->m0 / (p->eta[i] * cs2) + 0.5);
+        K.ceta[i] = (T)(cs2 * p->eta[i]);
+        K.h1f[i] = (T)(0.5 * s1);
+        K.h2f[i] = (T)(0.25 * s1 - 0.5);
     }
     K.m0 = (T)p->m0;
-    K.inv_m0 = (T)(1.0 / p->m0);
-    K.s0f = (T)p->s_f[0];
-    K.s21f = (T)p->s_f[1];
+    K.hs21f = (T)(0.5 * p->s_f[1]);
     // D3Q15 row norms under the weights: 1, d0, d0(1-d0), d0^2,
     // d0^2(1-d0), d0^2 (cx cy cz), d0^2 w0 (last row)
     const double n2d = d0 * (1.0 - d0), n2o = d0 * d0, n3 = d0 * d0 * (1.0 - d0), n4 = d0 * d0 * w0;
     K.lg0 = (T)p->s_g[0];
     K.lg1 = (T)(p->s_g[1] / d0);
+    K.cg0 = (T)(0.5 * p->s_g[0] - 1.0);
+    K.cg1 = (T)(0.5 * p->s_g[1] / d0 - 1.0 / d0);
     K.lg3 = (T)(p->s_g[2] / n3);
     K.lg3c = (T)(p->s_g[2] / (d0 * d0));
     K.lg4 = (T)(p->s_g[3] / n4);
@@ -1359,8 +1420,12 @@ void make_params(const ddcc3d_params* p, P3<T>& K) {
     K.cP = (T)(cs2 / (1.0 - w0));
     K.kk = (T)(Kc / 2.0 - w0 / (1.0 - cs2));
     K.c2m3 = (T)(1.0 - 3.0 * cs2);
-    K.diag_den = (T)(1.0 / (cs2 * (1.0 - cs2)));
-    K.off_den = (T)(1.0 / (cs2 * cs2));
+    K.half_K = (T)(0.5 * Kc);
+    K.two_cs2 = (T)(2.0 * cs2);
+    K.one_m = (T)(1.0 - cs2);
+    K.q0 = (T)(2.0 * cs2 * cs2);
+    K.qa = (T)(2.0 * cs2 * cs2 - cs2);
+    K.qc = (T)(1.0 - 3.0 * cs2 + 2.0 * cs2 * cs2);
     for (int a = 0; a < 3; ++a) K.body[a] = (T)p->body_force[a];
 }
 
@@ -1377,6 +1442,10 @@ void carve(const ddcc3d_params* p, char* ws, F3<T>& F) {
     F.cosf = take(N - 1);
     F.C = take(N - 1);
     F.mu = take(N);
+    if (sizeof(T) == 8) {
+        F.chi = take(1);
+        F.st = take(kStatic);
+    }
     F.stage = (double*)c;
     c += L.stage;
     F.partial = (double*)c;
@@ -1400,6 +1469,7 @@ struct ddcc3d_handle {
     double* dev_mass;
     int fused;        // one k3_fused launch per step (else the three kernels)
     int cmu_valid;    // F.C and F.mu hold the current state's C and mu (cleared by a step)
+    int macro_valid;  // the other copy's g planes 0..4 hold its rho, u and P (cleared by a step)
     int nchunk;       // z chunks of the fused step's grid
     int profiling;
     std::vector<cudaEvent_t> events;
@@ -1426,15 +1496,22 @@ int prof_end(ddcc3d_handle* h) {
     return cudaEventRecord(h->events[2 * i + 1], h->stream) == cudaSuccess ? DDCC_OK : DDCC_ERR_CUDA;
 }
 
+template <typename T>
 dim3 grid3(const ddcc3d_params& p) {
+    if (sizeof(T) == 8) {
+        const long long n = (long long)p.nx * p.ny * p.nz;
+        return dim3((unsigned)((n + kLinear - 1) / kLinear));
+    }
     return dim3((p.nx + kBX - 1) / kBX, (p.ny + kBY - 1) / kBY, (p.nz + kBZ - 1) / kBZ);
 }
+template <typename T>
+dim3 block3() { return sizeof(T) == 8 ? dim3(kLinear) : dim3(kBX, kBY, kBZ); }
 
 int launched() { return cudaGetLastError() == cudaSuccess ? DDCC_OK : DDCC_ERR_CUDA; }
 
 template <typename T, int NP>
 int order_mu(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F, bool order) {
-    const dim3 grid = grid3(h->prm), block(kBX, kBY, kBZ);
+    const dim3 grid = grid3<T>(h->prm), block = block3<T>();
     int rc;
     if (order) {
         if ((rc = prof_begin(h, 0))) return rc;
@@ -1459,12 +1536,12 @@ int order_mu(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F, bool order) {
 // Shared memory of the fused step and its z chunks: the count of chunks n
 // minimises (waves of CTAs) x (planes a CTA forms C for), i.e.
 // ceil(columns n / resident CTAs) x (ceil(nz / n) + 3).
-template <int NP, bool kVec>
-constexpr bool fused_stage() { return kVec && NP <= 2; }
+template <typename T, int NP>
+constexpr bool fused_stage() { return sizeof(T) == 4 && NP <= 2; }
 
 template <typename T, int NP, bool kVec>
 int fused_setup_v(ddcc3d_handle* h) {
-    constexpr bool kS = fused_stage<NP, kVec>();
+    constexpr bool kS = fused_stage<T, NP>();
     using G = FusedGeom<T, NP, kFusedTY, kVec, kS>;
     if (cudaFuncSetAttribute(k3_fused<T, NP, kFusedTY, kVec, kS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)G::smem) != cudaSuccess)
@@ -1504,7 +1581,7 @@ int fused_setup(ddcc3d_handle* h) {
 
 template <typename T, int NP, bool kVec>
 int fused_launch(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F) {
-    constexpr bool kS = fused_stage<NP, kVec>();
+    constexpr bool kS = fused_stage<T, NP>();
     using G = FusedGeom<T, NP, kFusedTY, kVec, kS>;
     const dim3 gf((h->prm.nx + kBX - 1) / kBX, (h->prm.ny + kFusedTY - 1) / kFusedTY, h->nchunk);
     k3_fused<T, NP, kFusedTY, kVec, kS><<<gf, G::NT, G::smem, h->stream>>>(K, F, h->cur, h->nchunk);
@@ -1513,7 +1590,7 @@ int fused_launch(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F) {
 
 template <typename T, int NP>
 int step_n(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F, int64_t n) {
-    const dim3 grid = grid3(h->prm), block(kBX, kBY, kBZ);
+    const dim3 grid = grid3<T>(h->prm), block = block3<T>();
     if (h->fused) {
         for (int64_t s = 0; s < n; ++s) {
             int rc;
@@ -1533,7 +1610,7 @@ int step_n(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F, int64_t n) {
         int rc = order_mu<T, NP>(h, K, F, true);
         if (rc) return rc;
         if ((rc = prof_begin(h, 2))) return rc;
-        k3_update<T, NP, false><<<grid, block, 0, h->stream>>>(K, F, h->cur, 0, nullptr);
+        k3_update<T, NP, false><<<grid, block, 0, h->stream>>>(K, F, h->cur, nullptr);
         if ((rc = launched()) || (rc = prof_end(h))) return rc;
         h->cur ^= 1;
         ++h->steps;
@@ -1543,16 +1620,20 @@ int step_n(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F, int64_t n) {
 
 template <typename T, int NP>
 int init_n(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F) {
-    const dim3 grid = grid3(h->prm), block(kBX, kBY, kBZ);
-    int rc = order_mu<T, NP>(h, K, F, false);
-    if (rc) return rc;
+    const dim3 grid = grid3<T>(h->prm), block = block3<T>();
+    int rc;
+    if constexpr (sizeof(T) == 8) {
+        k3_static<T><<<grid, block, 0, h->stream>>>(K, F);
+        if ((rc = launched())) return rc;
+    }
+    if ((rc = order_mu<T, NP>(h, K, F, false))) return rc;
     k3_init<T, NP><<<grid, block, 0, h->stream>>>(K, F);
     return launched();
 }
 
 template <typename T, int NP>
 int read_n(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F, int field, double* host_out) {
-    const dim3 grid = grid3(h->prm), block(kBX, kBY, kBZ);
+    const dim3 grid = grid3<T>(h->prm), block = block3<T>();
     const int N = NP + 1;
     const long long n = K.nxy * K.nz;
     int rc;
@@ -1571,7 +1652,17 @@ int read_n(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F, int field, double* 
         k3_to_double<T><<<cb, ct, 0, h->stream>>>(F.psi, F.stage, n);
     } else if (field == DDCC_FIELD_RHO || field == DDCC_FIELD_UX || field == DDCC_FIELD_UY ||
                field == DDCC_FIELD_UZ || field == DDCC_FIELD_P) {
-        k3_update<T, NP, true><<<grid, block, 0, h->stream>>>(K, F, h->cur, field, F.stage);
+        // rho, u and P of a state are formed together on the first read, in
+        // planes of the other population copy, which the next step overwrites
+        T* out = F.g[h->cur ^ 1];
+        if (!h->macro_valid) {
+            k3_update<T, NP, true><<<grid, block, 0, h->stream>>>(K, F, h->cur, out);
+            if ((rc = launched())) return rc;
+            h->macro_valid = 1;
+        }
+        const int k = field == DDCC_FIELD_RHO ? 0 : field == DDCC_FIELD_UX ? 1 : field == DDCC_FIELD_UY ? 2
+                      : field == DDCC_FIELD_UZ ? 3 : 4;
+        k3_to_double<T><<<cb, ct, 0, h->stream>>>(out + k * K.plane, F.stage, n);
     } else {
         return DDCC_ERR_PARAM;
     }
@@ -1700,6 +1791,7 @@ int ddcc3d_create(const ddcc3d_params* params, void* dev_workspace, size_t bytes
 int ddcc3d_step(ddcc3d_handle* h, int64_t nsteps) {
     if (!h || nsteps < 0) return DDCC_ERR_PARAM;
     h->cmu_valid = 0;
+    h->macro_valid = 0;
     const int np = h->prm.nphase - 1;
     if (h->prm.precision == DDCC_FP64) {
         if (np == 1) return step_n<double, 1>(h, h->kd, h->fd, nsteps);

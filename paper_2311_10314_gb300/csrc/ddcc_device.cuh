@@ -106,27 +106,21 @@ __device__ __forceinline__ void grad9(const KParams<T>& P, const A& chi, T& gx, 
 // g'(1 - c) = -g'(c) and sum_j C_j = 1: they vanish for two phases, are
 // -g'(C_k) of the third for three, and for four three pairs give the other
 // three.  For two phases mu_2 = -mu_1.
-// agp3 = 3 |grad psi| (3 with several solids) and inv_p0 = 1 / psi at the node.
-template <typename T, int NP, class CA, class PA>
-__device__ __forceinline__ void chem_pot_with(const KParams<T>& P, const CA& Cx, const PA& Ps,
-                                              const T* cth, T agp3, T inv_p0, T mu[NP]) {
-    const T p0 = Ps(0, 0);
-    const T pE = Ps(0, 1), pW = Ps(0, -1), pN = Ps(1, 0), pS = Ps(-1, 0);
-    const T pNE = Ps(1, 1), pNW = Ps(1, -1), pSW = Ps(-1, -1), pSE = Ps(-1, 1);
+// mu_i of one node from the fractions and V_j = (3 eps / 4) div(psi grad C_j)
+// of the N-1 evolved phases; agp3 = 3 |grad psi| (3 with several solids),
+// inv_p0 = 1 / psi.  Any lattice: PT holds the model's constants.
+template <typename T, int NP, class PT>
+__device__ __forceinline__ void mu_of(const PT& P, const T* C, const T* Lk, const T* cth, T agp3, T inv_p0, T mu[NP]) {
     T Cv[NP], V[NP];
-    T sumC = T(0), sumL = T(0);
+    T sumC = C[0], sumL = Lk[0];
 #pragma unroll
     for (int j = 0; j < NP - 1; ++j) {
-        const T c0 = Cx(j, 0, 0);
-        // (3 eps / 4) div(psi grad C), div = sum_p w_p (psi + psi_p)(C_p - C) / cs2
-        const T l = P.lk1 * ((p0 + pE) * (Cx(j, 0, 1) - c0) + (p0 + pW) * (Cx(j, 0, -1) - c0) +
-                             (p0 + pN) * (Cx(j, 1, 0) - c0) + (p0 + pS) * (Cx(j, -1, 0) - c0)) +
-                    P.lk2 * ((p0 + pNE) * (Cx(j, 1, 1) - c0) + (p0 + pNW) * (Cx(j, 1, -1) - c0) +
-                             (p0 + pSW) * (Cx(j, -1, -1) - c0) + (p0 + pSE) * (Cx(j, -1, 1) - c0));
-        Cv[j] = c0;
-        V[j] = l;
-        sumC = j == 0 ? c0 : sumC + c0;
-        sumL = j == 0 ? l : sumL + l;
+        Cv[j] = C[j];
+        V[j] = Lk[j];
+        if (j > 0) {
+            sumC += C[j];
+            sumL += Lk[j];
+        }
     }
     Cv[NP - 1] = T(1) - sumC;
     V[NP - 1] = -sumL;
@@ -183,6 +177,28 @@ __device__ __forceinline__ void chem_pot_with(const KParams<T>& P, const CA& Cx,
             mu[i] = bulk + v * inv_p0;
         }
     }
+}
+
+// agp3 = 3 |grad psi| (3 with several solids) and inv_p0 = 1 / psi at the node.
+template <typename T, int NP, class CA, class PA>
+__device__ __forceinline__ void chem_pot_with(const KParams<T>& P, const CA& Cx, const PA& Ps,
+                                              const T* cth, T agp3, T inv_p0, T mu[NP]) {
+    const T p0 = Ps(0, 0);
+    const T pE = Ps(0, 1), pW = Ps(0, -1), pN = Ps(1, 0), pS = Ps(-1, 0);
+    const T pNE = Ps(1, 1), pNW = Ps(1, -1), pSW = Ps(-1, -1), pSE = Ps(-1, 1);
+    T Cv[NP - 1], V[NP - 1];
+#pragma unroll
+    for (int j = 0; j < NP - 1; ++j) {
+        const T c0 = Cx(j, 0, 0);
+        // (3 eps / 4) div(psi grad C), div = sum_p w_p (psi + psi_p)(C_p - C) / cs2
+        const T l = P.lk1 * ((p0 + pE) * (Cx(j, 0, 1) - c0) + (p0 + pW) * (Cx(j, 0, -1) - c0) +
+                             (p0 + pN) * (Cx(j, 1, 0) - c0) + (p0 + pS) * (Cx(j, -1, 0) - c0)) +
+                    P.lk2 * ((p0 + pNE) * (Cx(j, 1, 1) - c0) + (p0 + pNW) * (Cx(j, 1, -1) - c0) +
+                             (p0 + pSW) * (Cx(j, -1, -1) - c0) + (p0 + pSE) * (Cx(j, -1, 1) - c0));
+        Cv[j] = c0;
+        V[j] = l;
+    }
+    mu_of<T, NP>(P, Cv, V, cth, agp3, inv_p0, mu);
 }
 
 template <typename T, int NP, class CA, class PA>

@@ -11,6 +11,7 @@ import torch
 
 import workloads as W
 from oracle import Oracle
+from oracle.ddcc_oracle3d import Oracle3D
 
 pytestmark = pytest.mark.gpu
 
@@ -76,3 +77,27 @@ def test_fp64_step_and_ghost_ring(D, nx, ny, N, py, field):
                          org + 9 * N * plane - pitch - 1).cpu().numpy()
     wrap = np.pad(a[1:-1, 1:-1], ((0, 0), (1, 1)), mode="wrap")
     assert np.array_equal(a, np.pad(wrap, ((1, 1), (0, 0)), mode="wrap" if py else "symmetric"))
+
+
+@pytest.mark.parametrize("precision,path", [(1, "fused"), (1, "split"), (0, "split"), (0, "fused")])
+@pytest.mark.parametrize("nx,ny,nz,N,field", [
+    (33, 9, 12, 2, True),     # copies node by node, one column and row over a block
+    (31, 8, 5, 3, False),
+    (64, 17, 4, 3, True),     # copies by quads, fewest planes a chunk can have
+    (36, 10, 9, 4, False),    # no staged node values
+])
+def test_3d_paths_on_ragged_boxes(D, nx, ny, nz, N, field, precision, path):
+    """The fused step with both kinds of copies and with and without staged
+    values, and the three kernels, in both precisions."""
+    pb = W.random_problem_3d(nx, ny, nz, N, seed=nx + N, theta_field=field, width=5.0)
+    o = Oracle3D(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field)
+    o.step(5)
+    ref = {k: v.numpy() for k, v in o.macroscopic().items()}
+    sim = D.Sim3D(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field, precision=precision, path=path)
+    sim.step(5)
+    got = sim.fields()
+    sim.close()
+    fl = pb.psi >= 0.01
+    tc, tu = (1e-10, 1e-10) if precision == D.DDCC_FP64 else (2e-5, 1e-6)
+    assert np.abs(ref["C"] - got["C"])[:, fl].max() <= tc
+    assert max(np.abs(ref[k] - got[k])[fl].max() for k in ("ux", "uy", "uz")) <= tu
