@@ -540,6 +540,19 @@ Step64Args args64(const Fields<double>& f, const double* pop_in, const double* l
     return Step64Args{pop_in, lag_in, pop_out, lag_out, nullptr, f.psi, f.cosf, f.st64, f.C, f.chi, f.mu};
 }
 
+// The rings that the next step's halo boxes read, where the fused kernel has
+// not written them: its 64 x 4 tiles do not, and in three rows a node has two
+// copies along y.
+template <typename T>
+int fused_rings(ddcc_handle* h, T* pop, T* lag) {
+    if (fused_writes_rings(fused_x(h->tile_wide)) && h->prm.ny >= 4) return DDCC_OK;
+    int st;
+    if ((st = prof_begin(h, 3))) return st;
+    DDCC_CU(launch_fill_ghosts2<T>(GhostRing<T>{pop, 9 * (h->prm.nphase - 1), kFusedGhostF, kFusedGhostF},
+                                   GhostRing<T>{lag, 1, kFusedGhostA, kFusedGhostA}, kp_of<T>(h), h->stream));
+    return prof_end(h);
+}
+
 template <typename T>
 int step_plain(ddcc_handle* h, int64_t n) {
     KParams<T>& k = kp_of<T>(h);
@@ -572,12 +585,7 @@ int step_plain(ddcc_handle* h, int64_t n) {
             if ((st = prof_end(h))) return st;
             if (h->prm.flags & DDCC_FLAG_OPEN_X)
                 DDCC_CU(launch_open_bc<T>(k, f.f[1 - c], f.lag[1 - c], f.psi, f.inflow, h->stream));
-            // the next step's halo boxes read the ghost frames of f and a
-            if ((st = prof_begin(h, 3))) return st;
-            DDCC_CU(launch_fill_ghosts2<T>(GhostRing<T>{f.f[1 - c], 9 * (N - 1), kFusedGhostF, kFusedGhostF},
-                                           GhostRing<T>{f.lag[1 - c], 1, kFusedGhostA, kFusedGhostA}, k,
-                                           h->stream));
-            if ((st = prof_end(h))) return st;
+            if ((st = fused_rings<T>(h, f.f[1 - c], f.lag[1 - c]))) return st;
         } else {
             if ((st = prof_begin(h, 0))) return st;
             DDCC_CU(launch_order_param<T>(k, f, c, h->stream));
@@ -810,7 +818,6 @@ int step_between_t(ddcc_handle* h, const void* state_in, void* state_out) {
     if (h->use_sweep || h->use_tile_tma < 2 || (h->prm.flags & DDCC_FLAG_OPEN_X)) return DDCC_ERR_UNSUPPORTED;
     KParams<T>& k = kp_of<T>(h);
     Fields<T>& f = fd_of<T>(h);
-    const int N = h->prm.nphase;
     size_t pb, lb;
     state_payload(h, &pb, &lb);
     const T* in_pop = reinterpret_cast<const T*>(static_cast<const char*>(state_in) + kAlign);
@@ -826,8 +833,7 @@ int step_between_t(ddcc_handle* h, const void* state_in, void* state_out) {
         if (!encode_fused<T>(&m, in_pop, in_lag, k, h->tile_wide)) return DDCC_ERR_CUDA;
         TileTmaArgs<T> a{&m.fh, &m.g, &m.lag, &h->tt_c, &h->tt_st, &m.a, &k, out_pop, out_lag, f.flag, h->tile_wide};
         DDCC_CU(launch_collide_fused<T>(a, h->stream));
-        DDCC_CU(launch_fill_ghosts2<T>(GhostRing<T>{out_pop, 9 * (N - 1), kFusedGhostF, kFusedGhostF},
-                                       GhostRing<T>{out_lag, 1, kFusedGhostA, kFusedGhostA}, k, h->stream));
+        return fused_rings<T>(h, out_pop, out_lag);
     }
     return DDCC_OK;
 }

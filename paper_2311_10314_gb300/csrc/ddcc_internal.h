@@ -132,6 +132,8 @@ struct SweepArgs {
 // lagged planes and stencil halos arrive by tensor copies.
 constexpr int kTileHaloW = kTileX + 8;   // halo box: tile + 4 columns a side
 constexpr int kWideX = 64, kWideY = 4;   // the fused kernel's other tile (fused_tile_wide)
+// Whether the fused kernel with tiles this wide writes the ghost rings itself.
+constexpr bool fused_writes_rings(int tile_x) { return tile_x == kTileX; }
 template <typename T>
 struct TileTmaArgs {
     const CUtensorMap* tm_pop;   // box {32, 8, 9N} over the input population planes, or (fused

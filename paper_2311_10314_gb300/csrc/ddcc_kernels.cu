@@ -163,6 +163,72 @@ __device__ __forceinline__ int opposite(int p) {
     return p == 0 ? 0 : (p <= 4 ? ((p + 1) & 3) + 1 : ((p - 3) & 3) + 5);
 }
 
+// Push targets of node (x, y) at offset o.
+template <typename T, int NP>
+__device__ __forceinline__ void tile_targets(const KParams<T>& P, int x, int y, long long o, TileSink<T, NP>& sink) {
+#pragma unroll
+    for (int p = 0; p < 9; ++p) {
+        int tx = x + kCx[p], ty = y + kCy[p];
+        bool bounce = false;
+        if (tx < 0 || tx >= P.nx) {
+            if (P.px) tx = tx < 0 ? tx + P.nx : tx - P.nx;
+            else bounce = true;
+        }
+        if (ty < 0 || ty >= P.ny) {
+            if (P.py) ty = ty < 0 ? ty + P.ny : ty - P.ny;
+            else bounce = true;
+        }
+        sink.tgt[p] = bounce ? o : P.org + (long long)ty * P.pitch + tx;
+        sink.tdir[p] = bounce ? opposite(p) : p;
+    }
+}
+
+// Step from coordinate v to its copy in the 2-node ghost ring (0: none):
+// periodic v -> v +- n, mirror -1 - v or 2 n - 1 - v.  One copy at most along
+// an axis of four nodes or more.
+__device__ __forceinline__ int ring2_step(int v, int n, int periodic) {
+    if (v < 2) return periodic ? n : -1 - 2 * v;
+    if (v >= n - 2) return periodic ? -n : 2 * (n - v) - 1;
+    return 0;
+}
+
+// Push sink of the edge tiles of the fused kernel's 32 x 8 form: wrap and
+// bounce-back as TileSink, and every phase population and the lagged plane a
+// are also written to the copies of their node in the 2-node ghost ring that
+// the next step's halo boxes read.  It takes a launch off a small grid's step
+// (256 x 256, N = 3: 10.3 -> 9.1 us); the 64 x 4 form, for states beyond L2,
+// keeps the launch (4096 x 4096, N = 4: 1177 us a step with it, 1196 with
+// this sink, whose registers also weigh on the inner tiles).
+template <typename T, int NP>
+struct EdgeSink {
+    long long tgt[9];              // target, plane of the direction included
+    unsigned bounced;              // bit p: population p comes back
+    int dx[3], dy[3];              // ring steps of columns x-1, x, x+1 (rows: y) after wrapping
+    long long o, plane;
+    int pitch;
+    T* __restrict__ pop;
+    T* __restrict__ lag;
+    __device__ void copies(T* q, int sx, int sy, T v) const {
+        const long long ry = (long long)sy * pitch;
+        if (sx) q[sx] = v;
+        if (sy) q[ry] = v;
+        if (sx && sy) q[ry + sx] = v;
+    }
+    __device__ void f_out(int i, int p, T v) {
+        T* q = pop + (long long)(9 * i) * plane + tgt[p];
+        *q = v;
+        const bool b = (bounced >> p) & 1;
+        copies(q, b ? dx[1] : dx[cxp(p) + 1], b ? dy[1] : dy[cyp(p) + 1], v);
+    }
+    __device__ void g_out(int p, T v) { pop[(long long)(9 * (NP - 1)) * plane + tgt[p]] = v; }
+    __device__ void lag_out(int k, T v) {
+        T* q = lag + k * plane + o;
+        *q = v;
+        if (k == 0) copies(q, dx[1], dy[1], v);
+    }
+    __device__ void macro(const T*, T, T, T, T, const T*) {}
+};
+
 // MODE 0: full step (collide + push-stream + lagged fields).
 // MODE 1: macroscopic read-out of the current state (no state change).
 template <typename T, int NP, int MODE>
@@ -196,21 +262,7 @@ __global__ void __launch_bounds__(NT) k_step(KParams<T> P, Fields<T> F, int cur)
     sink.lout = lag_out;
     sink.macro_out = F.macro;
     if (MODE == 0) {
-#pragma unroll
-        for (int p = 0; p < 9; ++p) {
-            int tx = x + kCx[p], ty = y + kCy[p];
-            bool bounce = false;
-            if (tx < 0 || tx >= P.nx) {
-                if (P.px) tx = tx < 0 ? tx + P.nx : tx - P.nx;
-                else bounce = true;
-            }
-            if (ty < 0 || ty >= P.ny) {
-                if (P.py) ty = ty < 0 ? ty + P.ny : ty - P.ny;
-                else bounce = true;
-            }
-            sink.tgt[p] = bounce ? o : P.org + (long long)ty * P.pitch + tx;
-            sink.tdir[p] = bounce ? opposite(p) : p;
-        }
+        tile_targets(P, x, y, o, sink);
     }
     dev::node_update<T, NP, MODE>(P, acc, sink);
 }
@@ -344,21 +396,7 @@ __global__ void __launch_bounds__(NT, 2)
     sink.gout = pop_out + (long long)9 * (NP - 1) * P.plane;
     sink.lout = lag_out;
     sink.macro_out = nullptr;
-#pragma unroll
-    for (int p = 0; p < 9; ++p) {
-        int tx = x + kCx[p], ty = y + kCy[p];
-        bool bounce = false;
-        if (tx < 0 || tx >= P.nx) {
-            if (P.px) tx = tx < 0 ? tx + P.nx : tx - P.nx;
-            else bounce = true;
-        }
-        if (ty < 0 || ty >= P.ny) {
-            if (P.py) ty = ty < 0 ? ty + P.ny : ty - P.ny;
-            else bounce = true;
-        }
-        sink.tgt[p] = bounce ? o : P.org + (long long)ty * P.pitch + tx;
-        sink.tdir[p] = bounce ? opposite(p) : p;
-    }
+    tile_targets(P, x, y, o, sink);
     dev::node_update<T, NP, 0>(P, acc, sink);
 }
 
@@ -537,34 +575,52 @@ __global__ void __launch_bounds__(TX * TY, 2)
     if (x >= P.nx || y >= P.ny) return;
     const long long o = P.org + (long long)y * P.pitch + x;
     FusedAcc<T, NP, TF, TX, TY> acc{P, sm, (int)threadIdx.x, (int)threadIdx.y};
-    // most tiles push only into the domain's interior: fixed neighbour
-    // offsets, no wrap or bounce-back, 32-bit offsets (a block-uniform branch)
-    if (off32 && x0 >= 1 && y0 >= 1 && x0 + TX < P.nx && y0 + TY < P.ny) {
+    // most tiles push only into the domain's interior, and (kRings) only to
+    // nodes without a copy in the 2-node ghost ring: fixed neighbour offsets,
+    // no wrap or bounce-back, 32-bit offsets (a block-uniform branch)
+    constexpr bool kRings = fused_writes_rings(TX);
+    constexpr int kIn = kRings ? 3 : 1;
+    if (off32 && x0 >= kIn && y0 >= kIn && x0 + TX + kIn <= P.nx && y0 + TY + kIn <= P.ny) {
         InnerSink<T, NP> in{pop_out + o, lag_out + o, (int)P.plane, P.pitch};
         dev::node_update<T, NP, 0>(P, acc, in);
         return;
     }
-    TileSink<T, NP> sink;
+    if constexpr (!kRings) {
+        TileSink<T, NP> sink;
+        sink.o = o;
+        sink.plane = P.plane;
+        sink.fout = pop_out;
+        sink.gout = pop_out + (long long)9 * (NP - 1) * P.plane;
+        sink.lout = lag_out;
+        sink.macro_out = nullptr;
+        tile_targets(P, x, y, o, sink);
+        dev::node_update<T, NP, 0>(P, acc, sink);
+        return;
+    }
+    EdgeSink<T, NP> sink;
     sink.o = o;
     sink.plane = P.plane;
-    sink.fout = pop_out;
-    sink.gout = pop_out + (long long)9 * (NP - 1) * P.plane;
-    sink.lout = lag_out;
-    sink.macro_out = nullptr;
+    sink.pitch = P.pitch;
+    sink.pop = pop_out;
+    sink.lag = lag_out;
+    sink.bounced = 0;
+    int tx[3], ty[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        tx[d] = x + d - 1;
+        ty[d] = y + d - 1;
+        if (P.px) tx[d] = tx[d] < 0 ? tx[d] + P.nx : tx[d] >= P.nx ? tx[d] - P.nx : tx[d];
+        if (P.py) ty[d] = ty[d] < 0 ? ty[d] + P.ny : ty[d] >= P.ny ? ty[d] - P.ny : ty[d];
+        sink.dx[d] = ring2_step(tx[d], P.nx, P.px);
+        sink.dy[d] = ring2_step(ty[d], P.ny, P.py);
+    }
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
-        int tx = x + kCx[p], ty = y + kCy[p];
-        bool bounce = false;
-        if (tx < 0 || tx >= P.nx) {
-            if (P.px) tx = tx < 0 ? tx + P.nx : tx - P.nx;
-            else bounce = true;
-        }
-        if (ty < 0 || ty >= P.ny) {
-            if (P.py) ty = ty < 0 ? ty + P.ny : ty - P.ny;
-            else bounce = true;
-        }
-        sink.tgt[p] = bounce ? o : P.org + (long long)ty * P.pitch + tx;
-        sink.tdir[p] = bounce ? opposite(p) : p;
+        const int X = tx[cxp(p) + 1], Y = ty[cyp(p) + 1];
+        const bool bounce = X < 0 || X >= P.nx || Y < 0 || Y >= P.ny;
+        sink.bounced |= (unsigned)bounce << p;
+        sink.tgt[p] = bounce ? opposite(p) * P.plane + o
+                             : p * P.plane + P.org + (long long)Y * P.pitch + X;
     }
     dev::node_update<T, NP, 0>(P, acc, sink);
 }
@@ -761,69 +817,84 @@ __global__ void k_fill_ghosts(GhostRing<T> g0, GhostRing<T> g1, KParams<T> P) {
 
 // Open x ends: equilibrium at (u_in(y), 0) with mu = 0 and m^C = 0 (Eqs. 3.5,
 // 3.8); C = C_in at the inlet, the neighbour column's at the outlet; psi P
-// from the neighbour column by Eq. 19 without its velocity terms.
+// from the neighbour column by Eq. 19 without its velocity terms.  A thread
+// has one population set (phase i, or the flow and the remaining lagged
+// planes) of one end node, in blocks of one warp: the launch is a chain of
+// dependent loads and is bound by their latency.  Phase populations and plane
+// a go to the node's copies in the 2-node ghost ring too.
+constexpr int kOpenThreads = 32;
 template <typename T, int NP>
-__global__ void k_open_bc(KParams<T> P, T* __restrict__ pop, T* __restrict__ lag, const T* __restrict__ psi,
-                          const T* __restrict__ inflow) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 2 * P.ny) return;
-    const int side = idx / P.ny, y = idx - side * P.ny;
+__global__ void __launch_bounds__(kOpenThreads) k_open_bc(KParams<T> P, T* __restrict__ pop, T* __restrict__ lag,
+                                                          const T* __restrict__ psi, const T* __restrict__ inflow) {
+    const int idx = blockIdx.x * kOpenThreads + threadIdx.x;
+    const int end = idx % (2 * P.ny), set = idx / (2 * P.ny);
+    if (set >= NP) return;
+    const int side = end / P.ny, y = end - side * P.ny;
     const int xb = side ? P.nx - 1 : 0, xn = side ? P.nx - 2 : 1;
     const long long pl = P.plane;
     const long long ob = P.org + (long long)y * P.pitch + xb, on = P.org + (long long)y * P.pitch + xn;
+    const int sx = ring2_step(xb, P.nx, 0);
+    const long long sy = (long long)ring2_step(y, P.ny, P.py) * P.pitch;
+    auto put = [&](T* q, T v) {
+        q[ob] = v;
+        q[ob + sx] = v;
+        if (sy) {
+            q[ob + sy] = v;
+            q[ob + sy + sx] = v;
+        }
+    };
     const T psib = psi[ob], psin = psi[on];
     const T u = inflow[y];
     const T cs2 = P.cs2;
-    T Cb[NP];
+    auto fraction = [&](int j) {
+        if (side == 0) return inflow[(1 + j) * P.ny + y];
+        T v[9], sf = T(0);
+#pragma unroll
+        for (int p = 0; p < 9; ++p) v[p] = pop[(9 * j + p) * pl + on];
+#pragma unroll
+        for (int p = 0; p < 9; ++p) sf += v[p];
+        return sf / psin;
+    };
+    if (set < NP - 1) {
+        // phase: f_0 = psi C, f_p = w_p psi C c_p.u / cs2
+        const T psiC = psib * fraction(set);
+        const T fa = P.w9[1] * psiC * u / cs2, fd = P.w9[2] * psiC * u / cs2;
+#pragma unroll
+        for (int p = 0; p < 9; ++p) {
+            const T m = p <= 4 ? fa : fd;
+            put(pop + (9 * set + p) * pl, p == 0 ? psiC : cxp(p) > 0 ? m : cxp(p) < 0 ? -m : T(0));
+        }
+        lag[(1 + 2 * set) * pl + ob] = psiC * u;
+        lag[(2 + 2 * set) * pl + ob] = T(0);
+        return;
+    }
+    T* g = pop + (long long)9 * (NP - 1) * pl;
+    T gn[9], sum_g = T(0);
+#pragma unroll
+    for (int p = 1; p < 9; ++p) gn[p] = g[p * pl + on];
+    const T pmn = lag[(2 * NP + 2) * pl + on];
     T rho = T(0), sC = T(0);
 #pragma unroll
     for (int j = 0; j < NP - 1; ++j) {
-        T c;
-        if (side == 0) {
-            c = inflow[(1 + j) * P.ny + y];
-        } else {
-            T sf = T(0);
-#pragma unroll
-            for (int p = 0; p < 9; ++p) sf += pop[(9 * j + p) * pl + on];
-            c = sf / psin;
-        }
-        Cb[j] = c;
+        const T c = fraction(j);
         sC += c;
         rho += c * P.rho[j];
     }
     rho += (T(1) - sC) * P.rho[NP - 1];
-    T* g = pop + (long long)9 * (NP - 1) * pl;
-    T sum_g = T(0);
 #pragma unroll
-    for (int p = 1; p < 9; ++p) sum_g += g[p * pl + on];
-    const T psiP = psib * (P.cP * (sum_g - P.Kh * lag[(2 * NP + 2) * pl + on]) / psin);
-    // phases: f_0 = psi C, f_p = w_p psi C c_p.u / cs2
-#pragma unroll
-    for (int j = 0; j < NP - 1; ++j) {
-        const T psiC = psib * Cb[j];
-#pragma unroll
-        for (int p = 0; p < 9; ++p) {
-            const T wp = P.w1d[kCx[p] + 1] * P.w1d[kCy[p] + 1];
-            pop[(9 * j + p) * pl + ob] = p == 0 ? psiC : wp * psiC * (T(kCx[p]) * u) / cs2;
-        }
-    }
+    for (int p = 1; p < 9; ++p) sum_g += gn[p];
+    const T psiP = psib * (P.cP * (sum_g - P.Kh * pmn) / psin);
     // flow: g_p = w_p psi P / cs2 + s_p (g_0 stored less rho0), s_p of the
     // resting-solid-free equilibrium with m^C = 0
     const T Axx = psib * rho * u * u;
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
-        const T wp = P.w1d[kCx[p] + 1] * P.w1d[kCy[p] + 1];
-        const T cx = T(kCx[p]), cy = T(kCy[p]);
+        const T wp = P.w9[p == 0 ? 0 : p <= 4 ? 1 : 2];
+        const T cx = T(cxp(p));
         const T sp = wp * (cx * psib * rho * u / cs2 + Axx * (cx * cx - cs2) / (cs2 - cs2 * cs2));
-        (void)cy;
         g[p * pl + ob] = (p == 0 ? (wp - T(1)) : wp) * psiP / cs2 + sp;
     }
-    lag[ob] = T(0);
-#pragma unroll
-    for (int j = 0; j < NP - 1; ++j) {
-        lag[(1 + 2 * j) * pl + ob] = psib * Cb[j] * u;
-        lag[(2 + 2 * j) * pl + ob] = T(0);
-    }
+    put(lag, T(0));
     lag[(2 * NP - 1) * pl + ob] = T(0);
     lag[(2 * NP) * pl + ob] = T(0);
     lag[(2 * NP + 1) * pl + ob] = T(0);
@@ -1027,7 +1098,8 @@ cudaError_t launch_fill_ghosts(T* base, int planes, const KParams<T>& kp, cudaSt
 
 template <typename T, int NP>
 cudaError_t open_bc_n(const KParams<T>& kp, T* pop, T* lag, const T* psi, const T* inflow, cudaStream_t s) {
-    k_open_bc<T, NP><<<(2 * kp.ny + 127) / 128, 128, 0, s>>>(kp, pop, lag, psi, inflow);
+    k_open_bc<T, NP><<<(2 * kp.ny * NP + kOpenThreads - 1) / kOpenThreads, kOpenThreads, 0, s>>>(kp, pop, lag, psi,
+                                                                                             inflow);
     return cudaGetLastError();
 }
 template <typename T>

@@ -101,3 +101,40 @@ def test_3d_paths_on_ragged_boxes(D, nx, ny, nz, N, field, precision, path):
     tc, tu = (1e-10, 1e-10) if precision == D.DDCC_FP64 else (2e-5, 1e-6)
     assert np.abs(ref["C"] - got["C"])[:, fl].max() <= tc
     assert max(np.abs(ref[k] - got[k])[fl].max() for k in ("ux", "uy", "uz")) <= tu
+
+
+@pytest.mark.parametrize("nx,ny,N,px,py,open_x", [
+    (25, 3, 2, 1, 1, False),      # narrowest fused grid; three rows keep the fill launch
+    (33, 4, 3, 1, 0, False),      # one column into the second tile
+    (64, 16, 2, 0, 0, False),     # whole tiles, walls all round
+    (35, 9, 3, 1, 1, False),      # last tile within the ring's two columns
+    (97, 33, 4, 0, 1, False),
+    (48, 17, 3, 0, 0, True),      # open ends write their own copies
+    (41, 22, 2, 0, 1, True),
+])
+def test_fp32_step_writes_its_ghost_rings(D, nx, ny, N, px, py, open_x):
+    """After steps of the fused kernel (plain and replayed) the 2-node ring of
+    the phase populations and the 1-node ring of the lagged plane a hold the
+    copies that loading the state anew would put there, bit for bit."""
+    from paper_2311_10314_gb300 import _lib
+    pb = W.random_problem(nx, ny, N, seed=nx * ny, periodic_x=px, periodic_y=py, theta_field=True, width=6.0)
+    y = np.arange(ny) + 0.5
+    ox = (0.01 * y * (ny - y) / ny ** 2, np.full((N - 1, ny), 0.2)) if open_x else None
+    sim = D.Sim(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field, precision=D.DDCC_FP32, open_x=ox)
+    org, pitch, plane = _lib.state_layout(nx, ny, N, 4)
+
+    def rings():
+        s = sim.save_state().view(torch.float32)
+        f = torch.as_strided(s, (9 * (N - 1), ny + 4, nx + 4), (plane, pitch, 1), org - 2 * pitch - 2)
+        a = torch.as_strided(s, (ny + 2, nx + 2), (pitch, 1), org + 9 * N * plane - pitch - 1)
+        return f.cpu().numpy().copy(), a.cpu().numpy().copy()
+
+    for n in (1, 6):
+        sim.step(n)
+        got = rings()
+        sim.load_state(sim.save_state())      # refills every ghost frame
+        want = rings()
+        assert np.isfinite(want[0]).all()
+        assert np.array_equal(got[0], want[0])
+        assert np.array_equal(got[1], want[1])
+    sim.close()
