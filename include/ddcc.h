@@ -187,8 +187,9 @@ int ddcc_set_inflow(ddcc_handle* h, const double* u_in, const double* C_in);
  * Advance nsteps >= 0 time steps (Eqs. 3.1 and 3.2 with the equilibria,
  * sources, velocity and pressure of Sec. 3).  Asynchronous on the stream.
  * On the fused tile path and the FP64 path, calls of four steps or more replay a CUDA graph of
- * two steps, captured on the first such call (not while profiling); the
- * arithmetic is the same as launching the kernels one by one.
+ * two steps, captured on the first such call, and once such calls have come
+ * to 128 steps one of eight (not while profiling); the arithmetic is the
+ * same as launching the kernels one by one.
  */
 int ddcc_step(ddcc_handle* h, int64_t nsteps);
 

@@ -47,6 +47,9 @@ constexpr int AX = 32;   // threads (and nodes) along x of every kernel here
 // ring nodes per node.
 template <typename T>
 __host__ __device__ constexpr int block_rows() { return sizeof(T) == 8 ? 2 : 8; }
+// Whether a kernel of the reverse step lets the next one start early.
+template <typename T>
+__host__ __device__ constexpr bool overlaps() { return sizeof(T) == 4; }
 // First node of the block.  FP64 counts the rows of blocks along grid x (grid
 // y ends at 65535 blocks, short of the tallest grids in rows of two).
 template <typename T>
@@ -207,6 +210,7 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_fields(KParams<T> 
                                                                      T* __restrict__ mu, T* __restrict__ chi) {
     constexpr int AY = block_rows<T>(), NT = AX * AY, W = AX + 2, H = AY + 2;
     __shared__ T sC[NP - 1][H][W], sP[H][W];
+    if constexpr (overlaps<T>()) wait_for_previous();
     const int x0 = first_x<T>(), y0 = first_y<T>();
     const int tid = threadIdx.y * AX + threadIdx.x;
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
@@ -241,6 +245,7 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_fields(KParams<T> 
         }
     }
     __syncthreads();
+    if constexpr (overlaps<T>()) dependents_may_start();
     if (x >= P.nx || y >= P.ny) return;
     const int ly = threadIdx.y + 1, lx = threadIdx.x + 1;
     const long long o = P.org + (long long)y * P.pitch + x;
@@ -274,6 +279,10 @@ __global__ void __launch_bounds__(AX * block_rows<T>(), sizeof(T) == 4 ? 2 : 4)
                const T* __restrict__ st_lag, const T* __restrict__ ad_pop_in, const T* __restrict__ ad_lag_in,
                T* __restrict__ ad_pop_out, T* __restrict__ ad_lag_out, AdjPlanes<T, NP> W) {
     constexpr int M = NP - 1, NM = mu_planes<NP>();
+    if constexpr (overlaps<T>()) {
+        wait_for_previous();
+        dependents_may_start();
+    }
     const int x = first_x<T>() + threadIdx.x, y = first_y<T>() + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
     const long long pl = P.plane;
@@ -736,10 +745,12 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather3(KParams<T>
     constexpr int NM = mu_planes<NP>(), NV = AdjPlanes<T, NP>::NV, RN = Ring<T>::N;
     extern __shared__ __align__(16) unsigned char g3_raw[];
     T* sm = reinterpret_cast<T*>(g3_raw);
+    wait_for_previous();
     const long long pl = P.plane;
     const int x0 = first_x<T>(), y0 = first_y<T>();
     load_ring<T, NV, true>(P, sm, W.lgC, x0, y0);
     __syncthreads();
+    if constexpr (overlaps<T>()) dependents_may_start();
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
     const int lx = threadIdx.x, ly = threadIdx.y;
@@ -788,8 +799,13 @@ __device__ __forceinline__ void mu_node_at(const KParams<T>& P, const T* __restr
     // beta_ij (g'(C_i) - g'(C_i + C_j)), v_i = sum_j sigma_ij V_j, V_j = (3 eps
     // / 4) div(psi grad C_j) + 3 |grad psi| W_j, W_j = C_j sum_q cos_jq C_q)
     const T p0 = Ps(0, 0);
-    T gpx, gpy;
-    dev::grad9(P, [&](int dy, int dx) { return Ps(dy, dx); }, gpx, gpy);
+    // summed side by side, not by diagonals as grad9: FP32 rounding decides
+    // which nodes of the fluid bulk pass kKinkGradPsi below, and this order is
+    // the one the FP32 gradients are stated for
+    const T pE = Ps(0, 1), pW = Ps(0, -1), pN = Ps(1, 0), pS = Ps(-1, 0);
+    const T pNE = Ps(1, 1), pNW = Ps(1, -1), pSW = Ps(-1, -1), pSE = Ps(-1, 1);
+    const T gpx = P.gw1 * (pE - pW) + P.gw2 * ((pNE - pNW) + (pSE - pSW));
+    const T gpy = P.gw1 * (pN - pS) + P.gw2 * ((pNE + pNW) - (pSE + pSW));
     const T agp = dev::root(gpx * gpx + gpy * gpy);
     T Cv[NP], V[NP];
     {
@@ -940,6 +956,7 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather2(KParams<T>
     extern __shared__ __align__(16) unsigned char g2_raw[];
     constexpr int RN = Ring<T>::N, RW = Ring<T>::W;
     T* sm = reinterpret_cast<T*>(g2_raw);
+    wait_for_previous();
     const long long pl = P.plane;
     const int x0 = first_x<T>(), y0 = first_y<T>();
     T* sG = sm;
@@ -951,6 +968,7 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather2(KParams<T>
     load_ring<T, 1, false>(P, sP, psi_pl, x0, y0);
     load_ring<T, NP - 1, false>(P, sC, W.C, x0, y0);
     __syncthreads();
+    if constexpr (overlaps<T>()) dependents_may_start();
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
     const int lx = threadIdx.x, ly = threadIdx.y;
@@ -1114,15 +1132,15 @@ cudaError_t adjoint_step_n(const AdjStepArgs<T>& a, cudaStream_t s) {
     W.a = a.st_lag;   // lagged plane 0
     const dim3 blk = node_block<T>(), grd = node_grid<T>(k.nx, k.ny);
     cudaError_t e;
-    k_adj_fields<T, NP, false><<<grd, blk, 0, s>>>(k, a.st_pop, a.psi, a.cosf, W.C, W.mu, W.chi);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_adj_node<T, NP><<<grd, blk, 0, s>>>(k, a.psi, a.st_pop, a.st_lag, a.ad_pop_in, a.ad_lag_in,
-                                          a.ad_pop_out, a.ad_lag_out, W);
-    k_adj_gather3<T, NP, true><<<grd, blk, sizeof(T) * Ring<T>::N * AdjPlanes<T, NP>::NV, s>>>(k, a.psi, W, a.ad_lag_out,
-                                                                                   a.cosf, a.dJ_dcos);
-    k_adj_gather2<T, NP><<<grd, blk, sizeof(T) * Ring<T>::N * (2 * (NP - 1) + 3), s>>>(k, a.psi, W, a.ad_pop_out,
-                                                                              a.dJ_dpsi, 0);
-    return cudaGetLastError();
+    if ((e = launch_dependent(overlaps<T>(), k_adj_fields<T, NP, false>, grd, blk, 0, s, k, a.st_pop, a.psi, a.cosf, W.C, W.mu, W.chi)) !=
+            cudaSuccess ||
+        (e = launch_dependent(overlaps<T>(), k_adj_node<T, NP>, grd, blk, 0, s, k, a.psi, a.st_pop, a.st_lag, a.ad_pop_in, a.ad_lag_in,
+                              a.ad_pop_out, a.ad_lag_out, W)) != cudaSuccess ||
+        (e = launch_dependent(overlaps<T>(), k_adj_gather3<T, NP, true>, grd, blk, sizeof(T) * Ring<T>::N * AdjPlanes<T, NP>::NV, s, k,
+                              a.psi, W, a.ad_lag_out, a.cosf, a.dJ_dcos)) != cudaSuccess)
+        return e;
+    return launch_dependent(overlaps<T>(), k_adj_gather2<T, NP>, grd, blk, sizeof(T) * Ring<T>::N * (2 * (NP - 1) + 3), s, k, a.psi, W,
+                            a.ad_pop_out, a.dJ_dpsi, 0);
 }
 
 template <typename T, int NP>

@@ -44,10 +44,11 @@ struct ddcc_handle {
     int use_tile_tma;     // FP32 1: halo-staged tile kernel, 2: fused order parameters; FP64 3: ddcc_fp64.cu
     int tile_wide;        // the fused kernel runs 64 x 4 tiles instead of 32 x 8
     CUtensorMap tt_pop[2], tt_lag[2], tt_c, tt_st, tt_a[2], tt_fh[2], tt_g[2];
-    // the fused tile step as a CUDA graph of two steps (from copy 0 back to
+    // the step as CUDA graphs of two and of eight steps (from copy 0 back to
     // copy 0), captured on first use: 0 not tried, 1 ready, -1 unavailable
-    int graph_state;
-    cudaGraphExec_t step_graph;
+    int graph_state[2];
+    cudaGraphExec_t step_graph[2];
+    int64_t replayed;     // steps run by the two-step graph
     // the read-out planes (f.macro) hold the fields of the current state;
     // cleared by every call that may change the state
     int macro_valid;
@@ -619,15 +620,22 @@ int step_plain(ddcc_handle* h, int64_t n) {
     return DDCC_OK;
 }
 
-// The fused tile step's launches of two consecutive steps (copy 0 -> 1 -> 0)
-// captured once into a CUDA graph on a private stream (the caller's stream
-// may be the legacy default stream, which cannot be captured).  The kernels
-// take the tensor maps and the parameters by value and the workspace never
-// moves, so the graph stays valid for the handle's life.  Any failure leaves
-// the plain launches in use.
+// The launches of consecutive steps (copy 0 -> 1 -> 0 ...) captured once into a
+// CUDA graph on a private stream (the caller's stream may be the legacy
+// default stream, which cannot be captured).  The kernels take the tensor
+// maps and the parameters by value and the workspace never moves, so the
+// graph stays valid for the handle's life.  Any failure leaves the plain
+// launches in use.
+constexpr int kGraphSteps[2] = {2, 8};
+// Between two graphs the GPU idles for a microsecond or two, so the longer
+// one is worth having (256 x 256, N = 3, FP32: 9.2 us a step with graphs of
+// two, 8.1 with graphs of sixteen), but its capture costs as much as a few
+// dozen steps save: it is made for a handle that has come to this many.
+constexpr int64_t kLongGraphAfter = 128;
+
 template <typename T>
-void build_step_graph(ddcc_handle* h) {
-    h->graph_state = -1;
+void build_step_graph(ddcc_handle* h, int which) {
+    h->graph_state[which] = -1;
     cudaStream_t cs = nullptr;
     if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return;
     const cudaStream_t user = h->stream;
@@ -638,13 +646,14 @@ void build_step_graph(ddcc_handle* h) {
     cudaGraph_t g = nullptr;
     int rc = DDCC_ERR_CUDA;
     if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-        rc = step_plain<T>(h, 2);
+        rc = step_plain<T>(h, kGraphSteps[which]);
         if (cudaStreamEndCapture(cs, &g) != cudaSuccess) rc = DDCC_ERR_CUDA;
     }
     h->stream = user;
     h->cur = cur;
     h->steps = steps;
-    if (rc == DDCC_OK && g && cudaGraphInstantiate(&h->step_graph, g, 0) == cudaSuccess) h->graph_state = 1;
+    if (rc == DDCC_OK && g && cudaGraphInstantiate(&h->step_graph[which], g, 0) == cudaSuccess)
+        h->graph_state[which] = 1;
     if (g) cudaGraphDestroy(g);
     cudaStreamDestroy(cs);
     cudaGetLastError();   // a refused capture leaves no sticky error behind
@@ -653,16 +662,27 @@ void build_step_graph(ddcc_handle* h) {
 template <typename T>
 int step_t(ddcc_handle* h, int64_t n) {
     if (h->profiling || h->use_sweep || h->use_tile_tma < 2 || n < 4) return step_plain<T>(h, n);
-    if (h->graph_state == 0) build_step_graph<T>(h);
-    if (h->graph_state != 1) return step_plain<T>(h, n);
+    if (h->graph_state[0] == 0) build_step_graph<T>(h, 0);
+    if (h->graph_state[0] != 1) return step_plain<T>(h, n);
     int st;
     if (h->cur == 1) {
         if ((st = step_plain<T>(h, 1))) return st;
         --n;
     }
-    for (int64_t i = 0; i < n / 2; ++i) DDCC_CU(cudaGraphLaunch(h->step_graph, h->stream));
-    h->steps += 2 * (n / 2);
-    return (n % 2) ? step_plain<T>(h, 1) : DDCC_OK;
+    for (int which = 1; which >= 0; --which) {
+        const int64_t G = kGraphSteps[which];
+        if (which == 1) {
+            if (n < G || h->replayed < kLongGraphAfter) continue;
+            if (h->graph_state[1] == 0) build_step_graph<T>(h, 1);
+            if (h->graph_state[1] != 1) continue;
+        }
+        for (; n >= G; n -= G) {
+            DDCC_CU(cudaGraphLaunch(h->step_graph[which], h->stream));
+            h->steps += G;
+            if (which == 0) h->replayed += G;
+        }
+    }
+    return n ? step_plain<T>(h, 1) : DDCC_OK;
 }
 
 // Error word of the kernels: bounded waits that ran out.
@@ -1351,7 +1371,8 @@ int ddcc_step_path(const ddcc_handle* h) {
 
 void ddcc_destroy(ddcc_handle* h) {
     if (!h) return;
-    if (h->graph_state == 1) cudaGraphExecDestroy(h->step_graph);
+    for (int w = 0; w < 2; ++w)
+        if (h->graph_state[w] == 1) cudaGraphExecDestroy(h->step_graph[w]);
     for (const auto& sg : h->seg_graphs) cudaGraphExecDestroy(sg.exec);
     if (h->side) cudaStreamDestroy(h->side);
     if (h->fork_ev) cudaEventDestroy(h->fork_ev);

@@ -19,6 +19,39 @@ constexpr int kMassBlocks = 304; // 2 x 152 SMs
 constexpr int kGX = 4;
 constexpr int kGY = 6;
 
+// Programmatic dependent launch, for the FP32 kernels that follow one another
+// on one stream in a step or a reverse step of a small grid.  A kernel lets
+// the next one start (dependents_may_start) once its blocks have what they
+// read, and takes its own place the same way: it sets up its barriers, then
+// waits for everything before it to have finished and become visible
+// (wait_for_previous) ahead of its first access to memory that another kernel
+// writes.  Every kernel launched with overlap executes that wait in all its
+// threads, so the order of a stream holds across any number of them; launched
+// without, both calls do nothing.  The FP64 kernels do without: the waiting
+// blocks of the next kernel take the places that keep the running one's
+// warps even over the SMs (300 x 170, N = 3: 74 us a step without, 89 and more
+// with).
+#ifdef __CUDACC__
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... K, class... A>
+cudaError_t launch_dependent(bool overlap, void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             A&&... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+#endif
+
 // Kernel constants in the arithmetic type T (all derived on the host from
 // ddcc_params; see ddcc_api.cu for each formula's source).
 template <typename T>

@@ -138,3 +138,33 @@ def test_fp32_step_writes_its_ghost_rings(D, nx, ny, N, px, py, open_x):
         assert np.array_equal(got[0], want[0])
         assert np.array_equal(got[1], want[1])
     sim.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("open_x", [False, True])
+def test_long_replay_matches_plain_launches(D, precision, open_x):
+    """Past 128 replayed steps ddcc_step uses the eight-step graph too: the
+    state after calls of many lengths, from either copy, is bit for bit that
+    of a handle whose launches stay plain (profiling on)."""
+    from paper_2311_10314_gb300 import _lib
+    pb = W.random_problem(70, 45, 3, seed=21, periodic_x=0 if open_x else 1, periodic_y=0, theta_field=True, width=5.0)
+    ox = (np.full(45, 0.002), np.full((2, 45), 0.1)) if open_x else None
+    sims = [D.Sim(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field, precision=precision, open_x=ox)
+            for _ in range(2)]
+    _lib.ddcc_profile(sims[0].h, True)
+    for n in (127, 4, 8, 9, 15, 16, 3, 27, 10):
+        for s in sims:
+            s.step(n)
+        _lib.ddcc_kernel_times(sims[0].h)
+    assert sims[0].steps == sims[1].steps == 219
+    a, b = sims[0].save_state(), sims[1].save_state()
+    fa, fb = sims[0].fields(), sims[1].fields()
+    assert np.isfinite(fa["C"]).all()
+    for k in ("C", "ux", "uy", "P", "mu"):
+        assert np.array_equal(fa[k], fb[k]), k
+    org, pitch, plane = _lib.state_layout(70, 45, 3, 8 if precision == 0 else 4)
+    v = [torch.as_strided(s.view(torch.float64 if precision == 0 else torch.float32), (36, 45, 70), (plane, pitch, 1), org)
+         for s in (a, b)]
+    assert torch.equal(*v)
+    for s in sims:
+        s.close()
