@@ -207,6 +207,13 @@ int ddcc_step(ddcc_handle* h, int64_t nsteps);
 int ddcc_read(ddcc_handle* h, int field, double* host_out);
 
 /*
+ * Every macroscopic field of the current state in one call: host_out receives
+ * (2N+4) x ny x nx doubles, C_1 .. C_N, rho, u_x, u_y, P, mu_1 .. mu_N, the
+ * values ddcc_read() gives one by one.  Synchronises the stream.
+ */
+int ddcc_read_fields(ddcc_handle* h, double* host_out);
+
+/*
  * Per-phase mass sum_x sum_p f^i_p (= sum_x psi C_i, conserved by the
  * method) for phases 1..N-1, reduced in FP64 on the device in a fixed
  * order.  host_out receives N-1 doubles.  Returns DDCC_ERR_NONFINITE if any

@@ -35,7 +35,7 @@ FIELD_PSI = 20
 
 # every symbol include/ddcc.h declares
 EXPORTED = (
-    "ddcc_workspace_bytes", "ddcc_create", "ddcc_step", "ddcc_read", "ddcc_mass",
+    "ddcc_workspace_bytes", "ddcc_create", "ddcc_step", "ddcc_read", "ddcc_read_fields", "ddcc_mass",
     "ddcc_state_bytes", "ddcc_save_state", "ddcc_load_state", "ddcc_step_count",
     "ddcc_destroy", "ddcc_status_string", "ddcc_version", "ddcc_profile", "ddcc_kernel_times",
     "ddcc_phase_mass_noalloc", "ddcc_step_path", "ddcc_adjoint_bytes", "ddcc_adjoint_step",
@@ -117,6 +117,8 @@ def load():
     lib.ddcc_step.restype = C.c_int
     lib.ddcc_read.argtypes = [vp, C.c_int, dp]
     lib.ddcc_read.restype = C.c_int
+    lib.ddcc_read_fields.argtypes = [vp, dp]
+    lib.ddcc_read_fields.restype = C.c_int
     lib.ddcc_mass.argtypes = [vp, dp]
     lib.ddcc_mass.restype = C.c_int
     lib.ddcc_state_bytes.argtypes = [vp]
@@ -276,6 +278,15 @@ def ddcc_read(h, field: int, out: np.ndarray):
     st = load().ddcc_read(C.c_void_p(h), C.c_int(int(field)), _dptr(out))
     if st != DDCC_OK:
         raise DdccError(st, "ddcc_read")
+    return out
+
+
+def ddcc_read_fields(h, out: np.ndarray):
+    """All 2N+4 fields into ``out`` (2N+4, ny, nx)."""
+    assert out.dtype == np.float64 and out.flags.c_contiguous
+    st = load().ddcc_read_fields(C.c_void_p(h), _dptr(out))
+    if st != DDCC_OK:
+        raise DdccError(st, "ddcc_read_fields")
     return out
 
 

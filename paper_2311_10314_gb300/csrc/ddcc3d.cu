@@ -1267,16 +1267,19 @@ __global__ void __launch_bounds__(256) k3_mass_partial(P3<T> P, F3<T> F, int cur
         for (int i = 0; i < NP; ++i) F.partial[blockIdx.x * kMaxN + i] = red[0][i];
 }
 
+// one warp: every lane sums every 32nd partial, then the lanes in a fixed order
 __global__ void k3_mass_final(const double* partial, int np, double* out, int* flag) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     int bad = 0;
     for (int i = 0; i < np; ++i) {
         double s = 0.0;
-        for (int b = 0; b < kMassBlocks; ++b) s += partial[b * kMaxN + i];
-        out[i] = s;
-        if (!isfinite(s)) bad = 1;
+        for (int b = threadIdx.x; b < kMassBlocks; b += 32) s += partial[b * kMaxN + i];
+        for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
+        if (threadIdx.x == 0) {
+            out[i] = s;
+            if (!isfinite(s)) bad = 1;
+        }
     }
-    *flag = bad;
+    if (threadIdx.x == 0) *flag = bad;
 }
 
 // ---------------------------------------------------------------------------

@@ -164,7 +164,8 @@ Layout layout_of(const ddcc_params* p) {
         L.st64 = take(pb * static64_planes());
     }
     L.partial = take(sizeof(double) * kMassBlocks * kMaxPhases);
-    L.stage = take(sizeof(double) * (size_t)p->nx * p->ny * (N - 1));
+    L.stage = take(sizeof(double) * (size_t)p->nx * p->ny *
+                   (p->precision == DDCC_FP64 ? stage_planes<double>(N) : stage_planes<float>(N)));
     L.inflow = take(es * (size_t)p->ny * N);
     L.mass = take(sizeof(double) * kMaxPhases);
     L.flag = take(sizeof(int) * 4);
@@ -700,48 +701,72 @@ int refresh_ghosts_t(ddcc_handle* h) {
 
 template <typename T>
 int check_flag(ddcc_handle* h) {
+    if (h->use_tile_tma == 3) return DDCC_OK;   // no kernel of that path waits
     int flag = 0;
     DDCC_CU(cudaMemcpyAsync(&flag, fd_of<T>(h).flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     DDCC_CU(cudaStreamSynchronize(h->stream));
     return flag ? DDCC_ERR_TIMEOUT : DDCC_OK;
 }
 
+// The read-out planes of the current state (C_i, rho, u_x, u_y, P, mu_i).
 template <typename T>
-int read_t(ddcc_handle* h, int field, double* out) {
-    const ddcc_params& p = h->prm;
-    const int N = p.nphase;
+int form_macro(ddcc_handle* h) {
+    if (h->macro_valid) return DDCC_OK;
     KParams<T>& k = kp_of<T>(h);
     Fields<T>& f = fd_of<T>(h);
-    const T* src = nullptr;
-    if (field == DDCC_FIELD_PSI) {
-        src = f.psi;
+    if constexpr (sizeof(T) == 8) {
+        Step64Args a = args64(f, f.f[h->cur], f.lag[h->cur], nullptr, nullptr);
+        a.macro = f.macro;
+        DDCC_CU(launch_fields64(k, a, h->stream));
+        DDCC_CU(launch_update64(k, a, h->stream));
     } else {
-        int plane = -1;
-        if (field >= DDCC_FIELD_C && field < DDCC_FIELD_C + N) plane = field - DDCC_FIELD_C;
-        else if (field == DDCC_FIELD_RHO) plane = N;
-        else if (field == DDCC_FIELD_UX) plane = N + 1;
-        else if (field == DDCC_FIELD_UY) plane = N + 2;
-        else if (field == DDCC_FIELD_P) plane = N + 3;
-        else if (field >= DDCC_FIELD_MU && field < DDCC_FIELD_MU + N) plane = N + 4 + field - DDCC_FIELD_MU;
-        if (plane < 0) return DDCC_ERR_PARAM;
-        if (!h->macro_valid) {
-            if constexpr (sizeof(T) == 8) {
-                Step64Args a = args64(f, f.f[h->cur], f.lag[h->cur], nullptr, nullptr);
-                a.macro = f.macro;
-                DDCC_CU(launch_fields64(k, a, h->stream));
-                DDCC_CU(launch_update64(k, a, h->stream));
-            } else {
-                DDCC_CU(launch_macro<T>(k, f, h->cur, h->stream));
-            }
-            h->macro_valid = 1;
-        }
-        src = f.macro + (size_t)plane * k.plane;
+        DDCC_CU(launch_macro<T>(k, f, h->cur, h->stream));
     }
-    DDCC_CU(launch_export<T>(src, f.stage, k, h->stream));
-    DDCC_CU(cudaMemcpyAsync(out, f.stage, sizeof(double) * (size_t)p.nx * p.ny,
-                            cudaMemcpyDeviceToHost, h->stream));
+    h->macro_valid = 1;
+    return DDCC_OK;
+}
+
+// n planes from src to the host, as many at a time as the staging area holds.
+template <typename T>
+int export_planes(ddcc_handle* h, const T* src, int n, double* out) {
+    const ddcc_params& p = h->prm;
+    KParams<T>& k = kp_of<T>(h);
+    Fields<T>& f = fd_of<T>(h);
+    const size_t nodes = (size_t)p.nx * p.ny;
+    const int group = stage_planes<T>(p.nphase);
+    for (int i = 0; i < n; i += group) {
+        const int m = n - i < group ? n - i : group;
+        DDCC_CU(launch_export<T>(src + (size_t)i * k.plane, f.stage, k, m, h->stream));
+        DDCC_CU(cudaMemcpyAsync(out + i * nodes, f.stage, sizeof(double) * nodes * m, cudaMemcpyDeviceToHost,
+                                h->stream));
+    }
     DDCC_CU(cudaStreamSynchronize(h->stream));
     return check_flag<T>(h);
+}
+
+template <typename T>
+int read_t(ddcc_handle* h, int field, double* out) {
+    const int N = h->prm.nphase;
+    Fields<T>& f = fd_of<T>(h);
+    if (field == DDCC_FIELD_PSI) return export_planes<T>(h, f.psi, 1, out);
+    int plane = -1;
+    if (field >= DDCC_FIELD_C && field < DDCC_FIELD_C + N) plane = field - DDCC_FIELD_C;
+    else if (field == DDCC_FIELD_RHO) plane = N;
+    else if (field == DDCC_FIELD_UX) plane = N + 1;
+    else if (field == DDCC_FIELD_UY) plane = N + 2;
+    else if (field == DDCC_FIELD_P) plane = N + 3;
+    else if (field >= DDCC_FIELD_MU && field < DDCC_FIELD_MU + N) plane = N + 4 + field - DDCC_FIELD_MU;
+    if (plane < 0) return DDCC_ERR_PARAM;
+    const int st = form_macro<T>(h);
+    if (st) return st;
+    return export_planes<T>(h, f.macro + (size_t)plane * kp_of<T>(h).plane, 1, out);
+}
+
+template <typename T>
+int read_fields_t(ddcc_handle* h, double* out) {
+    const int st = form_macro<T>(h);
+    if (st) return st;
+    return export_planes<T>(h, fd_of<T>(h).macro, 2 * h->prm.nphase + 4, out);
 }
 
 template <typename T>
@@ -1019,6 +1044,11 @@ int ddcc_read(ddcc_handle* h, int field, double* host_out) {
     if (!h || !host_out) return DDCC_ERR_PARAM;
     return h->prm.precision == DDCC_FP64 ? read_t<double>(h, field, host_out)
                                          : read_t<float>(h, field, host_out);
+}
+
+int ddcc_read_fields(ddcc_handle* h, double* host_out) {
+    if (!h || !host_out) return DDCC_ERR_PARAM;
+    return h->prm.precision == DDCC_FP64 ? read_fields_t<double>(h, host_out) : read_fields_t<float>(h, host_out);
 }
 
 int ddcc_mass(ddcc_handle* h, double* host_out) {

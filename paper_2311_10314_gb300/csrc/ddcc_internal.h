@@ -118,12 +118,18 @@ struct Fields {
     T* chi;           // (FP64) 1 plane: psi rho of the current step
     T* st64;          // (FP64) static64_planes() planes of psi's own terms, formed at create
     double* partial;  // kMassBlocks * kMaxPhases
-    double* stage;    // host-input staging (double), max(N-1,1) planes
+    double* stage;    // staging of host inputs and results (double), stage_planes(N) planes
     T* inflow;        // open x ends: u_in (ny values), then C_in ((N-1) x ny)
     int* flag;        // device error word
 };
 
 inline int lag_planes(int N) { return 2 * N + 3; }
+
+// Planes of the staging area: the N-1 of one host input; in FP64 all 2N+4
+// read-out fields, so that they leave in one copy (FP32 grids are the large
+// ones, and their fields leave in groups).
+template <typename T>
+constexpr int stage_planes(int N) { return sizeof(T) == 8 ? 2 * N + 4 : N - 1; }
 
 // Row-sweep kernel: strip width per precision, rows per iteration and
 // threads per CTA.  With 60 columns the order-parameter pass (strip + 2
@@ -227,7 +233,7 @@ template <typename T>
 cudaError_t launch_convert(const double* src, T* dst, const KParams<T>& kp, int planes,
                            cudaStream_t s);
 template <typename T>
-cudaError_t launch_export(const T* src, double* dst, const KParams<T>& kp, cudaStream_t s);
+cudaError_t launch_export(const T* src, double* dst, const KParams<T>& kp, int planes, cudaStream_t s);
 // Fill the ghost frame of `planes` consecutive planes starting at base, gx
 // columns and gy rows deep (at most kGX, kGY; the whole frame by default).
 template <typename T>

@@ -168,3 +168,22 @@ def test_long_replay_matches_plain_launches(D, precision, open_x):
     assert torch.equal(*v)
     for s in sims:
         s.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nx,ny,N", [(3, 3, 2), (33, 17, 3), (130, 45, 4)])
+def test_fields_in_one_call_are_the_fields_read_one_by_one(D, nx, ny, N, precision):
+    """ddcc_read_fields (in groups of the staging area's planes) against
+    ddcc_read, which a second handle of the same run uses."""
+    pb = W.random_problem(nx, ny, N, seed=nx, theta_field=True, width=6.0)
+    sims = [D.Sim(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field, precision=precision) for _ in range(2)]
+    for s in sims:
+        s.step(5)
+    a = sims[0].fields()
+    b = sims[1]
+    assert np.array_equal(a["C"], np.stack([b.read(D.FIELD_C + i) for i in range(N)]))
+    assert np.array_equal(a["mu"], np.stack([b.read(D.FIELD_MU + i) for i in range(N)]))
+    for k, f in (("rho", D.FIELD_RHO), ("ux", D.FIELD_UX), ("uy", D.FIELD_UY), ("P", D.FIELD_P)):
+        assert np.array_equal(a[k], b.read(f)), k
+    for s in sims:
+        s.close()
