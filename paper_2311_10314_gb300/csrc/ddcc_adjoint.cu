@@ -222,24 +222,32 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_fields(KParams<T> 
         if (sy) base[o + sy] = v;
         if (sx && sy) base[o + sx + sy] = v;
     };
+    // all the loads of a thread before the first use of one, so that they are
+    // in flight together (beyond the last ring node they repeat it)
+    constexpr int R = (H * W + NT - 1) / NT, NF = kC0 ? NP - 1 : 9 * (NP - 1);
+    T ps[R], v[R][NF];
 #pragma unroll
-    for (int r = 0; r < (H * W + NT - 1) / NT; ++r) {
-        const int k = tid + r * NT;
-        if (k >= H * W) break;
-        const int ly = k / W, lx = k - ly * W;
+    for (int r = 0; r < R; ++r) {
+        const int k = min(tid + r * NT, H * W - 1), ly = k / W, lx = k - ly * W;
         const long long o = P.org + (long long)ring_index(y0 + ly - 1, P.ny, P.py) * P.pitch +
                             ring_index(x0 + lx - 1, P.nx, P.px);
-        const T ps = psi[o];
-        sP[ly][lx] = ps;
-        const T inv = kC0 ? T(1) : dev::rcp(ps);
+        ps[r] = psi[o];
+#pragma unroll
+        for (int q = 0; q < NF; ++q) v[r][q] = kC0 ? C[q * pl + o] : f[q * pl + o];
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int k = min(tid + r * NT, H * W - 1), ly = k / W, lx = k - ly * W;
+        sP[ly][lx] = ps[r];
+        const T inv = kC0 ? T(1) : dev::rcp(ps[r]);
 #pragma unroll
         for (int i = 0; i < NP - 1; ++i) {
-            if (kC0) {
-                sC[i][ly][lx] = C[i * pl + o];
+            if constexpr (kC0) {
+                sC[i][ly][lx] = v[r][i];
             } else {
-                T s = f[(long long)(9 * i) * pl + o];
+                T s = v[r][9 * i];
 #pragma unroll
-                for (int p = 1; p < 9; ++p) s += f[(long long)(9 * i + p) * pl + o];
+                for (int p = 1; p < 9; ++p) s += v[r][9 * i + p];
                 sC[i][ly][lx] = s * inv;
             }
         }
@@ -692,25 +700,36 @@ __global__ void __launch_bounds__(AX * block_rows<T>(), sizeof(T) == 4 ? 2 : 4)
 // shared-memory stores and are all in flight at once.
 template <typename T>
 struct Ring {
-    static constexpr int AY = block_rows<T>(), W = AX + 2, H = AY + 2, N = W * H, NT = AX * AY;
+    static constexpr int AY = block_rows<T>(), W = AX + 2, H = AY + 2, N = W * H, NT = AX * AY, R = (N + NT - 1) / NT;
+    long long g[R];      // offsets of this thread's ring nodes (beyond the last they repeat it)
+    bool mx[R], my[R];   // mirrored along x, y
+    __device__ Ring(const KParams<T>& P, int x0, int y0) {
+        const int tid = threadIdx.y * AX + threadIdx.x;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int k = min(tid + r * NT, N - 1), ly = k / W, lx = k - ly * W;
+            const int X = x0 - 1 + lx, Y = y0 - 1 + ly;
+            mx[r] = !P.px && (X < 0 || X >= P.nx);
+            my[r] = !P.py && (Y < 0 || Y >= P.ny);
+            g[r] = P.org + (long long)ring_index(Y, P.ny, P.py) * P.pitch + ring_index(X, P.nx, P.px);
+        }
+    }
 };
 template <typename T, int NPL, bool kPairs>
-__device__ __forceinline__ void load_ring(const KParams<T>& P, T* sm, const T* __restrict__ base, int x0, int y0) {
+__device__ __forceinline__ void load_ring(const KParams<T>& P, const Ring<T>& ring, T* sm, const T* __restrict__ base) {
     using R = Ring<T>;
     const int tid = threadIdx.y * AX + threadIdx.x;
+    T v[R::R][NPL];
 #pragma unroll
-    for (int r = 0; r < (R::N + R::NT - 1) / R::NT; ++r) {
-        const int k = tid + r * R::NT;
-        if (k >= R::N) break;
-        const int ly = k / R::W, lx = k - ly * R::W;
-        const int X = x0 - 1 + lx, Y = y0 - 1 + ly;
-        const bool mx = !P.px && (X < 0 || X >= P.nx), my = !P.py && (Y < 0 || Y >= P.ny);
-        const long long g = P.org + (long long)ring_index(Y, P.ny, P.py) * P.pitch + ring_index(X, P.nx, P.px);
+    for (int r = 0; r < R::R; ++r)
 #pragma unroll
-        for (int q = 0; q < NPL; ++q) {
-            const T v = __ldg(base + q * P.plane + g);
-            sm[q * R::N + k] = kPairs && (q % 2 ? my : mx) ? -v : v;
-        }
+        for (int q = 0; q < NPL; ++q) v[r][q] = __ldg(base + q * P.plane + ring.g[r]);
+#pragma unroll
+    for (int r = 0; r < R::R; ++r) {
+        const int k = min(tid + r * R::NT, R::N - 1);
+#pragma unroll
+        for (int q = 0; q < NPL; ++q)
+            sm[q * R::N + k] = kPairs && (q % 2 ? ring.my[r] : ring.mx[r]) ? -v[r][q] : v[r][q];
     }
 }
 // sum_p gw_p (c_p . (vx, vy))(q - c_p) from the ring copy, q = thread's node
@@ -748,7 +767,7 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather3(KParams<T>
     wait_for_previous();
     const long long pl = P.plane;
     const int x0 = first_x<T>(), y0 = first_y<T>();
-    load_ring<T, NV, true>(P, sm, W.lgC, x0, y0);
+    load_ring<T, NV, true>(P, Ring<T>(P, x0, y0), sm, W.lgC);
     __syncthreads();
     if constexpr (overlaps<T>()) dependents_may_start();
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
@@ -963,10 +982,11 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather2(KParams<T>
     T* sL = sG + 2 * RN;
     T* sP = sL + (NP - 1) * RN;
     T* sC = sP + RN;
-    load_ring<T, 2, true>(P, sG, W.mgp, x0, y0);
-    load_ring<T, NP - 1, false>(P, sL, W.mL, x0, y0);
-    load_ring<T, 1, false>(P, sP, psi_pl, x0, y0);
-    load_ring<T, NP - 1, false>(P, sC, W.C, x0, y0);
+    const Ring<T> ring(P, x0, y0);
+    load_ring<T, 2, true>(P, ring, sG, W.mgp);
+    load_ring<T, NP - 1, false>(P, ring, sL, W.mL);
+    load_ring<T, 1, false>(P, ring, sP, psi_pl);
+    load_ring<T, NP - 1, false>(P, ring, sC, W.C);
     __syncthreads();
     if constexpr (overlaps<T>()) dependents_may_start();
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
@@ -1083,13 +1103,19 @@ __global__ void __launch_bounds__(256) k_centroid_partial(KParams<T> P, const T*
     }
 }
 
+// one warp; every lane sums every 32nd pair of partials, then the lanes in a
+// fixed order (one thread adding all 304 pairs took 30 us)
 __global__ void k_centroid_final(const double* __restrict__ part, int nblocks, double* __restrict__ out) {
-    if (threadIdx.x != 0) return;
     double s0 = 0.0, s1 = 0.0;
-    for (int b = 0; b < nblocks; ++b) {
+    for (int b = threadIdx.x; b < nblocks; b += 32) {
         s0 += part[2 * b];
         s1 += part[2 * b + 1];
     }
+    for (int d = 16; d > 0; d >>= 1) {
+        s0 += __shfl_down_sync(0xffffffffu, s0, d);
+        s1 += __shfl_down_sync(0xffffffffu, s1, d);
+    }
+    if (threadIdx.x != 0) return;
     out[0] = s1 / s0;   // J
     out[1] = s0;        // M
 }

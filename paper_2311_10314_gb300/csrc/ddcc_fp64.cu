@@ -67,28 +67,37 @@ __global__ void __launch_bounds__(FT) k_fields64(KParams<Real> P, const Real* __
     __shared__ Real sC[NP - 1][H][W], sP[H][W];
     const int tid = threadIdx.x;
     const int x0 = (blockIdx.x % tiles_x) * FX, y0 = (blockIdx.x / tiles_x) * FY;
+    // all the loads of a thread before the first use of one, so that they are
+    // in flight together (beyond the last ring node they repeat it)
+    constexpr int R = (H * W + FT - 1) / FT, NF = 9 * (NP - 1);
+    Real v[R][NF], inv[R], ps[R];
+    long long o_[R];
 #pragma unroll
-    for (int r = 0; r < (H * W + FT - 1) / FT; ++r) {
-        const int k = tid + r * FT;
-        if (k >= H * W) break;
-        const int ly = k / W, lx = k - ly * W;
-        const int X = x0 + lx - 1, Y = y0 + ly - 1;
-        if (X > P.nx || Y > P.ny) continue;
-        const long long o = P.org + (long long)map_index(Y, P.ny, P.py) * P.pitch + map_index(X, P.nx, P.px);
-        const Real inv = st[kInvPsi * P.plane + o], ps = psi[o];
+    for (int r = 0; r < R; ++r) {
+        const int k = min(tid + r * FT, H * W - 1), ly = k / W, lx = k - ly * W;
+        const int X = min(x0 + lx - 1, P.nx), Y = min(y0 + ly - 1, P.ny);
+        const long long o = o_[r] = P.org + (long long)map_index(Y, P.ny, P.py) * P.pitch + map_index(X, P.nx, P.px);
+        inv[r] = st[kInvPsi * P.plane + o];
+        ps[r] = psi[o];
+#pragma unroll
+        for (int q = 0; q < NF; ++q) v[r][q] = f[q * P.plane + o];
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int k = min(tid + r * FT, H * W - 1), ly = k / W, lx = k - ly * W;
         Real c[NP - 1];
 #pragma unroll
         for (int i = 0; i < NP - 1; ++i) {
-            Real s = f[(long long)(9 * i) * P.plane + o];
+            Real s = v[r][9 * i];
 #pragma unroll
-            for (int p = 1; p < 9; ++p) s += f[(long long)(9 * i + p) * P.plane + o];
-            sC[i][ly][lx] = c[i] = s * inv;
+            for (int p = 1; p < 9; ++p) s += v[r][9 * i + p];
+            sC[i][ly][lx] = c[i] = s * inv[r];
         }
-        sP[ly][lx] = ps;
-        if (lx >= 1 && lx <= FX && ly >= 1 && ly <= FY && X < P.nx && Y < P.ny) {
+        sP[ly][lx] = ps[r];
+        if (lx >= 1 && lx <= FX && ly >= 1 && ly <= FY && x0 + lx - 1 < P.nx && y0 + ly - 1 < P.ny) {
 #pragma unroll
-            for (int i = 0; i < NP - 1; ++i) C[i * P.plane + o] = c[i];
-            chi[o] = dev::psi_rho<Real, NP>(P, ps, [&](int j) { return c[j]; });
+            for (int i = 0; i < NP - 1; ++i) C[i * P.plane + o_[r]] = c[i];
+            chi[o_[r]] = dev::psi_rho<Real, NP>(P, ps[r], [&](int j) { return c[j]; });
         }
     }
     __syncthreads();
