@@ -255,6 +255,9 @@ cudaError_t launch_fill_ghosts2(const GhostRing<T>& g0, const GhostRing<T>& g1, 
 constexpr int kFusedGhostF = 2;
 constexpr int kFusedGhostA = 1;
 
+// *dst = v on the device.
+cudaError_t launch_store(long long* dst, long long v, cudaStream_t s);
+
 // Open x ends: reset the columns x = 0 and nx - 1 of the populations and
 // lagged planes at pop/lag (a state just written by a step) to the inflow /
 // outflow equilibrium.

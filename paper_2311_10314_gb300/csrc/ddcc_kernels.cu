@@ -945,6 +945,8 @@ __global__ void k_wall_accumulate(KParams<T> P, const T* __restrict__ stage, T* 
     }
 }
 
+__global__ void k_store(long long* dst, long long v) { *dst = v; }
+
 inline dim3 tile_grid(int nx, int ny) {
     return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY);
 }
@@ -987,6 +989,11 @@ cudaError_t mass_n(const KParams<T>& kp, const Fields<T>& fd, int cur, double* o
 }
 
 }  // namespace
+
+cudaError_t launch_store(long long* dst, long long v, cudaStream_t s) {
+    k_store<<<1, 1, 0, s>>>(dst, v);
+    return cudaGetLastError();
+}
 
 #define DDCC_DISPATCH(fn, ...)                                \
     switch (kp.N) {                                           \
