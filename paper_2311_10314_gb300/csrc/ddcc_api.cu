@@ -237,7 +237,11 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
         for (int a = 0; a < 9; ++a) k.lamf[i][a] = (T)(s[a] / Nab[a]);
         k.ceta[i] = (T)(cs2 * p->eta[i]);
         k.cV[i] = (T)(0.5 * s1 / n1 - 1.0 / n1);
+        k.qf[i] = (T)((p->s_f[1] - s1) / n1);
     }
+    k.one_rate = p->s_f[1] == p->s_f[2] && p->s_f[1] == p->s_f[3] && p->s_f[1] == p->s_f[4];
+    k.sf = (T)p->s_f[1];
+    k.one_m_sf = (T)(1.0 - p->s_f[1]);
     k.lg00 = (T)(p->s_g[0]);
     k.lg1 = (T)(p->s_g[1] / n1);
     k.cg0 = (T)(0.5 * p->s_g[0] - 1.0);

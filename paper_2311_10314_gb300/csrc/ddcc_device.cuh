@@ -300,6 +300,42 @@ __device__ __forceinline__ void hermite_relax_back(const T k[9], const KParams<T
     out[8] = v[8] - wd * (Em + Rm[1]);
 }
 
+// The phase collision where one rate s holds for every moment of second and
+// higher order (the paper's own choice, Secs. 4.1-4.4).  The rows are complete
+// (sum_ab w_p h_ab(c_p) m_ab / N_ab = v_p), so relaxing all of them by s is
+// (1 - s) v_p, and only the conserved and the first-order rows are put
+// right; f^eq less its first order is w_p emu + X delta_p0, emu = eta psi mu,
+// X = psi C - emu:
+//   out_p = (1 - s) v_p + w_p (s emu + c_p . q) + s X delta_p0,
+//   q = s j / cs2 - k_1,  k_1 = lambda_1 (j - psi C u) + cV V.
+// 26 FP64 instructions a phase less than the transforms (FP64 only: FP32 is
+// bound by memory).  The rest population's exchange and its rounding error
+// are treated as in hermite_relax_back.
+template <typename T>
+__device__ __forceinline__ void relax_one_rate(const KParams<T>& P, int i, const T v[9], T jx, T jy, T psiC, T emu,
+                                               T pcux, T pcuy, T Vx, T Vy, T out[9]) {
+    const T lam = P.lamf[i][1];
+    const T qx = P.qf[i] * jx + lam * pcux - P.cV[i] * Vx;
+    const T qy = P.qf[i] * jy + lam * pcuy - P.cV[i] * Vy;
+    const T se = P.sf * emu;
+    const T a = P.w9[1] * se, ax = P.w9[1] * qx, ay = P.w9[1] * qy;
+    const T d = P.w9[2] * se, dp = P.w9[2] * (qx + qy), dm = P.w9[2] * (qx - qy);
+    const T k = P.one_m_sf;
+    const T t0 = P.sf * (v[0] - (psiC - emu)) - P.w9[0] * se;
+    const T o0 = add_rn(v[0], -t0);
+    const T bb = add_rn(o0, -v[0]);                 // TwoSum(v_0, -t_0)
+    const T half = T(0.5) * add_rn(add_rn(v[0], -add_rn(o0, -bb)), add_rn(-t0, -bb));
+    out[0] = o0;
+    out[1] = add_rn(k * v[1] + (a + ax), half);
+    out[3] = add_rn(k * v[3] + (a - ax), half);
+    out[2] = k * v[2] + (a + ay);
+    out[4] = k * v[4] + (a - ay);
+    out[5] = k * v[5] + (d + dp);
+    out[7] = k * v[7] + (d - dp);
+    out[8] = k * v[8] + (d + dm);
+    out[6] = k * v[6] + (d - dm);
+}
+
 // psi rho at a node, rho = rho_N + sum_j (rho_j - rho_N) C_j
 template <typename T, int NP, class CA>
 __device__ __forceinline__ T psi_rho(const KParams<T>& P, T psi, const CA& C) {
@@ -322,7 +358,8 @@ __device__ __forceinline__ T psi_rho(const KParams<T>& P, T psi, const CA& C) {
 // above, the FP64 tile step (bound by its FP64 pipe) went from 629 to 511 us
 // at 512 x 512, N = 4, and from 51 to 40 us at 64 x 64, N = 2; in FP32, bound
 // by memory, these changes alone leave the time as it was.
-template <typename T, int NP, int MODE, class Acc, class Sink>
+// kOneRate: the phase collision by relax_one_rate.
+template <typename T, int NP, int MODE, bool kOneRate = false, class Acc, class Sink>
 __device__ __forceinline__ void node_update(const KParams<T>& P, const Acc& A, Sink& out) {
     const T cs2 = P.cs2;
     const T psi = A.psi(0, 0);
@@ -453,24 +490,37 @@ __device__ __forceinline__ void node_update(const KParams<T>& P, const Acc& A, S
         T v[9], m[9], k[9], o9[9];
 #pragma unroll
         for (int p = 0; p < 9; ++p) v[p] = A.f(i, p);
-        hermite_moments(v, cs2, m);
+        if constexpr (kOneRate) {
+            const T d1 = v[5] - v[7], d2 = v[8] - v[6];
+            m[1] = (v[1] - v[3]) + (d1 + d2);
+            m[2] = (v[2] - v[4]) + (d1 - d2);
+            // in the order of hermite_moments
+            m[0] = (((v[7] + v[8]) + v[4]) + (v[3] + v[1]) + ((v[6] + v[5]) + v[2])) + v[0];
+        } else {
+            hermite_moments(v, cs2, m);
+        }
         const T psiC = m[0];
         const T pcux = psiC * ux, pcuy = psiC * uy;
         // V = d_t(psi C u) + cs2 eta (mu grad psi - S), S = psi (Q - grad mu)
         const T Vx = (pcux - A.lag(1 + 2 * i)) + P.ceta[i] * (mu[i] * gpx + psi * (gmx[i] - Qx[i]));
         const T Vy = (pcuy - A.lag(2 + 2 * i)) + P.ceta[i] * (mu[i] * gpy + psi * (gmy[i] - Qy[i]));
-        const T X = psiC - P.eta[i] * psi * mu[i];
-        const T* lam = P.lamf[i];
-        k[0] = T(0);
-        k[1] = lam[1] * (m[1] - pcux) + P.cV[i] * Vx;
-        k[2] = lam[2] * (m[2] - pcuy) + P.cV[i] * Vy;
-        k[3] = lam[3] * (m[3] + cs2 * X);
-        k[4] = lam[4] * (m[4] + cs2 * X);
-        k[5] = lam[5] * m[5];
-        k[6] = lam[6] * m[6];
-        k[7] = lam[7] * m[7];
-        k[8] = lam[8] * (m[8] - P.cs4 * X);
-        hermite_relax_back<T, true>(k, P, v, o9);
+        if constexpr (kOneRate) {
+            const T emu = P.eta[i] * (psi * mu[i]);
+            relax_one_rate(P, i, v, m[1], m[2], psiC, emu, pcux, pcuy, Vx, Vy, o9);
+        } else {
+            const T X = psiC - P.eta[i] * psi * mu[i];
+            const T* lam = P.lamf[i];
+            k[0] = T(0);
+            k[1] = lam[1] * (m[1] - pcux) + P.cV[i] * Vx;
+            k[2] = lam[2] * (m[2] - pcuy) + P.cV[i] * Vy;
+            k[3] = lam[3] * (m[3] + cs2 * X);
+            k[4] = lam[4] * (m[4] + cs2 * X);
+            k[5] = lam[5] * m[5];
+            k[6] = lam[6] * m[6];
+            k[7] = lam[7] * m[7];
+            k[8] = lam[8] * (m[8] - P.cs4 * X);
+            hermite_relax_back<T, true>(k, P, v, o9);
+        }
 #pragma unroll
         for (int p = 0; p < 9; ++p) out.f_out(i, p, o9[p]);
         out.lag_out(1 + 2 * i, pcux);

@@ -21,7 +21,11 @@
 //    ghost ring of the lagged plane a, which the reverse step reads, is
 //    written along with the plane.
 // Against the one-kernel tile step with the same node arithmetic: 512 x 512,
-// N = 4, 511 -> 440 us a step; 64 x 64, N = 2, 40 -> 20 us.
+// N = 4, 511 -> 440 us a step; 64 x 64, N = 2, 40 -> 20 us.  With one rate for
+// the phases' higher moments (relax_one_rate) 398 and 16.  Both kernels then
+// run at 92 to 96% of the FP64 rate that chains of multiply-adds reach
+// (ddcc_measure_fp64_peak), with 848 FP64 instructions a node by the
+// transforms and 770 with one rate (N = 4; 1165 in the tile kernel at first).
 #include "ddcc_device.cuh"
 
 namespace ddcc {
@@ -175,7 +179,7 @@ __device__ __forceinline__ int ring_step(int v, int n, int periodic) {
     return 0;
 }
 
-template <int NP, int MODE>
+template <int NP, int MODE, bool kOneRate>
 __global__ void __launch_bounds__(UT, 5) k_update64(KParams<Real> P, Step64Args F) {
     const unsigned idx = blockIdx.x * (unsigned)UT + threadIdx.x;
     if (idx >= (unsigned)P.nx * (unsigned)P.ny) return;
@@ -204,7 +208,7 @@ __global__ void __launch_bounds__(UT, 5) k_update64(KParams<Real> P, Step64Args 
             sink.tgt[p] = bounce ? vopp(p) * P.plane + acc.o : p * P.plane + acc.at(vy(p), vx(p));
         }
     }
-    dev::node_update<Real, NP, MODE>(P, acc, sink);
+    dev::node_update<Real, NP, MODE, kOneRate>(P, acc, sink);
 }
 
 template <int NP>
@@ -217,7 +221,10 @@ cudaError_t fields_n(const KParams<Real>& kp, const Step64Args& a, cudaStream_t 
 template <int NP, int MODE>
 cudaError_t update_n(const KParams<Real>& kp, const Step64Args& a, cudaStream_t s) {
     const long long n = (long long)kp.nx * kp.ny;
-    k_update64<NP, MODE><<<(unsigned)((n + UT - 1) / UT), UT, 0, s>>>(kp, a);
+    const unsigned blocks = (unsigned)((n + UT - 1) / UT);
+    // 512 x 512, N = 4: 327 us a launch by the transforms, 285 with one rate
+    if (MODE == 0 && kp.one_rate) k_update64<NP, MODE, MODE == 0><<<blocks, UT, 0, s>>>(kp, a);
+    else k_update64<NP, MODE, false><<<blocks, UT, 0, s>>>(kp, a);
     return cudaGetLastError();
 }
 

@@ -87,6 +87,10 @@ struct KParams {
     // (00, 10, 01, 20, 02, 11, 21, 12, 22), and 1 / N_ab
     T lamf[kMaxPhases][9];
     T invN[9];
+    // one rate for the moments of second and higher order: that rate, 1 less it,
+    // and rate / cs2 - lambda_1 per phase
+    int one_rate;
+    T sf, one_m_sf, qf[kMaxPhases];
     // flow LB constant rates as lambda = s / N (00, 10, 01, 21, 12, 22)
     T lg00, lg1, lg3, lg4;
     T cg0, cg1;                   // lg00 / 2 - 1 and lg1 / 2 - 1 / N_1

@@ -187,3 +187,20 @@ def test_fields_in_one_call_are_the_fields_read_one_by_one(D, nx, ny, N, precisi
         assert np.array_equal(a[k], b.read(f)), k
     for s in sims:
         s.close()
+
+
+@pytest.mark.parametrize("N", [2, 3, 4])
+@pytest.mark.parametrize("rates", [(1.0, 1.2, 1.2, 1.2, 1.2), (0.9, 1.6, 1.6, 1.6, 1.6), (1.0, 1.2, 1.1, 1.2, 1.2),
+                                   (1.0, 1.2, 1.2, 1.2, 1.0)])
+def test_fp64_phase_rates(D, N, rates):
+    """FP64 against the oracle with one phase-LB rate above first order (its
+    own collision) and with rates that differ (the transforms), and the phase
+    mass, which the collision carries in its rest population."""
+    pb = W.random_problem(70, 33, N, seed=5 + N, periodic_y=0, theta_field=True, width=6.0)
+    pb.params["s_f"] = list(rates)
+    _against_oracle(D, pb, D.DDCC_FP64, 20)
+    sim = D.Sim(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field, precision=D.DDCC_FP64)
+    m0 = sim.mass()
+    sim.step(200)
+    assert np.abs(sim.mass() - m0).max() <= 1e-13 * np.abs(m0).max()
+    sim.close()
