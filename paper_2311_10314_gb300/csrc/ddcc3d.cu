@@ -503,9 +503,9 @@ struct GlobalSrc {     // the per-step C and mu planes in global memory
 // 1116 + 341 + 35 us for update, mu and C before sums over all phases, pair
 // identities of mu, psi's own terms, 256-thread blocks of 32 x 4 x 2 nodes and
 // divisions by the operator went; 10 steps and a read-out 18.0 -> 9.4 ms.
-// FP32 (fused): 24% fewer instructions, 753 -> 722 us at 208 x 192 x 160; the
-// loads and stores of this kernel alone take 504 us there (loads 314), the
-// stores in 128-byte rows of 45 planes.
+// FP32 (fused): 24% fewer instructions, 753 -> 722 us at 208 x 192 x 160, and
+// 617 with field a staged; the kernel's loads and stores alone take 504 us
+// there (loads 314), the stores in 128-byte rows of 45 planes.
 template <typename T, int NP, bool kMacro, class S>
 __device__ __forceinline__ void update_node(const P3<T>& P, const F3<T>& F, int cur, T* out, const S& src) {
     constexpr int N = NP + 1, NM = NP == 1 ? 1 : N;
@@ -858,14 +858,16 @@ __global__ void __launch_bounds__(node_threads<T>(), sizeof(T) == 4 ? 2 : 4) k3_
 // The copies of plane z+3 fly during the mu pass and the update of plane z.
 // (101 x 77 x 63, N = 2, where the copies are by node: 68 us a step with
 // plain loads, 62 with the copies.)
-// With kStage (FP32 and N <= 3, where the staging still leaves room for two
-// CTAs per SM) each thread also copies its own node's 15 flow populations
-// and 3N + 4 lagged values of plane z+1 (4-byte cp.async) as soon as its
-// update of plane z has read those of plane z; they fly during the C pass,
-// the mu pass and both barriers.  Copy groups are committed in the same
-// order by every thread (empty groups where a thread has nothing to copy):
-// raw(z+2), stage(z), raw(z+3), stage(z+1), ..., so "all but the newest
-// group" is the data each wait needs.
+// The lagged field a (three components, read at 36 neighbour positions) comes
+// the same way, a plane ahead, into a ring of three planes: 617 us a step
+// instead of 722 with those reads through L1 (208 x 192 x 160, N = 3).  With kStage (FP32
+// and N <= 3, where two CTAs per SM still fit) so do the column's 15 flow
+// populations and 3N + 4 lagged values.  Both are issued after the barrier
+// that ends the update of the plane before, fly during the mu pass, and are
+// waited for ahead of the barrier that starts the update.  Groups are
+// committed in the same order by every thread (empty ones where a thread has
+// nothing to copy): stage(z), raw(z+3), stage(z+1), raw(z+4), ..., so "all but
+// the newest group" is what the update needs and "all" what the C pass needs.
 // The per-step C and mu planes of global memory are neither read nor
 // written; the update arithmetic is update_node's, the same as the
 // three-kernel step's.
@@ -883,15 +885,14 @@ struct FusedGeom {
     static constexpr int NSTG = 15 + 3 * N + 4;                     // own-node g and lagged values
     static constexpr int STG = kStage ? NSTG * NT : 0;
     static constexpr int NMU = NP == 1 ? 1 : N;                     // mu planes (N = 2: mu_2 = -mu_1)
-    static constexpr int BASE = 5 * (NP + 1) * CN + 3 * NMU * MN + RAW + STG;
+    static constexpr int AW = CW, AH = TY + 2, AN = AW * AH;        // region of the lagged field a
+    static constexpr int A = kRaw ? 3 * 3 * AN : 0;                 // (FP32) a_xy, a_yz, a_zx, three planes
+    static constexpr int BASE = 5 * (NP + 1) * CN + 3 * NMU * MN + RAW + STG + A;
     // psi rho (with mu, three planes) and grad psi of the own nodes (two planes)
-    // kept by the mu pass, where two CTAs with them still leave the SM's
-    // larger L1 (shared memory up to 196 of its 256 KB; each CTA costs 1 KB and
-    // the column indices more): the update reads plane a's neighbours and its
-    // own populations through L1.  At N = 3 with staged copies they do not
-    // fit: 807 us a step with them, 722 with both formed again from C and psi
-    // (208 x 192 x 160).
-    static constexpr bool kKeep = sizeof(T) * (BASE + 3 * MN + 2 * 3 * NT) + 1280 <= 196 * 1024 / 2;
+    // kept by the mu pass where two CTAs still fit an SM with them (each costs
+    // 1 KB and the column indices more); else the update forms both again
+    // from C and psi.
+    static constexpr bool kKeep = sizeof(T) * (BASE + 3 * MN + 2 * 3 * NT) + 1280 <= 228 * 1024 / 2;
     static constexpr int NM = NMU + (kKeep ? 1 : 0);                // planes of the mu ring
     static constexpr int GP = kKeep ? 2 * 3 * NT : 0;
     static constexpr size_t smem = sizeof(T) * (BASE + (kKeep ? 3 * MN : 0) + GP);
@@ -907,6 +908,7 @@ struct SmemSrc {     // C, psi, mu and psi rho from the shared-memory rings
     const T* sMu;    // mu ring: slot k holds NM x MN values
     const T* sGp;    // (kKeep) grad psi: two slots of 3 x NT values
     const P3<T>* P;
+    const T* sA;     // (FP32) a ring, slots as mu's: three fields of AN values
     const T* stg;    // (kStage) own-node g (15) and lagged planes 3.. (NT apart)
     const T* f_;     // populations and lagged planes in global memory
     const T* g_;
@@ -914,7 +916,7 @@ struct SmemSrc {     // C, psi, mu and psi rho from the shared-memory rings
     long long plane;
     int c5[3], m3[3];  // ring slots of planes z-1, z, z+1
     int gp2;           // grad psi's slot of plane z
-    int ci, mi;        // the node in the C and mu regions
+    int ci, mi, ai;    // the node in the C, mu and a regions
     int tid;
     int xo[3], yo[3], zo[3];  // wrapped x, y nx, z nx ny of the node and its neighbours
     __device__ int at(int p) const { return zo[cz(p) + 1] + yo[cy(p) + 1] + xo[cx(p) + 1]; }
@@ -927,7 +929,10 @@ struct SmemSrc {     // C, psi, mu and psi rho from the shared-memory rings
         if constexpr (kStage) return stg[(12 + k) * G::NT + tid];
         else return __ldg(lag_ + k * plane + at(0));
     }
-    __device__ T a(int k, int p) const { return __ldg(lag_ + lag_a(k) * plane + at(p)); }
+    __device__ T a(int k, int p) const {
+        if constexpr (G::kRaw) return sA[(m3[cz(p) + 1] * 3 + k) * G::AN + ai + cy(p) * G::AW + cx(p)];
+        else return __ldg(lag_ + lag_a(k) * plane + at(p));
+    }
     __device__ T psi(int p) const { return sPs[c5[cz(p) + 1] * G::CN + ci + cy(p) * G::CW + cx(p)]; }
     __device__ T C(int j, int p) const {
         return sC[(c5[cz(p) + 1] * NP + j) * G::CN + ci + cy(p) * G::CW + cx(p)];
@@ -982,6 +987,7 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
     T* sGp = sMu + 3 * G::NM * MN;              // (kKeep) 2 slots x 3 x NT
     T* sRaw = sGp + G::GP;                      // (FP32) 7 NP + 1 planes x CN
     T* sStg = sRaw + G::RAW;                    // (kStage) NSTG x NT
+    T* sA = sStg + G::STG;                      // (FP32) 3 slots x 3 x AN
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * kBX, y0 = blockIdx.y * TY;
     const int zb = (int)((long long)blockIdx.z * P.nz / nchunk);
@@ -1029,14 +1035,13 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
         }
     };
     // C_i = sum_p f^i_p / psi and psi at plane z on the C region (as k3_order)
-    auto c_pass = [&](int z, bool steady) {
+    auto c_pass = [&](int z) {
         T* c = sC + slot5(z) * NP * CN;
         T* ps = sPs + slot5(z) * CN;
         if constexpr (kVec) {
             if (tid < G::NQ) {
                 const int o = 4 * tid;
-                if (steady) cp_async_wait<1>();   // stage(z - 2) may still fly
-                else cp_async_wait<0>();
+                cp_async_wait<0>();
                 const float4 psi = *reinterpret_cast<const float4*>(sRaw + 7 * NP * CN + o);
                 *reinterpret_cast<float4*>(ps + o) = psi;
 #pragma unroll
@@ -1057,8 +1062,7 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
         } else {
             const long long zo = zoff(z);
             if constexpr (G::kRaw) {
-                if (steady) cp_async_wait<1>();
-                else cp_async_wait<0>();
+                cp_async_wait<0>();
             }
 #pragma unroll
             for (int r = 0; r < G::KC; ++r) {
@@ -1136,6 +1140,8 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
     src.tid = tid;
     src.ci = (ty + 2) * CW + tx + 4;
     src.mi = (ty + 1) * MW + tx + 1;
+    src.ai = (ty + 1) * G::AW + tx + 4;
+    src.sA = sA;
     src.xo[0] = wrap_index(x - 1, P.nx);
     src.xo[1] = x;
     src.xo[2] = wrap_index(x + 1, P.nx);
@@ -1143,11 +1149,57 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
     src.yo[1] = y * P.nx;
     src.yo[2] = wrap_index(y + 1, P.ny) * P.nx;
     const int nxy = (int)P.nxy;   // nx ny nz < 2^31
-    // (kStage) copy this node's g and lagged values of plane z
-    auto stage = [&](int z, bool any) {
+    // (FP32) copy the lagged field a of plane z on the column and one node
+    // around it: quads of rows x0-4 .. x0+35 with kVec, else node by node
+    auto copy_a = [&](int z) {
+        if constexpr (G::kRaw) {
+            const int zo = wrap_index(z, P.nz) * nxy;
+            T* d = sA + slot3(z) * 3 * G::AN;
+            if constexpr (kVec) {
+                if (tid < G::AN / 4) {
+                    const int row = tid / (G::AW / 4), col = 4 * (tid % (G::AW / 4));
+                    const int i = zo + ys[row + 1] + xs[col];
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) cp_async16(d + k * G::AN + 4 * tid, src.lag_ + lag_a(k) * P.plane + i);
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < G::KM; ++r) {
+                    const int n = tid + r * NT;
+                    if (n < MN) {
+                        const int row = n / MW, col = n % MW + 3;
+                        const int i = zo + ys[row + 1] + xs[col];
+#pragma unroll
+                        for (int k = 0; k < 3; ++k)
+                            cp_async4(d + k * G::AN + row * G::AW + col, src.lag_ + lag_a(k) * P.plane + i);
+                    }
+                }
+            }
+        }
+    };
+    // (FP32) the group of copies that the update of plane z waits for: field a
+    // of plane z+1 and (kStage) the column's g and lagged values of plane z,
+    // by quads of a row with kVec (thread t: row t / 8 % TY, quad t % 8 of plane
+    // t / 64 and every fourth from there), else each thread its own node's
+    auto stage = [&](int z) {
+        copy_a(z + 1);
         if constexpr (kStage) {
-            if (any && live) {
-                const int i = wrap_index(z, P.nz) * nxy + src.yo[1] + src.xo[1];
+            const int zo = wrap_index(z, P.nz) * nxy;
+            if constexpr (kVec) {
+                constexpr int kPer = TY * kBX / 4;   // quads of a plane's column
+                const int row = tid / (kBX / 4) % TY, x4 = x0 + 4 * (tid % (kBX / 4));
+                if (x4 < P.nx && y0 + row < P.ny) {
+                    const int i = zo + (y0 + row) * P.nx + x4, o = row * kBX + 4 * (tid % (kBX / 4));
+#pragma unroll
+                    for (int r = 0; r < (G::NSTG * kPer + NT - 1) / NT; ++r) {
+                        const int q = tid / kPer + r * (NT / kPer);
+                        if (q < G::NSTG)
+                            cp_async16(sStg + q * NT + o,
+                                       (q < 15 ? src.g_ + q * P.plane : src.lag_ + (q - 12) * P.plane) + i);
+                    }
+                }
+            } else if (live) {
+                const int i = zo + src.yo[1] + src.xo[1];
 #pragma unroll
                 for (int p = 0; p < 15; ++p) cp_async4(sStg + p * NT + tid, src.g_ + p * P.plane + i);
 #pragma unroll
@@ -1159,18 +1211,21 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
 
     for (int z = zb - 2; z <= zb + 1; ++z) {
         issue(z, true);
-        c_pass(z, false);
+        c_pass(z);
     }
+    copy_a(zb - 1);
+    copy_a(zb);
     issue(zb + 2, true);
-    stage(zb, true);
     __syncthreads();
     mu_pass(zb - 1);
     mu_pass(zb);
     for (int z = zb; z < ze; ++z) {
-        c_pass(z + 2, true);
+        c_pass(z + 2);
+        __syncthreads();   // C of plane z + 2 is formed, the update of plane z - 1 done
+        stage(z);
         issue(z + 3, z + 1 < ze);
-        __syncthreads();
         mu_pass(z + 1);
+        if constexpr (G::kRaw) cp_async_wait<1>();   // raw(z + 3) may still fly
         __syncthreads();
         if (live) {
 #pragma unroll
@@ -1179,11 +1234,9 @@ __global__ void __launch_bounds__(kBX * TY, (sizeof(T) == 4 && TY <= 8) ? 2 : 1)
                 src.c5[d] = slot5(z - 1 + d);
                 src.m3[d] = slot3(z - 1 + d);
             }
-            if constexpr (kStage) cp_async_wait<1>();   // raw(z + 3) may still fly
             src.gp2 = (z - zb) & 1;
             update_node<T, NP, false>(P, F, cur, nullptr, src);
         }
-        stage(z + 1, z + 1 < ze);
     }
 }
 
