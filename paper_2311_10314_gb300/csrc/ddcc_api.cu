@@ -133,7 +133,7 @@ bool valid_params(const ddcc_params* p) {
 }
 
 struct Layout {
-    size_t pop[2], lag[2], st, C, macro, mu, chi, st64, partial, stage, inflow, mass, flag, total;
+    size_t pop[2], lag[2], st, C, macro, mu, chi, st64, partial, stage, inflow, mass, flag, count, total;
     size_t plane_bytes;
 };
 
@@ -169,6 +169,7 @@ Layout layout_of(const ddcc_params* p) {
     L.inflow = take(es * (size_t)p->ny * N);
     L.mass = take(sizeof(double) * kMaxPhases);
     L.flag = take(sizeof(int) * 4);
+    L.count = L.flag + 2 * sizeof(int);
     L.total = off;
     return L;
 }
@@ -1074,10 +1075,17 @@ int ddcc_save_state(ddcc_handle* h, void* buf, int on_device) {
     char* dst = static_cast<char*>(buf);
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (on_device) {
-        // by value through a launch: a copy from h->steps would have to be
-        // waited for (and left the GPU idle between a small grid's steps and
-        // the two copies below: 256 x 256 FP32, 50 steps and a save, 426 -> 420 us)
-        DDCC_CU(launch_store(reinterpret_cast<long long*>(dst), h->steps, h->stream));
+        // by value through a launch into the workspace and on by a device copy
+        // (buf may have any alignment and sit on another device): a copy from
+        // h->steps would have to be waited for, which left the GPU idle between
+        // a small grid's steps and the two copies below.  The wait also refused
+        // a save under capture, whose replays would all write this step count.
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        DDCC_CU(cudaStreamIsCapturing(h->stream, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return DDCC_ERR_CUDA;
+        long long* slot = reinterpret_cast<long long*>(h->ws + L.count);
+        DDCC_CU(launch_store(slot, h->steps, h->stream));
+        DDCC_CU(cudaMemcpyAsync(dst, slot, sizeof(int64_t), k, h->stream));
     } else {
         std::memcpy(dst, &h->steps, sizeof(int64_t));
     }

@@ -204,3 +204,20 @@ def test_fp64_phase_rates(D, N, rates):
     sim.step(200)
     assert np.abs(sim.mass() - m0).max() <= 1e-13 * np.abs(m0).max()
     sim.close()
+
+
+@pytest.mark.parametrize("off", [0, 1, 4])
+def test_device_save_to_any_address(D, off):
+    """A device save behind queued steps, at any byte offset, and its load."""
+    pb = W.random_problem(65, 21, 3, seed=2, width=6.0)
+    a, b = (D.Sim(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field, precision=D.DDCC_FP32) for _ in range(2))
+    a.step(7)
+    buf = torch.zeros(a.state_bytes() + off, dtype=torch.uint8, device="cuda")[off:]
+    a.save_state(buf)
+    a.step(3)
+    b.load_state(buf)
+    assert b.steps == 7
+    b.step(3)
+    assert np.array_equal(a.fields()["C"], b.fields()["C"])
+    for s in (a, b):
+        s.close()
