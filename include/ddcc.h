@@ -326,8 +326,9 @@ size_t ddcc_adjoint_bytes(const ddcc_handle* h);
  * the ghost rings that the step and ddcc_adjoint_step read (of the phase
  * populations and of plane a), as every state the library writes for that
  * precision has; state_out gets them.  The step-count word of state_out is
- * not written.  Only the fused tile path and the FP64 path provide it: DDCC_ERR_UNSUPPORTED otherwise (the caller
- * then loads, steps and saves).
+ * not written.  Only the fused tile path and, for grids as wide as its boxes
+ * (nx > 24), the FP64 path provide it: DDCC_ERR_UNSUPPORTED otherwise (the
+ * caller then loads, steps and saves).
  */
 int ddcc_step_between(ddcc_handle* h, const void* state_in, void* state_out);
 

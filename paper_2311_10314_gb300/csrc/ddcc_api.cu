@@ -861,11 +861,19 @@ int adjoint_initial_t(ddcc_handle* h, const double* C0, const void* adj0, void* 
     return DDCC_OK;
 }
 
+// Whether the handle steps from buffer to buffer: the fused tile path, and in
+// FP64 the grids that are as wide as its boxes (narrower ones load, step and
+// save in both precisions).
+template <typename T>
+bool steps_between(ddcc_handle* h) {
+    return !h->use_sweep && h->use_tile_tma >= 2 && kp_of<T>(h).pitch >= kTileHaloW;
+}
+
 // One step of the fused tile path from the state in state_in to state_out
 // (both in the saved-state layout), through tensor maps of those buffers.
 template <typename T>
 int step_between_t(ddcc_handle* h, const void* state_in, void* state_out) {
-    if (h->use_sweep || h->use_tile_tma < 2 || (h->prm.flags & DDCC_FLAG_OPEN_X)) return DDCC_ERR_UNSUPPORTED;
+    if (!steps_between<T>(h) || (h->prm.flags & DDCC_FLAG_OPEN_X)) return DDCC_ERR_UNSUPPORTED;
     KParams<T>& k = kp_of<T>(h);
     Fields<T>& f = fd_of<T>(h);
     size_t pb, lb;
@@ -1333,7 +1341,8 @@ int ddcc_adjoint_segment_pipelined(ddcc_handle* h, const void* const* states, in
         for (int s = 0; s < n; ++s)
             if (next[t] == states[s]) return DDCC_ERR_PARAM;
     }
-    if (n_next > 1 && (h->use_sweep || h->use_tile_tma < 2)) return DDCC_ERR_UNSUPPORTED;
+    if (n_next > 1 && !(h->prm.precision == DDCC_FP64 ? steps_between<double>(h) : steps_between<float>(h)))
+        return DDCC_ERR_UNSUPPORTED;
     if (n_next > 1 && !h->side) {
         // all three or none
         cudaStream_t side = nullptr;
