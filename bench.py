@@ -137,7 +137,8 @@ def ncu_record(kind, key, path=os.path.join(ROOT, "profiles", "ncu_traffic.json"
     with open(path) as fh:
         d = json.load(fh)
     entry = d.get(kind)
-    files = ("ddcc3d.cu",) if "_3d" in kind else None
+    files = (("ddcc3d.cu", "ddcc_device.cuh") if "_3d" in kind
+             else ("ddcc_fp64.cu", "ddcc_device.cuh", "ddcc_internal.h") if "fp64" in kind else None)
     if not entry or entry.get("source_hash") != (kernel_source_hash(files) if files else kernel_source_hash()):
         return None
     return float(entry[key])

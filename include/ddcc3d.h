@@ -81,8 +81,9 @@ typedef struct ddcc3d_handle ddcc3d_handle;
  * invalid: two copies of the populations (7(N-1) D3Q7 planes and 15
  * D3Q15 planes) and of the 3N + 7 lagged planes (a_xy, a_yz, a_zx, (psi C_i u)_{x,y,z},
  * T_{xx,yy,zz,xy,yz,zx}, psi m.u), psi, the angle field, the volume
- * fractions and chemical potentials of the current step, read-out and
- * reduction scratch.  Each plane is nx*ny*nz elements of the precision,
+ * fractions and chemical potentials of the current step, in FP64 also psi
+ * rho and five planes formed from psi at create (1 / psi, grad psi and
+ * 3 |grad psi|), read-out and reduction scratch.  Each plane is nx*ny*nz elements of the precision,
  * rounded up to 256 bytes.
  */
 size_t ddcc3d_workspace_bytes(const ddcc3d_params* params);
@@ -120,8 +121,9 @@ int ddcc3d_step(ddcc3d_handle* h, int64_t nsteps);
  * compute it (nx*ny*nz doubles to host_out): DDCC_FIELD_C + i and
  * DDCC_FIELD_MU + i (i < N), DDCC_FIELD_RHO, DDCC_FIELD_UX, DDCC_FIELD_UY,
  * DDCC_FIELD_UZ, DDCC_FIELD_P, DDCC_FIELD_PSI.  Synchronises the stream.
- * C and mu of a state are formed on its first read and kept until the next
- * ddcc3d_step.
+ * C and mu of a state are formed on its first read, rho, u and P on the first
+ * read of one of them (into planes of the population copy that the next step
+ * overwrites), and all are kept until the next ddcc3d_step.
  */
 int ddcc3d_read(ddcc3d_handle* h, int field, double* host_out);
 
