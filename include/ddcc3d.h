@@ -37,9 +37,11 @@ extern "C" {
 #define DDCC_FIELD_UZ 21            /* velocity z                              */
 
 /* ddcc3d_params.flags: how ddcc3d_step runs (the same arithmetic either
- * way).  0: the fused kernel in FP32, the three kernels in FP64 (where the
- * fused kernel's recomputed halo chemical potentials cost more FP64 work
- * than the saved traffic); SPLIT or FUSED force one; not both. */
+ * way).  0: the fused kernel in FP32 (the three kernels for N >= 3 where nx is
+ * above 32 and no multiple of 4, whose rows the fused kernel copies value by
+ * value), the three kernels in FP64 (where the fused kernel's recomputed halo
+ * chemical potentials cost more FP64 work than the saved traffic); SPLIT or
+ * FUSED force one; not both. */
 #define DDCC3D_FLAG_SPLIT 1u
 #define DDCC3D_FLAG_FUSED 2u
 

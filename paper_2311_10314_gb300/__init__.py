@@ -134,7 +134,8 @@ class Sim3D:
     (nz, ny, nx), ``C0`` (N-1, nz, ny, nx), ``cos_theta`` (N-1,) or
     ``cos_theta_field`` (N-1, nz, ny, nx); float64 host arrays.  ``path``
     "fused" (one kernel per step), "split" (three kernels) or "auto"
-    (fused in FP32, split in FP64)."""
+    (fused in FP32, but for N >= 3 where nx is above 32 and no multiple of 4;
+    split there and in FP64)."""
 
     def __init__(self, params, psi, C0, cos_theta=None, cos_theta_field=None,
                  precision=DDCC_FP64, stream=None, path="auto"):

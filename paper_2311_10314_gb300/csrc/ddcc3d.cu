@@ -1589,6 +1589,17 @@ int order_mu(ddcc3d_handle* h, const P3<T>& K, const F3<T>& F, bool order) {
     return DDCC_OK;
 }
 
+// Whether FP32 takes the fused step where the caller leaves the choice: for
+// rows of whole quads, for N = 2, and for boxes of one column in x, where a
+// small step's three launches weigh most.  With other rows every population is
+// copied by itself (and a C is formed node by node), which from N = 3 costs
+// more than the fields' way through memory that the fused step saves (us a
+// step, fused and three kernels; N = 3: 33 x 32 x 32 19.8 and 16.6, 101 x 77 x
+// 63 101 and 88, 131 x 97 x 100 255 and 199, 255 x 256 x 200 1829 and 1616; N =
+// 4: 26.7 and 18.5, 140 and 111, 350 and 260, 2553 and 2117; N = 2 within 13%
+// either way, 1043 and 1101 at the largest; 25 x 31 x 31, N = 3, 12.4 and 15.0).
+bool fused_pays(const ddcc3d_params* p) { return p->nx % 4 == 0 || p->nphase == 2 || p->nx <= kBX; }
+
 // Shared memory of the fused step and its z chunks: the count of chunks n
 // minimises (waves of CTAs) x (planes a CTA forms C for), i.e.
 // ceil(columns n / resident CTAs) x (ceil(nz / n) + 3).
@@ -1816,7 +1827,7 @@ int ddcc3d_create(const ddcc3d_params* params, void* dev_workspace, size_t bytes
     // FP32 steps fused by default; FP64 with the three kernels (its fused
     // kernel recomputes mu on the column halos and is bound by the FP64 pipe)
     h->fused = (params->flags & DDCC3D_FLAG_FUSED) ||
-               (!(params->flags & DDCC3D_FLAG_SPLIT) && params->precision == DDCC_FP32);
+               (!(params->flags & DDCC3D_FLAG_SPLIT) && params->precision == DDCC_FP32 && fused_pays(params));
     h->nchunk = 1;
     int rc;
     if (params->precision == DDCC_FP64) {

@@ -221,3 +221,25 @@ def test_device_save_to_any_address(D, off):
     assert np.array_equal(a.fields()["C"], b.fields()["C"])
     for s in (a, b):
         s.close()
+
+
+@pytest.mark.parametrize("nx,N,path", [(32, 3, "fused"), (33, 2, "fused"), (33, 3, "split"), (34, 4, "split"),
+                                       (31, 4, "fused"), (36, 4, "fused")])
+def test_3d_default_path_in_fp32(D, nx, N, path):
+    """The path taken where the caller leaves the choice, bit for bit that of
+    the forced one, and both paths against the oracle."""
+    pb = W.random_problem_3d(nx, 9, 7, N, seed=nx, theta_field=True, width=5.0)
+    sims = [D.Sim3D(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field, precision=D.DDCC_FP32, path=p)
+            for p in ("auto", path)]
+    for s in sims:
+        s.step(5)
+    v = [np.stack([s.read(k) for k in (*range(D.FIELD_C, D.FIELD_C + N), D.FIELD_UX, D.FIELD_UY)]) for s in sims]
+    assert np.array_equal(*v)
+    o = Oracle3D(pb.params, pb.psi, pb.C0, pb.cos_theta, pb.cos_theta_field)
+    o.step(5)
+    ref = {k: t.numpy() for k, t in o.macroscopic().items()}
+    fl = pb.psi >= 0.01
+    assert np.abs(ref["C"] - v[0][:N])[:, fl].max() <= 2e-5
+    assert max(np.abs(ref[k] - v[0][N + j])[fl].max() for j, k in enumerate(("ux", "uy"))) <= 1e-6
+    for s in sims:
+        s.close()
