@@ -95,7 +95,7 @@ int prof_end(ddcc_handle* h) {
 
 constexpr size_t kAlign = 256;
 // half of the 129 MB L2: a step reads one state and writes another
-constexpr long long kWideStateBytes = 64LL << 20;
+constexpr long long kWideStateBytes = 128LL << 20;
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -411,8 +411,11 @@ int setup_sweep(ddcc_handle* h) {
 // this kernel's loads and stores and no arithmetic takes 1.04 ms instead of
 // 1.19 (stores alone: 1.20 ms in 32 x 8 tiles, 0.86 in 128 x 2), and the step
 // 1.177 instead of 1.270 (1021 x 1024, N = 3: 71.0 instead of 72.5 us).
-// Smaller states stay in L2, where the 32 x 8 tile's smaller halo counts
-// (256 x 256, N = 3: 10.3 us a step against 11.2).  More rows of tiles than
+// Smaller states stay in L2, where the 32 x 8 tile's smaller halo counts and
+// its step is one launch (us a step, 32 x 8 and 64 x 4: 704 x 700, N = 3, 68
+// MB, 37.5 and 38.7; 1024 x 1024, N = 2, 100 MB, 52.0 and 53.0; 97 x 9000, N =
+// 2, 83 MB, 69.9 and 72.8; at 144 MB, N = 3, 72.2 and 70.8; at 188 MB, N = 4,
+// 94.7 and 89.0).  More rows of tiles than
 // a launch grid has keep the taller tile.
 template <typename T>
 bool fused_tile_wide(const ddcc_params& p) {

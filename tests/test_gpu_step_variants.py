@@ -41,14 +41,14 @@ def _against_oracle(D, pb, precision, steps, **kw):
 
 
 @pytest.mark.parametrize("nx,ny,N,py,field", [
-    (64, 5601, 4, 1, True),      # one tile wide, one row over a tile
-    (191, 1871, 4, 0, False),    # a column short of three tiles, walls
-    (256, 2300, 3, 1, True),
-    (641, 1201, 2, 0, True),     # one column into the eleventh tile
+    (64, 11201, 4, 1, True),     # one tile wide, one row over a tile
+    (191, 3751, 4, 0, False),    # a column short of three tiles, walls
+    (256, 3700, 3, 1, True),
+    (641, 2101, 2, 0, True),     # one column into the eleventh tile
 ])
 def test_fp32_wide_tiles(D, nx, ny, N, py, field):
-    """States beyond L2 (over 64 MB) take the 64 x 4 tiles in FP32."""
-    assert nx * ny * (11 * N + 3) * 4 > 64 << 20
+    """States beyond L2 (over 128 MB) take the 64 x 4 tiles in FP32."""
+    assert nx * ny * (11 * N + 3) * 4 > 128 << 20
     pb = W.random_problem(nx, ny, N, seed=nx + N, periodic_y=py, theta_field=field, width=6.0, n_circles=12, n_drops=9)
     _against_oracle(D, pb, D.DDCC_FP32, 3)
 
