@@ -204,7 +204,7 @@ __device__ __forceinline__ int ring_index(int v, int n, int periodic) {
 // to its copies in the ghost ring.  From the populations, or (kC0) from the
 // C planes themselves, as the initial state's reverse has them.
 template <typename T, int NP, bool kC0>
-__global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_fields(KParams<T> P, const T* __restrict__ f,
+__global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_fields(KParams<T> P, const T* f,
                                                                      const T* __restrict__ psi,
                                                                      const T* __restrict__ cosf, T* C,
                                                                      T* __restrict__ mu, T* __restrict__ chi) {
@@ -283,8 +283,8 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_fields(KParams<T> 
 
 template <typename T, int NP>
 __global__ void __launch_bounds__(AX * block_rows<T>(), sizeof(T) == 4 ? 2 : 4)
-    k_adj_node(KParams<T> P, const T* __restrict__ psi_pl, const T* __restrict__ st_pop,
-               const T* __restrict__ st_lag, const T* __restrict__ ad_pop_in, const T* __restrict__ ad_lag_in,
+    k_adj_node(KParams<T> P, const T* __restrict__ psi_pl, const T* st_pop,
+               const T* st_lag, const T* ad_pop_in, const T* ad_lag_in,
                T* __restrict__ ad_pop_out, T* __restrict__ ad_lag_out, AdjPlanes<T, NP> W) {
     constexpr int M = NP - 1, NM = mu_planes<NP>();
     if constexpr (overlaps<T>()) {
@@ -695,9 +695,10 @@ __global__ void __launch_bounds__(AX * block_rows<T>(), sizeof(T) == 4 ? 2 : 4)
 // gives the node (x, 0) by c_py = +1; scalars carry over unchanged.  (With
 // zeros beyond the edge and the images gathered from memory by the edge
 // nodes, gather3 took 18.6 us at 256 x 256 in FP32, N = 2, and gather2 11.)
-// The planes are read through the read-only path (no kernel that loads a
-// ring writes those planes), so the loads need not wait for the earlier
-// shared-memory stores and are all in flight at once.
+// Plain loads, all of a call's before its first shared-memory store, so that
+// they are in flight at once.  (Not the read-only path: the kernel before
+// this one may still write these planes when this one starts, see
+// wait_for_previous.)
 template <typename T>
 struct Ring {
     static constexpr int AY = block_rows<T>(), W = AX + 2, H = AY + 2, N = W * H, NT = AX * AY, R = (N + NT - 1) / NT;
@@ -716,14 +717,14 @@ struct Ring {
     }
 };
 template <typename T, int NPL, bool kPairs>
-__device__ __forceinline__ void load_ring(const KParams<T>& P, const Ring<T>& ring, T* sm, const T* __restrict__ base) {
+__device__ __forceinline__ void load_ring(const KParams<T>& P, const Ring<T>& ring, T* sm, const T* base) {
     using R = Ring<T>;
     const int tid = threadIdx.y * AX + threadIdx.x;
     T v[R::R][NPL];
 #pragma unroll
     for (int r = 0; r < R::R; ++r)
 #pragma unroll
-        for (int q = 0; q < NPL; ++q) v[r][q] = __ldg(base + q * P.plane + ring.g[r]);
+        for (int q = 0; q < NPL; ++q) v[r][q] = base[q * P.plane + ring.g[r]];
 #pragma unroll
     for (int r = 0; r < R::R; ++r) {
         const int k = min(tid + r * R::NT, R::N - 1);
@@ -751,7 +752,7 @@ __device__ __forceinline__ T grad_T_sm(const KParams<T>& P, const T* vx, const T
 template <typename T, int NP>
 __device__ __forceinline__ void mu_node_at(const KParams<T>& P, const T* __restrict__ psi_pl,
                                            const T* __restrict__ cosf, const AdjPlanes<T, NP>& W,
-                                           double* __restrict__ dJ_dcos, int x, int y,
+                                           double* dJ_dcos, int x, int y,
                                            const T (&Lmu_kept)[mu_planes<NP>()]);
 
 // kMu: the chemical-potential VJP (mu_node_at) of the node follows in the
@@ -760,7 +761,7 @@ __device__ __forceinline__ void mu_node_at(const KParams<T>& P, const T* __restr
 template <typename T, int NP, bool kMu>
 __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather3(KParams<T> P, const T* __restrict__ psi_pl,
                                                      AdjPlanes<T, NP> W, T* __restrict__ ad_lag_out,
-                                                     const T* __restrict__ cosf, double* __restrict__ dJ_dcos) {
+                                                     const T* __restrict__ cosf, double* dJ_dcos) {
     constexpr int NM = mu_planes<NP>(), NV = AdjPlanes<T, NP>::NV, RN = Ring<T>::N;
     extern __shared__ __align__(16) unsigned char g3_raw[];
     T* sm = reinterpret_cast<T*>(g3_raw);
@@ -804,7 +805,7 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather3(KParams<T>
 template <typename T, int NP>
 __device__ __forceinline__ void mu_node_at(const KParams<T>& P, const T* __restrict__ psi_pl,
                                            const T* __restrict__ cosf, const AdjPlanes<T, NP>& W,
-                                           double* __restrict__ dJ_dcos, int x, int y,
+                                           double* dJ_dcos, int x, int y,
                                            const T (&Lmu_kept)[mu_planes<NP>()]) {
     const long long pl = P.plane;
     const long long o = P.org + (long long)y * P.pitch + x;
@@ -970,8 +971,8 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_mu_node(KParams<T>
 // Ring copies: grad psi pair, mL_j (N-1), psi, C_j (N-1).
 template <typename T, int NP>
 __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather2(KParams<T> P, const T* __restrict__ psi_pl,
-                                                     AdjPlanes<T, NP> W, T* __restrict__ ad_pop_out,
-                                                     double* __restrict__ dJ_dpsi, int initial) {
+                                                     AdjPlanes<T, NP> W, T* ad_pop_out,
+                                                     double* dJ_dpsi, int initial) {
     extern __shared__ __align__(16) unsigned char g2_raw[];
     constexpr int RN = Ring<T>::N, RW = Ring<T>::W;
     T* sm = reinterpret_cast<T*>(g2_raw);

@@ -27,7 +27,13 @@ constexpr int kGY = 6;
 // (wait_for_previous) ahead of its first access to memory that another kernel
 // writes.  Every kernel launched with overlap executes that wait in all its
 // threads, so the order of a stream holds across any number of them; launched
-// without, both calls do nothing.  The FP64 kernels do without: the waiting
+// without, both calls do nothing.  What another kernel writes is read by plain
+// loads through pointers without __restrict__, or by tensor copies: while this
+// kernel is resident the one before it may still be writing, so neither the
+// read-only path (__ldg, const __restrict__) nor the compiler's licence to
+// move loads through a __restrict__ pointer across the wait applies.  Only
+// planes that no kernel of a step writes (psi, the angles, the inflow) and
+// pointers that a kernel only stores through are __restrict__.  The FP64 kernels do without: the waiting
 // blocks of the next kernel take the places that keep the running one's
 // warps even over the SMs (300 x 170, N = 3: 74 us a step without, 89 and more
 // with).

@@ -836,7 +836,7 @@ __global__ void k_fill_ghosts(GhostRing<T> g0, GhostRing<T> g1, KParams<T> P) {
 // a go to the node's copies in the 2-node ghost ring too.
 constexpr int kOpenThreads = 32;
 template <typename T, int NP>
-__global__ void __launch_bounds__(kOpenThreads) k_open_bc(KParams<T> P, T* __restrict__ pop, T* __restrict__ lag,
+__global__ void __launch_bounds__(kOpenThreads) k_open_bc(KParams<T> P, T* pop, T* lag,
                                                           const T* __restrict__ psi, const T* __restrict__ inflow) {
     dependents_may_start();
     wait_for_previous();
