@@ -37,6 +37,7 @@ namespace ddcc {
 namespace {
 
 using dev::map_index;
+using dev::ring_step;
 
 constexpr int AX = 32;   // threads (and nodes) along x of every kernel here
 // Rows of a block.  FP64 is bound by FP64 warp instructions per SM
@@ -183,14 +184,6 @@ struct AdjPlanes {
     __host__ __device__ static constexpr int planes() { return 7 * (NP - 1) + 5 * NM + 11 + (sizeof(T) == 8 ? 1 : 0); }
 };
 
-// The copies of coordinate v (0 .. n-1) in the 1-node ghost ring, as steps
-// from v: periodic 0 -> n and n-1 -> -1, mirror 0 -> -1 and n-1 -> n; 0: none
-// (n >= 3: at most one along an axis).
-__device__ __forceinline__ int ring_step(int v, int n, int periodic) {
-    if (v == 0) return periodic ? n : -1;
-    if (v == n - 1) return periodic ? -n : 1;
-    return 0;
-}
 // Coordinate v in [-1, n] of the ring taken into the domain (values of v
 // beyond, in the unused part of a block, land anywhere inside).
 __device__ __forceinline__ int ring_index(int v, int n, int periodic) {

@@ -35,6 +35,15 @@ __device__ __forceinline__ int map_index(int g, int n, int periodic) {
     return m >= n ? n2 - 1 - m : m;
 }
 
+// The image of coordinate v (0 .. n-1) in the one-node ghost ring, as a step
+// from v: periodic 0 -> n and n-1 -> -1, mirror 0 -> -1 and n-1 -> n; 0: none
+// (n >= 3, so a node has at most one image along an axis).
+__device__ __forceinline__ int ring_step(int v, int n, int periodic) {
+    if (v == 0) return periodic ? n : -1;
+    if (v == n - 1) return periodic ? -n : 1;
+    return 0;
+}
+
 // g(C) = C^2 (C - 1)^2  =>  g'(C) = 2 C (C - 1) (2 C - 1)  (Sec. 2.1), with
 // every factor exact to a rounding near its own root.
 template <typename T>

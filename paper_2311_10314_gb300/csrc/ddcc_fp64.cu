@@ -32,6 +32,7 @@ namespace ddcc {
 namespace {
 
 using dev::map_index;
+using dev::ring_step;
 using Real = double;
 
 constexpr int FX = 32, FY = 4, FT = FX * FY;   // threads (and nodes) of k_fields64
@@ -169,15 +170,6 @@ struct Sink64 {
         mac[(NP + 3) * plane + o] = Pr;
     }
 };
-
-// The image of coordinate v (0 .. n-1) in the one-node ghost ring, as a step
-// from v: periodic 0 -> n and n-1 -> -1, mirror 0 -> -1 and n-1 -> n; 0: none
-// (n >= 3, so a node has at most one image along an axis).
-__device__ __forceinline__ int ring_step(int v, int n, int periodic) {
-    if (v == 0) return periodic ? n : -1;
-    if (v == n - 1) return periodic ? -n : 1;
-    return 0;
-}
 
 template <int NP, int MODE, bool kOneRate>
 __global__ void __launch_bounds__(UT, 5) k_update64(KParams<Real> P, Step64Args F) {

@@ -139,6 +139,23 @@ struct TileSink {
     }
 };
 
+// The sink of k_step: its state's readers take the one-node ghost ring of the
+// lagged plane a from the state (the reverse step, and a load into a handle of
+// another path), so the plane is written with its images.
+template <typename T, int NP>
+struct PlainSink : TileSink<T, NP> {
+    long long ax, ay;   // offsets of a's images (0: none)
+    __device__ void lag_out(int k, T v) {
+        T* q = this->lout + k * this->plane + this->o;
+        *q = v;
+        if (k == 0) {
+            if (ax) q[ax] = v;
+            if (ay) q[ay] = v;
+            if (ax && ay) q[ax + ay] = v;
+        }
+    }
+};
+
 // D2Q9 velocity components as compile-time functions of p (after unrolling
 // they fold into the addresses).
 __host__ __device__ constexpr int cxp(int p) { return (p == 1 || p == 5 || p == 8) ? 1 : (p == 3 || p == 6 || p == 7) ? -1 : 0; }
@@ -254,7 +271,7 @@ __global__ void __launch_bounds__(NT) k_step(KParams<T> P, Fields<T> F, int cur)
     const long long o = P.org + (long long)y * P.pitch + x;
     TileAcc<T, NP> acc{P, sm, (int)threadIdx.y + 2, (int)threadIdx.x + 2, (int)threadIdx.y + 1,
                        (int)threadIdx.x + 1, o, P.plane, lag_in, fin, gin};
-    TileSink<T, NP> sink;
+    PlainSink<T, NP> sink;
     sink.o = o;
     sink.plane = P.plane;
     sink.fout = fout;
@@ -262,7 +279,9 @@ __global__ void __launch_bounds__(NT) k_step(KParams<T> P, Fields<T> F, int cur)
     sink.lout = lag_out;
     sink.macro_out = F.macro;
     if (MODE == 0) {
-        tile_targets(P, x, y, o, sink);
+        tile_targets<T, NP>(P, x, y, o, sink);
+        sink.ax = dev::ring_step(x, P.nx, P.px);
+        sink.ay = (long long)dev::ring_step(y, P.ny, P.py) * P.pitch;
     }
     dev::node_update<T, NP, MODE>(P, acc, sink);
 }
