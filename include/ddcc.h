@@ -455,6 +455,15 @@ int ddcc_phase_mass_noalloc(const void* dev_populations, int precision, int npha
 int ddcc_selftest_bounded_wait(void* cuda_stream, int* dev_flag, int deliver);
 
 /*
+ * Self-test of the FP64 reciprocal, square root and max(x, 0) that the
+ * kernels use in place of the operators: for the n arguments at dev_x
+ * (device), dev_out (device, 5n doubles) receives 1 / x, sqrt(x), max(x, 0)
+ * and the hardware seeds of 1 / x and 1 / sqrt(x), n values each.
+ * Asynchronous on the stream.
+ */
+int ddcc_selftest_math64(void* cuda_stream, const double* dev_x, double* dev_out, int64_t n);
+
+/*
  * Measured FP64 fused multiply-add rate of the current device in TFLOP/s
  * (2 flops per FMA), written to *tflops_out (host): the denominator of the
  * FP64 step's roofline, which the FP64 units bound on this GPU.  The paper

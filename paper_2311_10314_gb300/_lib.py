@@ -41,7 +41,7 @@ EXPORTED = (
     "ddcc_phase_mass_noalloc", "ddcc_step_path", "ddcc_adjoint_bytes", "ddcc_adjoint_step",
     "ddcc_adjoint_initial", "ddcc_objective_centroid", "ddcc_step_between", "ddcc_create_walls",
     "ddcc_set_inflow", "ddcc_adjoint_segment", "ddcc_adjoint_segment_pipelined",
-    "ddcc_selftest_bounded_wait", "ddcc_measure_fp64_peak", "ddcc_rows_bytes", "ddcc_get_rows", "ddcc_set_rows",
+    "ddcc_selftest_bounded_wait", "ddcc_selftest_math64", "ddcc_measure_fp64_peak", "ddcc_rows_bytes", "ddcc_get_rows", "ddcc_set_rows",
 )
 # every symbol include/ddcc3d.h declares
 EXPORTED_3D = (
@@ -167,6 +167,8 @@ def load():
     lib.ddcc_adjoint_segment_pipelined.restype = C.c_int
     lib.ddcc_selftest_bounded_wait.argtypes = [vp, vp, C.c_int]
     lib.ddcc_selftest_bounded_wait.restype = C.c_int
+    lib.ddcc_selftest_math64.argtypes = [vp, vp, vp, C.c_int64]
+    lib.ddcc_selftest_math64.restype = C.c_int
     lib.ddcc_measure_fp64_peak.argtypes = [vp, vp, dp]
     lib.ddcc_measure_fp64_peak.restype = C.c_int
     lib.ddcc_rows_bytes.argtypes = [vp, C.c_int]
@@ -466,6 +468,10 @@ def ddcc_measure_fp64_peak(stream: int, dev_sink: int) -> float:
     if st != DDCC_OK:
         raise DdccError(st, "ddcc_measure_fp64_peak")
     return float(out.value)
+
+
+def ddcc_selftest_math64(stream: int, dev_x: int, dev_out: int, n: int) -> int:
+    return int(load().ddcc_selftest_math64(C.c_void_p(stream), C.c_void_p(dev_x), C.c_void_p(dev_out), int(n)))
 
 
 def ddcc_selftest_bounded_wait(stream: int, dev_flag: int, deliver: bool) -> int:

@@ -326,10 +326,10 @@ __global__ void __launch_bounds__(node_threads<T>()) k3_static(P3<T> P, F3<T> F)
     const long long i0 = s.self();
     T g[3];
     grad15(P, [&](int p) { return F.psi[s.at(cx(p), cy(p), cz(p))]; }, g);
-    F.st[kInvPsi * P.plane + i0] = rcp(F.psi[i0]);
+    F.st[kInvPsi * P.plane + i0] = T(1) / F.psi[i0];
 #pragma unroll
     for (int a = 0; a < 3; ++a) F.st[(kGrad + a) * P.plane + i0] = g[a];
-    F.st[kAgp3 * P.plane + i0] = T(3) * root(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+    F.st[kAgp3 * P.plane + i0] = T(3) * sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
 }
 
 // The same chemical potentials for four consecutive x nodes per thread

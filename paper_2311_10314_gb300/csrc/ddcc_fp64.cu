@@ -53,11 +53,11 @@ __global__ void k_static64(KParams<Real> P, const Real* __restrict__ psi, Real* 
         const long long o = P.org + (long long)y * P.pitch + x;
         Real gx, gy;
         dev::grad9(P, [&](int dy, int dx) { return psi[o + (long long)dy * P.pitch + dx]; }, gx, gy);
-        st[kInvPsi * P.plane + o] = dev::rcp(psi[o]);
+        st[kInvPsi * P.plane + o] = 1.0 / psi[o];
         st[kGradX * P.plane + o] = gx;
         st[kGradY * P.plane + o] = gy;
         // with several solids the angle planes already carry |grad psi_k|
-        st[kAgp3 * P.plane + o] = P.wet_field ? 3.0 : 3.0 * dev::root(gx * gx + gy * gy);
+        st[kAgp3 * P.plane + o] = P.wet_field ? 3.0 : 3.0 * sqrt(gx * gx + gy * gy);
     }
 }
 

@@ -5,7 +5,10 @@
 // deliver (nothing is in flight, so nothing can land after the kernel ends)
 // and waits on it with a short poll limit; its control case arrives without
 // expecting bytes and completes at once.
+//
+// And of the FP64 reciprocal, square root and clamp of the node update.
 #include "ddcc.h"
+#include "ddcc_device.cuh"
 #include "ddcc_tma.cuh"
 
 namespace ddcc {
@@ -28,8 +31,28 @@ __global__ void k_wait_selftest(int* __restrict__ err, int deliver, unsigned lim
     if (!__syncthreads_and(ok) && threadIdx.x == 0) atomicOr(err, 1);
 }
 
+__global__ void k_math_selftest(const double* __restrict__ x, double* __restrict__ out, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const double v = x[i];
+        double r, y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+        out[i] = dev::rcp(v);
+        out[n + i] = dev::root(v);
+        out[2 * n + i] = dev::clamp0(v);
+        out[3 * n + i] = r;
+        out[4 * n + i] = y;
+    }
+}
+
 }  // namespace
 }  // namespace ddcc
+
+extern "C" int ddcc_selftest_math64(void* cuda_stream, const double* dev_x, double* dev_out, int64_t n) {
+    if (!dev_x || !dev_out || n < 1) return DDCC_ERR_PARAM;
+    ddcc::k_math_selftest<<<304, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(dev_x, dev_out, n);
+    return cudaGetLastError() == cudaSuccess ? DDCC_OK : DDCC_ERR_CUDA;
+}
 
 extern "C" int ddcc_selftest_bounded_wait(void* cuda_stream, int* dev_flag, int deliver) {
     if (!dev_flag) return DDCC_ERR_PARAM;
