@@ -243,6 +243,7 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
     k.one_rate = p->s_f[1] == p->s_f[2] && p->s_f[1] == p->s_f[3] && p->s_f[1] == p->s_f[4];
     k.sf = (T)p->s_f[1];
     k.one_m_sf = (T)(1.0 - p->s_f[1]);
+    k.cse = (T)(p->s_f[1] * 4.0 * ((double)k.w9[1] + (double)k.w9[2]));
     k.lg00 = (T)(p->s_g[0]);
     k.lg1 = (T)(p->s_g[1] / n1);
     k.cg0 = (T)(0.5 * p->s_g[0] - 1.0);

@@ -329,11 +329,15 @@ __device__ __forceinline__ void hermite_relax_back(const T k[9], const KParams<T
 // X = psi C - emu:
 //   out_p = (1 - s) v_p + w_p (s emu + c_p . q) + s X delta_p0,
 //   q = s j / cs2 - k_1,  k_1 = lambda_1 (j - psi C u) + cV V.
-// 26 FP64 instructions a phase less than the transforms (FP64 only: FP32 is
-// bound by memory).  The rest population's exchange and its rounding error
-// are treated as in hermite_relax_back.
+// What the rest population gives, t_0 = v_0 - out_0 = s (1 - w_0) emu - s m,
+// is formed from the sum m of the moving populations: with psi C in its
+// place the node's mass would change by s times the rounding of that sum
+// (5e-17 rms at psi C = 1; so it is of the order of m's rounding, 2e-20 at
+// moving populations of 1e-3).  Its rounding error is treated as in
+// hermite_relax_back.  28 FP64 instructions a phase less than the transforms
+// (FP64 only: FP32 is bound by memory).
 template <typename T>
-__device__ __forceinline__ void relax_one_rate(const KParams<T>& P, int i, const T v[9], T jx, T jy, T psiC, T emu,
+__device__ __forceinline__ void relax_one_rate(const KParams<T>& P, int i, const T v[9], T jx, T jy, T moving, T emu,
                                                T pcux, T pcuy, T Vx, T Vy, T out[9]) {
     const T lam = P.lamf[i][1];
     const T qx = P.qf[i] * jx + lam * pcux - P.cV[i] * Vx;
@@ -342,7 +346,7 @@ __device__ __forceinline__ void relax_one_rate(const KParams<T>& P, int i, const
     const T a = P.w9[1] * se, ax = P.w9[1] * qx, ay = P.w9[1] * qy;
     const T d = P.w9[2] * se, dp = P.w9[2] * (qx + qy), dm = P.w9[2] * (qx - qy);
     const T k = P.one_m_sf;
-    const T t0 = P.sf * (v[0] - (psiC - emu)) - P.w9[0] * se;
+    const T t0 = P.cse * emu - P.sf * moving;
     const T o0 = add_rn(v[0], -t0);
     const T bb = add_rn(o0, -v[0]);                 // TwoSum(v_0, -t_0)
     const T half = T(0.5) * add_rn(add_rn(v[0], -add_rn(o0, -bb)), add_rn(-t0, -bb));
@@ -508,7 +512,7 @@ __device__ __forceinline__ void node_update(const KParams<T>& P, const Acc& A, S
     // ---- phase LB, Eqs. 3.1, 3.5-3.7 ---------------------------------------
 #pragma unroll
     for (int i = 0; i < NP - 1; ++i) {
-        T v[9], m[9], k[9], o9[9];
+        T v[9], m[9], k[9], o9[9], moving;
 #pragma unroll
         for (int p = 0; p < 9; ++p) v[p] = A.f(i, p);
         if constexpr (kOneRate) {
@@ -516,9 +520,10 @@ __device__ __forceinline__ void node_update(const KParams<T>& P, const Acc& A, S
             m[1] = (v[1] - v[3]) + (d1 + d2);
             m[2] = (v[2] - v[4]) + (d1 - d2);
             // in the order of hermite_moments
-            m[0] = (((v[7] + v[8]) + v[4]) + (v[3] + v[1]) + ((v[6] + v[5]) + v[2])) + v[0];
+            moving = ((v[7] + v[8]) + v[4]) + (v[3] + v[1]) + ((v[6] + v[5]) + v[2]);
+            m[0] = moving + v[0];
         } else {
-            hermite_moments(v, cs2, m);
+            moving = hermite_moments(v, cs2, m);
         }
         const T psiC = m[0];
         const T pcux = psiC * ux, pcuy = psiC * uy;
@@ -527,7 +532,7 @@ __device__ __forceinline__ void node_update(const KParams<T>& P, const Acc& A, S
         const T Vy = (pcuy - A.lag(2 + 2 * i)) + P.ceta[i] * (mu[i] * gpy + psi * (gmy[i] - Qy[i]));
         if constexpr (kOneRate) {
             const T emu = P.eta[i] * (psi * mu[i]);
-            relax_one_rate(P, i, v, m[1], m[2], psiC, emu, pcux, pcuy, Vx, Vy, o9);
+            relax_one_rate(P, i, v, m[1], m[2], moving, emu, pcux, pcuy, Vx, Vy, o9);
         } else {
             const T X = psiC - P.eta[i] * psi * mu[i];
             const T* lam = P.lamf[i];

@@ -94,9 +94,10 @@ struct KParams {
     T lamf[kMaxPhases][9];
     T invN[9];
     // one rate for the moments of second and higher order: that rate, 1 less it,
-    // and rate / cs2 - lambda_1 per phase
+    // rate times the moving directions' weights 1 - w_0, and rate / cs2 -
+    // lambda_1 per phase
     int one_rate;
-    T sf, one_m_sf, qf[kMaxPhases];
+    T sf, one_m_sf, cse, qf[kMaxPhases];
     // flow LB constant rates as lambda = s / N (00, 10, 01, 21, 12, 22)
     T lg00, lg1, lg3, lg4;
     T cg0, cg1;                   // lg00 / 2 - 1 and lg1 / 2 - 1 / N_1
