@@ -205,6 +205,14 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
     k.w1d[0] = (T)(d0 / 2.0);
     k.w1d[1] = (T)(1.0 - d0);
     k.w1d[2] = (T)(d0 / 2.0);
+    // the phases' weights are products of the rounded 1D weights, not roundings
+    // of the products: the sums over them that must vanish for the phase mass
+    // (sum_p w_p h_ab(c_p)) then factor into 1D sums, which vanish as well as
+    // w1d and cs2 allow (FP32, d0 = 0.3, populations far from equilibrium:
+    // mean change of a node's sum 3e-11 instead of 9.6e-10)
+    k.wf[0] = k.w1d[1] * k.w1d[1];
+    k.wf[1] = k.w1d[1] * k.w1d[2];
+    k.wf[2] = k.w1d[2] * k.w1d[2];
     for (int i = 0; i < N; ++i) {
         k.rho[i] = (T)p->rho[i];
         k.nu[i] = (T)p->nu[i];
@@ -243,7 +251,7 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
     k.one_rate = p->s_f[1] == p->s_f[2] && p->s_f[1] == p->s_f[3] && p->s_f[1] == p->s_f[4];
     k.sf = (T)p->s_f[1];
     k.one_m_sf = (T)(1.0 - p->s_f[1]);
-    k.cse = (T)(p->s_f[1] * 4.0 * ((double)k.w9[1] + (double)k.w9[2]));
+    k.cse = (T)(p->s_f[1] * 4.0 * ((double)k.wf[1] + (double)k.wf[2]));
     k.lg00 = (T)(p->s_g[0]);
     k.lg1 = (T)(p->s_g[1] / n1);
     k.cg0 = (T)(0.5 * p->s_g[0] - 1.0);

@@ -298,7 +298,8 @@ __device__ __forceinline__ void hermite_relax_back(const T k[9], const KParams<T
     }
     // B(cx, cy) = R_0 + cx R_1 + (cx^2 - cs2) R_2; even parts once per row
     const T E0 = R0[0] + one_m * R0[2], Ep = Rp[0] + one_m * Rp[2], Em = Rm[0] + one_m * Rm[2];
-    const T w0 = P.w9[0], wa = P.w9[1], wd = P.w9[2];
+    const T* w = kConserve ? P.wf : P.w9;
+    const T w0 = w[0], wa = w[1], wd = w[2];
     out[1] = v[1] - wa * (E0 + R0[1]);
     out[3] = v[3] - wa * (E0 - R0[1]);
     if constexpr (kConserve) {
@@ -343,8 +344,8 @@ __device__ __forceinline__ void relax_one_rate(const KParams<T>& P, int i, const
     const T qx = P.qf[i] * jx + lam * pcux - P.cV[i] * Vx;
     const T qy = P.qf[i] * jy + lam * pcuy - P.cV[i] * Vy;
     const T se = P.sf * emu;
-    const T a = P.w9[1] * se, ax = P.w9[1] * qx, ay = P.w9[1] * qy;
-    const T d = P.w9[2] * se, dp = P.w9[2] * (qx + qy), dm = P.w9[2] * (qx - qy);
+    const T a = P.wf[1] * se, ax = P.wf[1] * qx, ay = P.wf[1] * qy;
+    const T d = P.wf[2] * se, dp = P.wf[2] * (qx + qy), dm = P.wf[2] * (qx - qy);
     const T k = P.one_m_sf;
     const T t0 = P.cse * emu - P.sf * moving;
     const T o0 = add_rn(v[0], -t0);

@@ -75,6 +75,7 @@ struct KParams {
     T lk1, lk2;                   // (3 eps / 4) times lw1, lw2
     T w1d[3];                     // 1D weights of c = -1, 0, +1: d0/2, 1-d0, d0/2
     T w9[3];                      // 2D weights: rest, axis, diagonal
+    T wf[3];                      // the same as products of w1d, for the phase collision
     T rho[kMaxPhases], nu[kMaxPhases];
     T drho[kMaxPhases], dnu[kMaxPhases];   // rho_j - rho_N, nu_j - nu_N
     T sig[kMaxPhases][kMaxPhases];     // sigma_ij
