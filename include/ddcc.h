@@ -213,6 +213,10 @@ int ddcc_read(ddcc_handle* h, int field, double* host_out);
  */
 int ddcc_read_fields(ddcc_handle* h, double* host_out);
 
+/* The same with a destination for each of the 2N+4 fields (ny x nx doubles
+ * at host_out[i]), so that a program can keep some and release the others. */
+int ddcc_read_fields_to(ddcc_handle* h, double* const* host_out);
+
 /*
  * Per-phase mass sum_x sum_p f^i_p (= sum_x psi C_i, conserved by the
  * method) for phases 1..N-1, reduced in FP64 on the device in a fixed

@@ -35,7 +35,7 @@ FIELD_PSI = 20
 
 # every symbol include/ddcc.h declares
 EXPORTED = (
-    "ddcc_workspace_bytes", "ddcc_create", "ddcc_step", "ddcc_read", "ddcc_read_fields", "ddcc_mass",
+    "ddcc_workspace_bytes", "ddcc_create", "ddcc_step", "ddcc_read", "ddcc_read_fields", "ddcc_read_fields_to", "ddcc_mass",
     "ddcc_state_bytes", "ddcc_save_state", "ddcc_load_state", "ddcc_step_count",
     "ddcc_destroy", "ddcc_status_string", "ddcc_version", "ddcc_profile", "ddcc_kernel_times",
     "ddcc_phase_mass_noalloc", "ddcc_step_path", "ddcc_adjoint_bytes", "ddcc_adjoint_step",
@@ -119,6 +119,8 @@ def load():
     lib.ddcc_read.restype = C.c_int
     lib.ddcc_read_fields.argtypes = [vp, dp]
     lib.ddcc_read_fields.restype = C.c_int
+    lib.ddcc_read_fields_to.argtypes = [vp, C.POINTER(vp)]
+    lib.ddcc_read_fields_to.restype = C.c_int
     lib.ddcc_mass.argtypes = [vp, dp]
     lib.ddcc_mass.restype = C.c_int
     lib.ddcc_state_bytes.argtypes = [vp]
@@ -290,6 +292,19 @@ def ddcc_read_fields(h, out: np.ndarray):
     if st != DDCC_OK:
         raise DdccError(st, "ddcc_read_fields")
     return out
+
+
+def ddcc_read_fields_to(h, *arrays: np.ndarray):
+    """All 2N+4 fields in the order of ddcc_read_fields into the arrays, each
+    of one or more fields (fields first)."""
+    ptrs = []
+    for a in arrays:
+        assert a.dtype == np.float64 and a.flags.c_contiguous and a.ndim in (2, 3)
+        n = a.shape[0] if a.ndim == 3 else 1
+        ptrs += [a.ctypes.data + k * (a.nbytes // n) for k in range(n)]
+    st = load().ddcc_read_fields_to(C.c_void_p(h), (C.c_void_p * len(ptrs))(*ptrs))
+    if st != DDCC_OK:
+        raise DdccError(st, "ddcc_read_fields_to")
 
 
 def ddcc_mass(h, nphase: int) -> np.ndarray:

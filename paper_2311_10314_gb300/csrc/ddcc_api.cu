@@ -743,9 +743,10 @@ int form_macro(ddcc_handle* h) {
     return DDCC_OK;
 }
 
-// n planes from src to the host, as many at a time as the staging area holds.
+// n planes from src to the host, plane i to out[i], as many at a time as the
+// staging area holds; planes that follow one another at out in one copy.
 template <typename T>
-int export_planes(ddcc_handle* h, const T* src, int n, double* out) {
+int export_planes(ddcc_handle* h, const T* src, int n, double* const* out) {
     const ddcc_params& p = h->prm;
     KParams<T>& k = kp_of<T>(h);
     Fields<T>& f = fd_of<T>(h);
@@ -754,8 +755,11 @@ int export_planes(ddcc_handle* h, const T* src, int n, double* out) {
     for (int i = 0; i < n; i += group) {
         const int m = n - i < group ? n - i : group;
         DDCC_CU(launch_export<T>(src + (size_t)i * k.plane, f.stage, k, m, h->stream));
-        DDCC_CU(cudaMemcpyAsync(out + i * nodes, f.stage, sizeof(double) * nodes * m, cudaMemcpyDeviceToHost,
-                                h->stream));
+        for (int j = 0, len; j < m; j += len) {
+            for (len = 1; j + len < m && out[i + j + len] == out[i + j] + len * nodes;) ++len;
+            DDCC_CU(cudaMemcpyAsync(out[i + j], f.stage + j * nodes, sizeof(double) * nodes * len,
+                                    cudaMemcpyDeviceToHost, h->stream));
+        }
     }
     DDCC_CU(cudaStreamSynchronize(h->stream));
     return check_flag<T>(h);
@@ -765,7 +769,7 @@ template <typename T>
 int read_t(ddcc_handle* h, int field, double* out) {
     const int N = h->prm.nphase;
     Fields<T>& f = fd_of<T>(h);
-    if (field == DDCC_FIELD_PSI) return export_planes<T>(h, f.psi, 1, out);
+    if (field == DDCC_FIELD_PSI) return export_planes<T>(h, f.psi, 1, &out);
     int plane = -1;
     if (field >= DDCC_FIELD_C && field < DDCC_FIELD_C + N) plane = field - DDCC_FIELD_C;
     else if (field == DDCC_FIELD_RHO) plane = N;
@@ -776,11 +780,11 @@ int read_t(ddcc_handle* h, int field, double* out) {
     if (plane < 0) return DDCC_ERR_PARAM;
     const int st = form_macro<T>(h);
     if (st) return st;
-    return export_planes<T>(h, f.macro + (size_t)plane * kp_of<T>(h).plane, 1, out);
+    return export_planes<T>(h, f.macro + (size_t)plane * kp_of<T>(h).plane, 1, &out);
 }
 
 template <typename T>
-int read_fields_t(ddcc_handle* h, double* out) {
+int read_fields_t(ddcc_handle* h, double* const* out) {
     const int st = form_macro<T>(h);
     if (st) return st;
     return export_planes<T>(h, fd_of<T>(h).macro, 2 * h->prm.nphase + 4, out);
@@ -1071,9 +1075,18 @@ int ddcc_read(ddcc_handle* h, int field, double* host_out) {
                                          : read_t<float>(h, field, host_out);
 }
 
+int ddcc_read_fields_to(ddcc_handle* h, double* const* host_out) {
+    if (!h || !host_out) return DDCC_ERR_PARAM;
+    for (int i = 0; i < 2 * h->prm.nphase + 4; ++i)
+        if (!host_out[i]) return DDCC_ERR_PARAM;
+    return h->prm.precision == DDCC_FP64 ? read_fields_t<double>(h, host_out) : read_fields_t<float>(h, host_out);
+}
+
 int ddcc_read_fields(ddcc_handle* h, double* host_out) {
     if (!h || !host_out) return DDCC_ERR_PARAM;
-    return h->prm.precision == DDCC_FP64 ? read_fields_t<double>(h, host_out) : read_fields_t<float>(h, host_out);
+    double* out[2 * kMaxPhases + 4];
+    for (int i = 0; i < 2 * h->prm.nphase + 4; ++i) out[i] = host_out + (size_t)i * h->prm.nx * h->prm.ny;
+    return ddcc_read_fields_to(h, out);
 }
 
 int ddcc_mass(ddcc_handle* h, double* host_out) {
