@@ -110,8 +110,10 @@ typedef struct ddcc_handle ddcc_handle;
  * Bytes of device workspace ddcc_create() needs for these parameters, or 0
  * if they are invalid.  The workspace holds two copies of the populations
  * and of the lagged fields (ping-pong), psi, the contact-angle field, the
- * order-parameter scratch and reduction scratch; in FP64 also the chemical
- * potentials and psi rho of the current step and the terms of psi alone.
+ * order-parameter scratch, staging and reduction scratch; in FP64 also the
+ * chemical potentials and psi rho of the current step and the terms of psi
+ * alone, in FP32 2N+4 planes for the read-out (which FP64 forms in the
+ * population copy that the next step overwrites).
  */
 size_t ddcc_workspace_bytes(const ddcc_params* params);
 

@@ -49,7 +49,7 @@ struct ddcc_handle {
     int graph_state[2];
     cudaGraphExec_t step_graph[2];
     int64_t replayed;     // steps run by the two-step graph
-    // the read-out planes (f.macro) hold the fields of the current state;
+    // the read-out planes (macro_planes) hold the fields of the current state;
     // cleared by every call that may change the state
     int macro_valid;
     // reverse segments (ddcc_adjoint_segment, ddcc_adjoint_segment_pipelined)
@@ -135,6 +135,7 @@ bool valid_params(const ddcc_params* p) {
 struct Layout {
     size_t pop[2], lag[2], st, C, macro, mu, chi, st64, partial, stage, inflow, mass, flag, count, total;
     size_t plane_bytes;
+    int out_planes;
 };
 
 // Workspace: per ping-pong copy the 9N population planes (f^1..f^{N-1},
@@ -156,16 +157,24 @@ Layout layout_of(const ddcc_params* p) {
     for (int c = 0; c < 2; ++c) L.pop[c] = take(pb * 9 * N);
     for (int c = 0; c < 2; ++c) L.lag[c] = take(pb * lag_planes(N));
     L.st = take(pb * N);
-    L.C = take(pb * (N - 1));
-    L.macro = take(pb * (2 * N + 4));
+    L.partial = take(sizeof(double) * kMassBlocks * kMaxPhases);
+    const size_t dense = sizeof(double) * (size_t)p->nx * p->ny;
     if (p->precision == DDCC_FP64) {
+        // no read-out planes (macro_planes), and results are staged over the
+        // step's scratch: C, mu, psi rho and the staging area in one piece,
+        // for all 2N+4 fields at once from N = 3
+        L.st64 = take(pb * static64_planes());
+        L.C = take(pb * (N - 1));
         L.mu = take(pb * N);
         L.chi = take(pb);
-        L.st64 = take(pb * static64_planes());
+        L.stage = take(dense * (2 * N - 2));
+        L.out_planes = (int)((off - L.C) / dense);
+    } else {
+        L.C = take(pb * (N - 1));
+        L.macro = take(pb * (2 * N + 4));
+        L.stage = take(dense * (N - 1));
+        L.out_planes = N - 1;
     }
-    L.partial = take(sizeof(double) * kMassBlocks * kMaxPhases);
-    L.stage = take(sizeof(double) * (size_t)p->nx * p->ny *
-                   (p->precision == DDCC_FP64 ? stage_planes<double>(N) : stage_planes<float>(N)));
     L.inflow = take(es * (size_t)p->ny * N);
     L.mass = take(sizeof(double) * kMaxPhases);
     L.flag = take(sizeof(int) * 4);
@@ -294,6 +303,13 @@ Fields<double>& fd_of<double>(ddcc_handle* h) { return h->fd; }
 template <>
 Fields<float>& fd_of<float>(ddcc_handle* h) { return h->ff; }
 
+// The read-out planes.  FP64: nodes of the other population copy, all of which
+// the next step writes anew.
+template <typename T>
+T* macro_planes(ddcc_handle* h) {
+    return sizeof(T) == 8 ? fd_of<T>(h).f[1 - h->cur] : fd_of<T>(h).macro;
+}
+
 template <typename T>
 void carve(ddcc_handle* h, const Layout& L, Fields<T>& f) {
     char* b = h->ws;
@@ -306,14 +322,18 @@ void carve(ddcc_handle* h, const Layout& L, Fields<T>& f) {
     f.psi = reinterpret_cast<T*>(b + L.st);
     f.cosf = reinterpret_cast<T*>(b + L.st + L.plane_bytes);
     f.C = reinterpret_cast<T*>(b + L.C);
-    f.macro = reinterpret_cast<T*>(b + L.macro);
+    f.stage = reinterpret_cast<double*>(b + L.stage);
     if (sizeof(T) == 8) {
         f.mu = reinterpret_cast<T*>(b + L.mu);
         f.chi = reinterpret_cast<T*>(b + L.chi);
         f.st64 = reinterpret_cast<T*>(b + L.st64);
+        f.out_stage = reinterpret_cast<double*>(b + L.C);
+    } else {
+        f.macro = reinterpret_cast<T*>(b + L.macro);
+        f.out_stage = f.stage;
     }
+    f.out_planes = L.out_planes;
     f.partial = reinterpret_cast<double*>(b + L.partial);
-    f.stage = reinterpret_cast<double*>(b + L.stage);
     f.inflow = reinterpret_cast<T*>(b + L.inflow);
     f.flag = reinterpret_cast<int*>(b + L.flag);
 }
@@ -523,12 +543,15 @@ int create_t(ddcc_handle* h, const double* psi, const double* cosf, const double
         k.wet_field = 1;
         DDCC_CU(launch_walls_init<T>(k, f.psi, f.cosf, h->stream));
         const size_t plane = (size_t)p.nx * p.ny;
+        T* scratch = macro_planes<T>(h);
         for (int w = 0; w < n_walls; ++w) {
-            if ((st = upload<T>(h, wall_psi + w * plane, f.macro, 1))) return st;
-            if ((st = upload<T>(h, wall_cos + w * plane * (N - 1), f.macro + k.plane, N - 1))) return st;
-            DDCC_CU(launch_fill_ghosts<T>(f.macro, 1, k, h->stream, 1, 1));
-            DDCC_CU(launch_wall_accumulate<T>(k, f.macro, f.psi, f.cosf, h->stream));
+            if ((st = upload<T>(h, wall_psi + w * plane, scratch, 1))) return st;
+            if ((st = upload<T>(h, wall_cos + w * plane * (N - 1), scratch + k.plane, N - 1))) return st;
+            DDCC_CU(launch_fill_ghosts<T>(scratch, 1, k, h->stream, 1, 1));
+            DDCC_CU(launch_wall_accumulate<T>(k, scratch, f.psi, f.cosf, h->stream));
         }
+        // a population copy's ghost frames start as zero
+        if (sizeof(T) == 8) DDCC_CU(cudaMemsetAsync(scratch, 0, sizeof(T) * k.plane * N, h->stream));
     } else {
         k.has_cos_field = cosf ? 1 : 0;
         for (int i = 0; i < N - 1; ++i) k.cos_uni[i] = cosf ? T(0) : (T)cosu[i];
@@ -733,7 +756,7 @@ int form_macro(ddcc_handle* h) {
     Fields<T>& f = fd_of<T>(h);
     if constexpr (sizeof(T) == 8) {
         Step64Args a = args64(f, f.f[h->cur], f.lag[h->cur], nullptr, nullptr);
-        a.macro = f.macro;
+        a.macro = macro_planes<T>(h);
         DDCC_CU(launch_fields64(k, a, h->stream));
         DDCC_CU(launch_update64(k, a, h->stream));
     } else {
@@ -751,13 +774,13 @@ int export_planes(ddcc_handle* h, const T* src, int n, double* const* out) {
     KParams<T>& k = kp_of<T>(h);
     Fields<T>& f = fd_of<T>(h);
     const size_t nodes = (size_t)p.nx * p.ny;
-    const int group = stage_planes<T>(p.nphase);
+    const int group = f.out_planes;
     for (int i = 0; i < n; i += group) {
         const int m = n - i < group ? n - i : group;
-        DDCC_CU(launch_export<T>(src + (size_t)i * k.plane, f.stage, k, m, h->stream));
+        DDCC_CU(launch_export<T>(src + (size_t)i * k.plane, f.out_stage, k, m, h->stream));
         for (int j = 0, len; j < m; j += len) {
             for (len = 1; j + len < m && out[i + j + len] == out[i + j] + len * nodes;) ++len;
-            DDCC_CU(cudaMemcpyAsync(out[i + j], f.stage + j * nodes, sizeof(double) * nodes * len,
+            DDCC_CU(cudaMemcpyAsync(out[i + j], f.out_stage + j * nodes, sizeof(double) * nodes * len,
                                     cudaMemcpyDeviceToHost, h->stream));
         }
     }
@@ -780,14 +803,14 @@ int read_t(ddcc_handle* h, int field, double* out) {
     if (plane < 0) return DDCC_ERR_PARAM;
     const int st = form_macro<T>(h);
     if (st) return st;
-    return export_planes<T>(h, f.macro + (size_t)plane * kp_of<T>(h).plane, 1, &out);
+    return export_planes<T>(h, macro_planes<T>(h) + (size_t)plane * kp_of<T>(h).plane, 1, &out);
 }
 
 template <typename T>
 int read_fields_t(ddcc_handle* h, double* const* out) {
     const int st = form_macro<T>(h);
     if (st) return st;
-    return export_planes<T>(h, fd_of<T>(h).macro, 2 * h->prm.nphase + 4, out);
+    return export_planes<T>(h, macro_planes<T>(h), 2 * h->prm.nphase + 4, out);
 }
 
 template <typename T>

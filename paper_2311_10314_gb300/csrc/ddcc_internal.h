@@ -125,23 +125,19 @@ struct Fields {
     T* psi;           // 1 plane
     T* cosf;          // N-1 planes or null
     T* C;             // N-1 planes (order-parameter scratch)
-    T* macro;         // 2N+4 planes (read-out scratch)
+    T* macro;         // (FP32) 2N+4 planes (read-out scratch); FP64: macro_planes()
     T* mu;            // (FP64) N planes: chemical potentials of the current step
     T* chi;           // (FP64) 1 plane: psi rho of the current step
     T* st64;          // (FP64) static64_planes() planes of psi's own terms, formed at create
     double* partial;  // kMassBlocks * kMaxPhases
-    double* stage;    // staging of host inputs and results (double), stage_planes(N) planes
+    double* stage;    // staging of host inputs (double), N-1 planes or more
+    double* out_stage;  // staging of results, out_planes planes (FP64: from C to stage's end)
+    int out_planes;
     T* inflow;        // open x ends: u_in (ny values), then C_in ((N-1) x ny)
     int* flag;        // device error word
 };
 
 inline int lag_planes(int N) { return 2 * N + 3; }
-
-// Planes of the staging area: the N-1 of one host input; in FP64 all 2N+4
-// read-out fields, so that they leave in one copy (FP32 grids are the large
-// ones, and their fields leave in groups).
-template <typename T>
-constexpr int stage_planes(int N) { return sizeof(T) == 8 ? 2 * N + 4 : N - 1; }
 
 // Row-sweep kernel: strip width per precision, rows per iteration and
 // threads per CTA.  With 60 columns the order-parameter pass (strip + 2
