@@ -585,14 +585,12 @@ Step64Args args64(const Fields<double>& f, const double* pop_in, const double* l
 // The rings that the next step's halo boxes read, where the fused kernel has
 // not written them: its 64 x 4 tiles do not, and in three rows a node has two
 // copies along y.
+bool needs_ring_fill(const ddcc_handle* h) { return !fused_writes_rings(fused_x(h->tile_wide)) || h->prm.ny < 4; }
 template <typename T>
-int fused_rings(ddcc_handle* h, T* pop, T* lag) {
-    if (fused_writes_rings(fused_x(h->tile_wide)) && h->prm.ny >= 4) return DDCC_OK;
-    int st;
-    if ((st = prof_begin(h, 3))) return st;
+int fill_rings(ddcc_handle* h, T* pop, T* lag) {
     DDCC_CU(launch_fill_ghosts2<T>(GhostRing<T>{pop, 9 * (h->prm.nphase - 1), kFusedGhostF, kFusedGhostF},
                                    GhostRing<T>{lag, 1, kFusedGhostA, kFusedGhostA}, kp_of<T>(h), h->stream));
-    return prof_end(h);
+    return DDCC_OK;
 }
 
 template <typename T>
@@ -627,7 +625,11 @@ int step_plain(ddcc_handle* h, int64_t n) {
             if ((st = prof_end(h))) return st;
             if (h->prm.flags & DDCC_FLAG_OPEN_X)
                 DDCC_CU(launch_open_bc<T>(k, f.f[1 - c], f.lag[1 - c], f.psi, f.inflow, h->stream));
-            if ((st = fused_rings<T>(h, f.f[1 - c], f.lag[1 - c]))) return st;
+            if (needs_ring_fill(h)) {
+                if ((st = prof_begin(h, 3))) return st;
+                if ((st = fill_rings<T>(h, f.f[1 - c], f.lag[1 - c]))) return st;
+                if ((st = prof_end(h))) return st;
+            }
         } else {
             if ((st = prof_begin(h, 0))) return st;
             DDCC_CU(launch_order_param<T>(k, f, c, h->stream));
@@ -930,7 +932,7 @@ int step_between_t(ddcc_handle* h, const void* state_in, void* state_out) {
         if (!encode_fused<T>(&m, in_pop, in_lag, k, h->tile_wide)) return DDCC_ERR_CUDA;
         TileTmaArgs<T> a{&m.fh, &m.g, &m.lag, &h->tt_c, &h->tt_st, &m.a, &k, out_pop, out_lag, f.flag, h->tile_wide};
         DDCC_CU(launch_collide_fused<T>(a, h->stream));
-        return fused_rings<T>(h, out_pop, out_lag);
+        if (needs_ring_fill(h)) return fill_rings<T>(h, out_pop, out_lag);
     }
     return DDCC_OK;
 }
