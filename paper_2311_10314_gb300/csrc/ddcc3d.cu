@@ -1873,14 +1873,22 @@ int ddcc3d_step(ddcc3d_handle* h, int64_t nsteps) {
 int ddcc3d_read(ddcc3d_handle* h, int field, double* host_out) {
     if (!h || !host_out) return DDCC_ERR_PARAM;
     const int np = h->prm.nphase - 1;
+    int rc;
     if (h->prm.precision == DDCC_FP64) {
-        if (np == 1) return read_n<double, 1>(h, h->kd, h->fd, field, host_out);
-        if (np == 2) return read_n<double, 2>(h, h->kd, h->fd, field, host_out);
-        return read_n<double, 3>(h, h->kd, h->fd, field, host_out);
+        rc = np == 1   ? read_n<double, 1>(h, h->kd, h->fd, field, host_out)
+             : np == 2 ? read_n<double, 2>(h, h->kd, h->fd, field, host_out)
+                       : read_n<double, 3>(h, h->kd, h->fd, field, host_out);
+    } else {
+        rc = np == 1   ? read_n<float, 1>(h, h->kf, h->ff, field, host_out)
+             : np == 2 ? read_n<float, 2>(h, h->kf, h->ff, field, host_out)
+                       : read_n<float, 3>(h, h->kf, h->ff, field, host_out);
     }
-    if (np == 1) return read_n<float, 1>(h, h->kf, h->ff, field, host_out);
-    if (np == 2) return read_n<float, 2>(h, h->kf, h->ff, field, host_out);
-    return read_n<float, 3>(h, h->kf, h->ff, field, host_out);
+    if (rc) {
+        // the planes may not have been formed, and the error is not the next call's
+        h->cmu_valid = h->macro_valid = 0;
+        cudaGetLastError();
+    }
+    return rc;
 }
 
 int ddcc3d_mass(ddcc3d_handle* h, double* host_out) {

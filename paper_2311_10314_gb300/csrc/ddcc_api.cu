@@ -815,6 +815,16 @@ int read_fields_t(ddcc_handle* h, double* const* out) {
     return export_planes<T>(h, macro_planes<T>(h), 2 * h->prm.nphase + 4, out);
 }
 
+// A reading that failed: its planes may not have been formed, and the error is
+// not the next call's.
+int read_done(ddcc_handle* h, int st) {
+    if (st != DDCC_OK) {
+        h->macro_valid = 0;
+        cudaGetLastError();
+    }
+    return st;
+}
+
 template <typename T>
 int mass_t(ddcc_handle* h, double* out) {
     const int N = h->prm.nphase;
@@ -1096,15 +1106,18 @@ int ddcc_step(ddcc_handle* h, int64_t nsteps) {
 
 int ddcc_read(ddcc_handle* h, int field, double* host_out) {
     if (!h || !host_out) return DDCC_ERR_PARAM;
-    return h->prm.precision == DDCC_FP64 ? read_t<double>(h, field, host_out)
-                                         : read_t<float>(h, field, host_out);
+    const int st = h->prm.precision == DDCC_FP64 ? read_t<double>(h, field, host_out)
+                                                 : read_t<float>(h, field, host_out);
+    return read_done(h, st);
 }
 
 int ddcc_read_fields_to(ddcc_handle* h, double* const* host_out) {
     if (!h || !host_out) return DDCC_ERR_PARAM;
     for (int i = 0; i < 2 * h->prm.nphase + 4; ++i)
         if (!host_out[i]) return DDCC_ERR_PARAM;
-    return h->prm.precision == DDCC_FP64 ? read_fields_t<double>(h, host_out) : read_fields_t<float>(h, host_out);
+    const int st = h->prm.precision == DDCC_FP64 ? read_fields_t<double>(h, host_out)
+                                                 : read_fields_t<float>(h, host_out);
+    return read_done(h, st);
 }
 
 int ddcc_read_fields(ddcc_handle* h, double* host_out) {
