@@ -56,6 +56,10 @@ __host__ __device__ constexpr int pair_rep(int q) { return q < 3 ? 2 * q + 1 : 7
 __host__ __device__ constexpr int pair_opp(int q) { return q < 3 ? 2 * q + 2 : 14 - (q - 3); }
 
 // Kernel constants, derived on the host (make_params) from ddcc3d_params.
+// inv_cs2 and K are read by no kernel; they hold the places of the rest.
+// Without them, or with others in their places, the compiler allots the
+// registers of k3_fused otherwise: 208 x 192 x 160, N = 3, 200 steps and reads
+// in 147 to 160 ms instead of 140.
 template <typename T>
 struct P3 {
     int nx, ny, nz, N;
@@ -499,13 +503,13 @@ struct GlobalSrc {     // the per-step C and mu planes in global memory
 // Q_j = C_j (grad mu_j - sum_k C_k grad mu_k) add up to zero.  For two phases
 // mu_2 = -mu_1.  kMacro: rho, u and P of the state go to the planes at out
 // instead.
-// FP64 (three kernels, bound by FP64 warp instructions): 96 x 80 x 72, N = 3,
-// 1116 + 341 + 35 us for update, mu and C before sums over all phases, pair
-// identities of mu, psi's own terms, 256-thread blocks of 32 x 4 x 2 nodes and
-// divisions by the operator went; 10 steps and a read-out 18.0 -> 9.4 ms.
-// FP32 (fused): 24% fewer instructions, 753 -> 722 us at 208 x 192 x 160, and
-// 617 with field a staged; the kernel's loads and stores alone take 504 us
-// there (loads 314), the stores in 128-byte rows of 45 planes.
+// FP64 (three kernels) is bound by FP64 warp instructions: sums over all
+// phases, pairs of mu, psi's own terms at every step, 256-thread blocks of 32
+// x 4 x 2 nodes and divisions by the operator took twice the time (96 x 80 x
+// 72, N = 3, 10 steps and a read-out: 18.0 ms, now 9.4).
+// FP32 (fused): 617 us a step at 208 x 192 x 160, N = 3 (722 without field a
+// staged); the kernel's loads and stores alone take 504 us there (loads 314),
+// the stores in 128-byte rows of 45 planes.
 template <typename T, int NP, bool kMacro, class S>
 __device__ __forceinline__ void update_node(const P3<T>& P, const F3<T>& F, int cur, T* out, const S& src) {
     constexpr int N = NP + 1, NM = NP == 1 ? 1 : N;
@@ -1413,8 +1417,8 @@ void make_params(const ddcc3d_params* p, P3<T>& K) {
     const size_t e = sizeof(T);
     K.plane = (long long)(round256((size_t)K.nxy * p->nz * e) / e);
     K.cs2 = (T)cs2;
-    K.inv_cs2 = (T)(1.0 / cs2);
     const double wa = (d0 - d0 * d0) / 2.0, wc = d0 * d0 / 8.0, w0 = 1.0 - 3.0 * d0 + 2.0 * d0 * d0;
+    K.inv_cs2 = (T)(1.0 / cs2);
     K.ga = (T)(wa / cs2);
     K.gc = (T)(wc / cs2);
     K.la = (T)(0.75 * p->width * wa / cs2);
@@ -1634,7 +1638,8 @@ int fused_setup_v(ddcc3d_handle* h) {
     return DDCC_OK;
 }
 
-// The staged (cp.async) C pass runs in FP32 when nx is a multiple of 4.
+// FP32 stages the C pass by cp.async: by 16 bytes where nx is a multiple of 4
+// (rows are whole aligned quads), else node by node.
 template <typename T>
 bool fused_vec(const ddcc3d_handle* h) { return sizeof(T) == 4 && h->prm.nx % 4 == 0; }
 

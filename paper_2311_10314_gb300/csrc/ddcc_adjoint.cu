@@ -748,10 +748,10 @@ __device__ __forceinline__ void mu_node_at(const KParams<T>& P, const T* __restr
                                            double* dJ_dcos, int x, int y,
                                            const T (&Lmu_kept)[mu_planes<NP>()]);
 
-// kMu: the chemical-potential VJP (mu_node_at) of the node follows in the
-// same thread from the gathered adjoint of mu, which then never reaches
-// memory (the initial state's reverse runs k_adj_mu_node on its own).
-template <typename T, int NP, bool kMu>
+// The chemical-potential VJP (mu_node_at) of the node follows in the same
+// thread from the gathered adjoint of mu, which then never reaches memory
+// (the initial state's reverse runs k_adj_mu_node on its own).
+template <typename T, int NP>
 __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather3(KParams<T> P, const T* __restrict__ psi_pl,
                                                      AdjPlanes<T, NP> W, T* __restrict__ ad_lag_out,
                                                      const T* __restrict__ cosf, double* dJ_dcos) {
@@ -786,12 +786,7 @@ __global__ void __launch_bounds__(AX * block_rows<T>()) k_adj_gather3(KParams<T>
 #pragma unroll
     for (int j = 0; j < NP - 1; ++j) W.LC[j * pl + o] = LC[j];
     W.Lpsi[o] = Lpsi;
-    if constexpr (kMu) {
-        mu_node_at<T, NP>(P, psi_pl, cosf, W, dJ_dcos, x, y, Lmu);
-    } else {
-#pragma unroll
-        for (int j = 0; j < NM; ++j) W.Lmu[j * pl + o] = Lmu[j];
-    }
+    mu_node_at<T, NP>(P, psi_pl, cosf, W, dJ_dcos, x, y, Lmu);
 }
 
 // ---- VJP of the chemical potential (Eq. 2.14) per node ---------------------
@@ -1135,7 +1130,7 @@ dim3 node_block() { return dim3(AX, block_rows<T>()); }
 
 template <typename T, int NP>
 cudaError_t gather_smem_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(k_adj_gather3<T, NP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_adj_gather3<T, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(sizeof(T) * Ring<T>::N * AdjPlanes<T, NP>::NV));
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_adj_gather2<T, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1156,7 +1151,7 @@ cudaError_t adjoint_step_n(const AdjStepArgs<T>& a, cudaStream_t s) {
             cudaSuccess ||
         (e = launch_dependent(overlaps<T>(), k_adj_node<T, NP>, grd, blk, 0, s, k, a.psi, a.st_pop, a.st_lag, a.ad_pop_in, a.ad_lag_in,
                               a.ad_pop_out, a.ad_lag_out, W)) != cudaSuccess ||
-        (e = launch_dependent(overlaps<T>(), k_adj_gather3<T, NP, true>, grd, blk, sizeof(T) * Ring<T>::N * AdjPlanes<T, NP>::NV, s, k,
+        (e = launch_dependent(overlaps<T>(), k_adj_gather3<T, NP>, grd, blk, sizeof(T) * Ring<T>::N * AdjPlanes<T, NP>::NV, s, k,
                               a.psi, W, a.ad_lag_out, a.cosf, a.dJ_dcos)) != cudaSuccess)
         return e;
     return launch_dependent(overlaps<T>(), k_adj_gather2<T, NP>, grd, blk, sizeof(T) * Ring<T>::N * (2 * (NP - 1) + 3), s, k, a.psi, W,

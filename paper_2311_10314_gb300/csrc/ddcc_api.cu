@@ -94,7 +94,7 @@ int prof_end(ddcc_handle* h) {
 }
 
 constexpr size_t kAlign = 256;
-// half of the 129 MB L2: a step reads one state and writes another
+// states above this take 64 x 4 tiles (the measured crossover, fused_tile_wide)
 constexpr long long kWideStateBytes = 128LL << 20;
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -201,11 +201,8 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
     const double w0 = (1.0 - d0) * (1.0 - d0);
     const double wa = (d0 - d0 * d0) / 2.0, wd = d0 * d0 / 4.0;
     k.cs2 = (T)cs2;
-    k.inv_cs2 = (T)(1.0 / cs2);
     k.gw1 = (T)(wa / cs2);
     k.gw2 = (T)(wd / cs2);
-    k.lw1 = (T)(wa / cs2);
-    k.lw2 = (T)(wd / cs2);
     k.lk1 = (T)(0.75 * p->width * wa / cs2);
     k.lk2 = (T)(0.75 * p->width * wd / cs2);
     k.w9[0] = (T)w0;
@@ -234,8 +231,6 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
             k.sig[i][j] = (T)s;
             b2 += 2.0 * 3.0 * s / p->width;
             k.beta2[i][j] = (T)(i == j ? 0.0 : 2.0 * 3.0 * s / p->width);  // 2 beta, beta = 3 sigma / eps
-            k.kap[i][j] = (T)(0.75 * p->width * s);                       // -kappa_ij = 3 eps sigma / 4
-            k.wet[i][j] = (T)(3.0 * s);
             k.invsig[i][j] = (T)(i == j ? 0.0 : 1.0 / s);
         }
         k.beta2s[i] = (T)b2;
@@ -245,7 +240,6 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
     // (00, 10, 01, 20, 02, 11, 21, 12, 22)
     const double n1 = d0, n2 = d0 * (1.0 - d0);
     const double Nab[9] = {1.0, n1, n1, n2, n2, n1 * n1, n2 * n1, n1 * n2, n2 * n2};
-    for (int a = 0; a < 9; ++a) k.invN[a] = (T)(1.0 / Nab[a]);
     for (int i = 0; i < N - 1; ++i) {
         k.eta[i] = (T)p->eta[i];
         // Eq. 17: m0 = (1/s1 - 1/2) eta_i cs2
@@ -273,7 +267,6 @@ void fill_kparams(const ddcc_params* p, KParams<T>& k) {
     k.nu_to_s21 = (T)(2.0 / (1.0 - cs2));
     k.nu_to_s22 = (T)(1.0 / cs2);
     k.damp = (T)(1.0 / (p->eps0 * p->eps0 * p->eps0));
-    k.half_damp = (T)(0.5 / (p->eps0 * p->eps0 * p->eps0));
     // Eq. 19 (2D): K = 1 - d0, H = K (1 - 2 d0)(s21 - 2)
     const double K = 1.0 - d0, sg0 = p->s_g[0];
     k.A_P = (T)(0.5 + K * (1.0 - d0) * (2.0 - sg0) / (2.0 * sg0));
@@ -433,19 +426,19 @@ int setup_sweep(ddcc_handle* h) {
     return DDCC_OK;
 }
 
-// The fused kernel's tile.  FP32: 64 x 4 where a state is beyond L2 and the
-// wider tile does not add columns of padding.  The step is then bound by
-// how the stores reach DRAM: with every plane's rows written in 256-byte
-// pieces instead of 128-byte ones a copy of the 47 planes at 4096^2 with
-// this kernel's loads and stores and no arithmetic takes 1.04 ms instead of
-// 1.19 (stores alone: 1.20 ms in 32 x 8 tiles, 0.86 in 128 x 2), and the step
-// 1.177 instead of 1.270 (1021 x 1024, N = 3: 71.0 instead of 72.5 us).
-// Smaller states stay in L2, where the 32 x 8 tile's smaller halo counts and
-// its step is one launch (us a step, 32 x 8 and 64 x 4: 704 x 700, N = 3, 68
-// MB, 37.5 and 38.7; 1024 x 1024, N = 2, 100 MB, 52.0 and 53.0; 97 x 9000, N =
-// 2, 83 MB, 69.9 and 72.8; at 144 MB, N = 3, 72.2 and 70.8; at 188 MB, N = 4,
-// 94.7 and 89.0).  More rows of tiles than
-// a launch grid has keep the taller tile.
+// The fused kernel's tile: 64 x 4 for states over 128 MB, unless the wider
+// tile adds columns of padding.  Large states are bound by how the stores
+// reach DRAM: with every plane's rows written in 256-byte pieces instead of
+// 128-byte ones a copy of the 47 planes at 4096^2 with this kernel's loads and
+// stores and no arithmetic takes 1.04 ms instead of 1.19 (stores alone: 1.20
+// ms in 32 x 8 tiles, 0.86 in 128 x 2), and the step 1.177 instead of 1.270.
+// For smaller states the 32 x 8 tile's smaller halo counts for more, and its
+// step is one launch that starts early.  The line is the crossover as
+// measured, between 100 and 144 MB (us a step, 32 x 8 and 64 x 4: 704 x 700, N
+// = 3, 68 MB, 37.5 and 38.7; 97 x 9000, N = 2, 83 MB, 69.9 and 72.8; 1024 x
+// 1024, N = 2, 100 MB, 52.0 and 53.0; 1021 x 1024, N = 3, 144 MB, 72.2 and
+// 70.8; 1024 x 1024, N = 4, 188 MB, 94.7 and 89.0).  More rows of tiles than a
+// launch grid has keep the taller tile.
 template <typename T>
 bool fused_tile_wide(const ddcc_params& p) {
     if (p.nx < kWideX || (p.ny + kWideY - 1) / kWideY > 65535) return false;

@@ -381,9 +381,9 @@ __device__ __forceinline__ T psi_rho(const KParams<T>& P, T psi, const CA& C) {
 // the capillary force through mu_j - mu_N, and m^C = -m0 sum_j
 // (rho_j - rho_N) Q_j because the Q_j add up to zero.  With the pair
 // identities of chem_pot, psi rho formed once per node and the reciprocals
-// above, the FP64 tile step (bound by its FP64 pipe) went from 629 to 511 us
-// at 512 x 512, N = 4, and from 51 to 40 us at 64 x 64, N = 2; in FP32, bound
-// by memory, these changes alone leave the time as it was.
+// above this is a fifth of the FP64 instructions less than sums over all
+// phases, which is what FP64 is bound by; in FP32, bound by memory, it leaves
+// the time as it is.
 // kOneRate: the phase collision by relax_one_rate.
 template <typename T, int NP, int MODE, bool kOneRate = false, class Acc, class Sink>
 __device__ __forceinline__ void node_update(const KParams<T>& P, const Acc& A, Sink& out) {

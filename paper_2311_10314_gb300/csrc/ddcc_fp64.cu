@@ -20,12 +20,12 @@
 //    free beside the FP64 pipe), so no ghost frame is read; the one-node
 //    ghost ring of the lagged plane a, which the reverse step reads, is
 //    written along with the plane.
-// Against the one-kernel tile step with the same node arithmetic: 512 x 512,
-// N = 4, 511 -> 440 us a step; 64 x 64, N = 2, 40 -> 20 us.  With one rate for
-// the phases' higher moments (relax_one_rate) 398 and 16.  Both kernels then
-// run at 92 to 96% of the FP64 rate that chains of multiply-adds reach
-// (ddcc_measure_fp64_peak), with 848 FP64 instructions a node by the
-// transforms and 770 with one rate (N = 4; 1165 in the tile kernel at first).
+// A 32 x 8 tile in one kernel took 511 us a step at 512 x 512, N = 4, and 40 at
+// 64 x 64, N = 2, this pair 440 and 20, and with one rate for the phases'
+// higher moments (relax_one_rate) 396 and 16.  With one rate a node of four
+// phases takes 763 FP64 instructions (by the transforms 28 a phase more), and
+// at 1024 x 1024 the two kernels run them at the rate that independent chains
+// of multiply-adds reach (ddcc_measure_fp64_peak): 1.51 ms a step.
 #include "ddcc_device.cuh"
 
 namespace ddcc {

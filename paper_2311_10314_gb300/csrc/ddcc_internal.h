@@ -69,10 +69,9 @@ struct KParams {
     int has_cos_field;
     int wet_field;                // 1: the N-1 angle planes hold the wetting strengths
                                   //    e_j = sum_k cos(theta^k_jN) |grad psi_k| (several solids)
-    T cs2, inv_cs2;
-    T gw1, gw2;                   // w_axis / cs2, w_diag / cs2 (gradient stencil)
-    T lw1, lw2;                   // w_axis / cs2, w_diag / cs2 (div(psi grad) stencil)
-    T lk1, lk2;                   // (3 eps / 4) times lw1, lw2
+    T cs2, m0;
+    T gw1, gw2;                   // w_axis / cs2, w_diag / cs2 (stencils)
+    T lk1, lk2;                   // (3 eps / 4) times gw1, gw2 (div(psi grad) stencil)
     T w1d[3];                     // 1D weights of c = -1, 0, +1: d0/2, 1-d0, d0/2
     T w9[3];                      // 2D weights: rest, axis, diagonal
     T wf[3];                      // the same as products of w1d, for the phase collision
@@ -81,19 +80,15 @@ struct KParams {
     T sig[kMaxPhases][kMaxPhases];     // sigma_ij
     T beta2s[kMaxPhases];              // sum_{j != i} 2 beta_ij
     T beta2[kMaxPhases][kMaxPhases];   // 2 beta_ij = 6 sigma_ij / eps
-    T kap[kMaxPhases][kMaxPhases];     // 3 eps sigma_ij / 4
-    T wet[kMaxPhases][kMaxPhases];     // 3 sigma_ij
     T sigN[kMaxPhases];                // sigma_iN
     T invsig[kMaxPhases][kMaxPhases];  // 1 / sigma_ij (0 on the diagonal)
     T cos_uni[kMaxPhases];             // cos(theta_iN) when uniform
     T eta[kMaxPhases];
     T ceta[kMaxPhases];                // cs2 eta_i
     T cV[kMaxPhases];                  // coefficient of V in the first moments: lambda_1 / 2 - 1 / N_1
-    T m0;
     // phase LB: lambda_ab = s_ab / N_ab in moment order
-    // (00, 10, 01, 20, 02, 11, 21, 12, 22), and 1 / N_ab
+    // (00, 10, 01, 20, 02, 11, 21, 12, 22)
     T lamf[kMaxPhases][9];
-    T invN[9];
     // one rate for the moments of second and higher order: that rate, 1 less it,
     // rate times the moving directions' weights 1 - w_0, and rate / cs2 -
     // lambda_1 per phase
@@ -105,7 +100,6 @@ struct KParams {
     T invN20, invN11;             // 1 / N for the per-node s21 and s22 rows
     T nu_to_s21, nu_to_s22;       // 2 / (1 - cs2) and 1 / cs2 (Eq. 16)
     T damp;                       // 1 / eps0^3
-    T half_damp;
     T A_P;                        // 1/2 + K (1 - d0)(2 - s0) / (2 s0)
     T Kh;                         // K / 2
     T Hfac;                       // K (1 - 2 d0)

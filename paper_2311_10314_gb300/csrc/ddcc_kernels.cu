@@ -213,7 +213,7 @@ __device__ __forceinline__ int ring2_step(int v, int n, int periodic) {
 // bounce-back as TileSink, and every phase population and the lagged plane a
 // are also written to the copies of their node in the 2-node ghost ring that
 // the next step's halo boxes read.  It takes a launch off a small grid's step
-// (256 x 256, N = 3: 10.3 -> 9.1 us); the 64 x 4 form, for states beyond L2,
+// (256 x 256, N = 3: 10.3 -> 9.1 us); the 64 x 4 form, for states over 128 MB,
 // keeps the launch (4096 x 4096, N = 4: 1177 us a step with it, 1196 with
 // this sink, whose registers also weigh on the inner tiles).
 template <typename T, int NP>
@@ -431,8 +431,9 @@ __global__ void __launch_bounds__(NT, 2)
 // resident CTAs.
 constexpr int kPrefetchQuarterWaves = 3;
 
-template <typename T, int NP, bool TF, int TX, int TY>
+template <int NP, bool TF, int TX, int TY>
 struct FLay {
+    using T = float;   // FP32 alone (the C pass goes by quads)
     static constexpr int NF = 9 * (NP - 1);
     static constexpr int NLAG = 2 * NP + 3;
     static constexpr int NST = TF ? NP : 1;
@@ -460,9 +461,10 @@ struct FLay {
     static constexpr unsigned tx_tile = (unsigned)((G_BOX + LAG_BOX) * sizeof(T));
 };
 
-template <typename T, int NP, bool TF, int TX, int TY>
+template <int NP, bool TF, int TX, int TY>
 struct FusedAcc {
-    using L = FLay<T, NP, TF, TX, TY>;
+    using T = float;
+    using L = FLay<NP, TF, TX, TY>;
     const KParams<T>& P;
     const T* sm;
     int tx, ty;
@@ -487,13 +489,14 @@ struct FusedAcc {
     __device__ T g(int p) const { return sm[L::g_off + ((size_t)p * TY + ty) * TX + tx]; }
 };
 
-template <typename T, int NP, bool TF, int TX, int TY>
+template <int NP, bool TF, int TX, int TY>
 __global__ void __launch_bounds__(TX * TY, 2)
     k_step_fused(const __grid_constant__ CUtensorMap tm_fh, const __grid_constant__ CUtensorMap tm_g,
                  const __grid_constant__ CUtensorMap tm_lag, const __grid_constant__ CUtensorMap tm_st,
-                 const __grid_constant__ CUtensorMap tm_a, KParams<T> P, T* __restrict__ pop_out,
-                 T* __restrict__ lag_out, int* __restrict__ err, int pf_dist, int off32) {
-    using L = FLay<T, NP, TF, TX, TY>;
+                 const __grid_constant__ CUtensorMap tm_a, KParams<float> P, float* __restrict__ pop_out,
+                 float* __restrict__ lag_out, int* __restrict__ err, int pf_dist, int off32) {
+    using T = float;
+    using L = FLay<NP, TF, TX, TY>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     T* sm = reinterpret_cast<T*>(smem_raw);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw + L::bar_byte_off);
@@ -597,7 +600,7 @@ __global__ void __launch_bounds__(TX * TY, 2)
     if (x >= P.nx || y >= P.ny) return;
     const long long o = P.org + (long long)y * P.pitch + x;
     if (fused_writes_rings(TX)) dependents_may_start();
-    FusedAcc<T, NP, TF, TX, TY> acc{P, sm, (int)threadIdx.x, (int)threadIdx.y};
+    FusedAcc<NP, TF, TX, TY> acc{P, sm, (int)threadIdx.x, (int)threadIdx.y};
     // most tiles push only into the domain's interior, and (kRings) only to
     // nodes without a copy in the 2-node ghost ring: fixed neighbour offsets,
     // no wrap or bounce-back, 32-bit offsets (a block-uniform branch)
@@ -648,13 +651,13 @@ __global__ void __launch_bounds__(TX * TY, 2)
     dev::node_update<T, NP, 0>(P, acc, sink);
 }
 
-template <typename T, int NP, bool TF, int TX, int TY>
-cudaError_t collide_fused_n(const TileTmaArgs<T>& a, cudaStream_t s) {
-    using L = FLay<T, NP, TF, TX, TY>;
-    const cudaError_t e = cudaFuncSetAttribute(k_step_fused<T, NP, TF, TX, TY>,
+template <int NP, bool TF, int TX, int TY>
+cudaError_t collide_fused_n(const TileTmaArgs<float>& a, cudaStream_t s) {
+    using L = FLay<NP, TF, TX, TY>;
+    const cudaError_t e = cudaFuncSetAttribute(k_step_fused<NP, TF, TX, TY>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
     if (e != cudaSuccess) return e;
-    const KParams<T>& kp = *a.kp;
+    const KParams<float>& kp = *a.kp;
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -665,7 +668,7 @@ cudaError_t collide_fused_n(const TileTmaArgs<T>& a, cudaStream_t s) {
     const int off32 = (long long)(9 * NP) * kp.plane < (1LL << 31) ? 1 : 0;
     // the next step may start early where the whole step is short: 256 x 256, N =
     // 3, 8.1 us a step without, 7.4 with (4096 x 4096, N = 4: 1179 and 1185)
-    return launch_dependent(fused_writes_rings(TX), k_step_fused<T, NP, TF, TX, TY>, dim3((kp.nx + TX - 1) / TX, (kp.ny + TY - 1) / TY),
+    return launch_dependent(fused_writes_rings(TX), k_step_fused<NP, TF, TX, TY>, dim3((kp.nx + TX - 1) / TX, (kp.ny + TY - 1) / TY),
                             dim3(TX, TY), L::bytes, s, *a.tm_pop, *a.tm_g, *a.tm_lag, *a.tm_st, *a.tm_a, kp, a.pop_out,
                             a.lag_out, a.err, pf_dist, off32);
 }
@@ -1056,38 +1059,38 @@ size_t tile_tma_smem_bytes(int N, bool tf) {
     }
 }
 // The fused kernel's tile: 32 x 8 or 64 x 4 (see fused_tile_wide).
-template <typename T, int TX, int TY>
+template <int TX, int TY>
 size_t fused_smem_shape(int N, bool tf) {
     switch (N * 2 + (tf ? 1 : 0)) {
-        case 4: return FLay<T, 2, false, TX, TY>::bytes;
-        case 5: return FLay<T, 2, true, TX, TY>::bytes;
-        case 6: return FLay<T, 3, false, TX, TY>::bytes;
-        case 7: return FLay<T, 3, true, TX, TY>::bytes;
-        case 8: return FLay<T, 4, false, TX, TY>::bytes;
-        case 9: return FLay<T, 4, true, TX, TY>::bytes;
+        case 4: return FLay<2, false, TX, TY>::bytes;
+        case 5: return FLay<2, true, TX, TY>::bytes;
+        case 6: return FLay<3, false, TX, TY>::bytes;
+        case 7: return FLay<3, true, TX, TY>::bytes;
+        case 8: return FLay<4, false, TX, TY>::bytes;
+        case 9: return FLay<4, true, TX, TY>::bytes;
         default: return 0;
     }
 }
 template <typename T>
 size_t tile_fused_smem_bytes(int N, bool tf, bool wide) {
-    return wide ? fused_smem_shape<T, kWideX, kWideY>(N, tf) : fused_smem_shape<T, BX, BY>(N, tf);
+    return wide ? fused_smem_shape<kWideX, kWideY>(N, tf) : fused_smem_shape<BX, BY>(N, tf);
 }
-template <typename T, int TX, int TY>
-cudaError_t fused_shape(const TileTmaArgs<T>& a, cudaStream_t s) {
+template <int TX, int TY>
+cudaError_t fused_shape(const TileTmaArgs<float>& a, cudaStream_t s) {
     const bool tf = a.kp->has_cos_field != 0;
     switch (a.kp->N * 2 + (tf ? 1 : 0)) {
-        case 4: return collide_fused_n<T, 2, false, TX, TY>(a, s);
-        case 5: return collide_fused_n<T, 2, true, TX, TY>(a, s);
-        case 6: return collide_fused_n<T, 3, false, TX, TY>(a, s);
-        case 7: return collide_fused_n<T, 3, true, TX, TY>(a, s);
-        case 8: return collide_fused_n<T, 4, false, TX, TY>(a, s);
-        case 9: return collide_fused_n<T, 4, true, TX, TY>(a, s);
+        case 4: return collide_fused_n<2, false, TX, TY>(a, s);
+        case 5: return collide_fused_n<2, true, TX, TY>(a, s);
+        case 6: return collide_fused_n<3, false, TX, TY>(a, s);
+        case 7: return collide_fused_n<3, true, TX, TY>(a, s);
+        case 8: return collide_fused_n<4, false, TX, TY>(a, s);
+        case 9: return collide_fused_n<4, true, TX, TY>(a, s);
         default: return cudaErrorInvalidValue;
     }
 }
 template <typename T>
 cudaError_t launch_collide_fused(const TileTmaArgs<T>& a, cudaStream_t s) {
-    return a.wide ? fused_shape<T, kWideX, kWideY>(a, s) : fused_shape<T, BX, BY>(a, s);
+    return a.wide ? fused_shape<kWideX, kWideY>(a, s) : fused_shape<BX, BY>(a, s);
 }
 template <typename T>
 cudaError_t launch_collide_tma(const TileTmaArgs<T>& a, cudaStream_t s) {
